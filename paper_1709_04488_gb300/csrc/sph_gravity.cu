@@ -26,6 +26,14 @@ namespace sph {
 namespace {
 
 constexpr int kGravThreads = 128;  // two particles per thread: 256 per block
+constexpr int kGravBlocksPerSM = 8;
+// The partner ranges (see gravity_chunks): blocks wanted (constants: the split
+// depends on N alone), the smallest range, most ranges (partial forces take
+// 24 bytes per particle and range), and the bytes per particle of the rest
+// of the largest layout beside which the partials of up to 32768 particles
+// have to fit the allocation-free entry point's fixed scratch
+constexpr int kGravBlocks = 4 * 152 * kGravBlocksPerSM, kGravMinSpan = 128, kGravMaxChunks = 32;
+constexpr long long kGravFixedN = 32768, kGravFixedBytes = 24ll << 20, kGravFixedRest = 540;
 
 // M(q) of the force kernel with every operation's rounding fixed, so that
 // both particles of a pair get the same bits
@@ -39,11 +47,11 @@ __device__ __forceinline__ T grav_mass_rn(T q)
                                T(-1.0 / 60.0)));
 }
 
-// partners per range: ceil(N/C) rounded up to whole tiles
+// partners per range: ceil(N/C) rounded up to whole warps of loads
 __host__ __device__ inline long long gravity_span(long long n, int c)
 {
     const long long s = (n + c - 1) / c;
-    return (s + 2 * kGravThreads - 1) / (2 * kGravThreads) * (2 * kGravThreads);
+    return (s + 31) / 32 * 32;
 }
 
 template <typename T>
@@ -80,10 +88,122 @@ __device__ __forceinline__ void grav_pair(T xi, T yi, T zi, T mi, T hi, T hinv_i
     az.add(-mul_rn(w, rz));
 }
 
+// Two FP32 values in one 64-bit register and the packed operations on them
+// (each half rounded as the scalar operation rounds it).
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float a, float b)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(F2 x, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 operator+(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+// a - b, rounded once: fma(b, -1, a)
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
+
+// TwoSumAcc of two particles at once
+struct TwoSumAcc2 {
+    F2 s, c;
+    __device__ __forceinline__ void add(F2 x)
+    {
+        const F2 t = s + x, xp = t - s, sp = t - xp;
+        c = c + ((s - sp) + (x - xp));
+        s = t;
+    }
+};
+
+// The sums of the two particles of a thread over staged partners.  pair()
+// is grav_pair for both, operation for operation (FP32: in packed
+// arithmetic, which halves the instructions of a kernel whose bound is their
+// issue; only the reciprocal roots and the rare softened pairs stay scalar).
+template <typename T>
+struct GravTwo {
+    using P = typename GravVec<T>::P;
+    using H = typename GravVec<T>::H;
+    P x0, x1;
+    H h0, h1;
+    TwoSumAcc<T> a[3][2];
+    __device__ __forceinline__ GravTwo(const P &x0_, const P &x1_, const H &h0_, const H &h1_)
+        : x0(x0_), x1(x1_), h0(h0_), h1(h1_)
+    {
+        for (int k = 0; k < 3; ++k) a[k][0] = a[k][1] = TwoSumAcc<T>{T(0), T(0)};
+    }
+    __device__ __forceinline__ void pair(const P &q, const H &hq)
+    {
+        grav_pair(x0.x, x0.y, x0.z, x0.w, h0.x, h0.y, q, hq, a[0][0], a[1][0], a[2][0]);
+        grav_pair(x1.x, x1.y, x1.z, x1.w, h1.x, h1.y, q, hq, a[0][1], a[1][1], a[2][1]);
+    }
+    __device__ __forceinline__ double sum(int axis, int k) const { return (double)a[axis][k].s + (double)a[axis][k].c; }
+};
+template <>
+struct GravTwo<float> {
+    F2 x, y, z, m;
+    float h[2], hinv[2];
+    TwoSumAcc2 a[3];
+    __device__ __forceinline__ GravTwo(const float4 &x0, const float4 &x1, const float2 &h0, const float2 &h1)
+        : x(pack2(x0.x, x1.x)), y(pack2(x0.y, x1.y)), z(pack2(x0.z, x1.z)), m(pack2(x0.w, x1.w)),
+          h{h0.x, h1.x}, hinv{h0.y, h1.y}
+    {
+        for (int k = 0; k < 3; ++k) a[k] = TwoSumAcc2{pack2(0.f, 0.f), pack2(0.f, 0.f)};
+    }
+    __device__ __forceinline__ void pair(const float4 &q, const float2 &hq)
+    {
+        const F2 rx = x - pack2(q.x, q.x), ry = y - pack2(q.y, q.y), rz = z - pack2(q.z, q.z);
+        const F2 r2 = fma2(rz, rz, fma2(ry, ry, rx * rx));
+        float r2a, r2b;
+        unpack2(r2, r2a, r2b);
+        const F2 rinv = pack2(rsqrt_t(r2a), rsqrt_t(r2b));
+        const F2 rinv2 = rinv * rinv, r = r2 * rinv;
+        float ra, rb, fa, fb;
+        unpack2(r, ra, rb);
+        unpack2(rinv2, fa, fb);  // beyond both supports: 1/r^2
+        if (ra < 2.f * (h[0] > hq.x ? h[0] : hq.x))
+            fa = mul_rn(mul_rn(0.5f, add_rn(grav_mass_rn(mul_rn(ra, hinv[0])), grav_mass_rn(mul_rn(ra, hq.y)))), fa);
+        if (rb < 2.f * (h[1] > hq.x ? h[1] : hq.x))
+            fb = mul_rn(mul_rn(0.5f, add_rn(grav_mass_rn(mul_rn(rb, hinv[1])), grav_mass_rn(mul_rn(rb, hq.y)))), fb);
+        float wa, wb;
+        unpack2(((m * pack2(q.w, q.w)) * pack2(fa, fb)) * rinv, wa, wb);
+        const F2 w = pack2(r2a > 0.f ? -wa : 0.f, r2b > 0.f ? -wb : 0.f);  // (-w) r = -(w r)
+        a[0].add(w * rx);
+        a[1].add(w * ry);
+        a[2].add(w * rz);
+    }
+    __device__ __forceinline__ double sum(int axis, int k) const
+    {
+        float s[2], c[2];
+        unpack2(a[axis].s, s[0], s[1]);
+        unpack2(a[axis].c, c[0], c[1]);
+        return (double)s[k] + (double)c[k];
+    }
+};
+
 // Each thread serves two particles (kGravThreads apart), so that each staged
 // partner is read from shared memory once per two pair terms.
 template <typename T>
-__global__ void __launch_bounds__(kGravThreads) k_gravity(BatchView b)
+__global__ void __launch_bounds__(kGravThreads, sizeof(T) == 4 ? kGravBlocksPerSM : 1) k_gravity(BatchView b)
 {
     using P = typename GravVec<T>::P;
     using H = typename GravVec<T>::H;
@@ -123,8 +243,7 @@ __global__ void __launch_bounds__(kGravThreads) k_gravity(BatchView b)
     h0.x = h0.y = h1.x = h1.y = T(1);
     if (i0 < end) load(i0, x0, h0);
     if (i1 < end) load(i1, x1, h1);
-    TwoSumAcc<T> a0x{T(0), T(0)}, a0y{T(0), T(0)}, a0z{T(0), T(0)};
-    TwoSumAcc<T> a1x{T(0), T(0)}, a1y{T(0), T(0)}, a1z{T(0), T(0)};
+    GravTwo<T> two(x0, x1, h0, h1);
     for (long long j0 = jlo; j0 < jhi; j0 += 2 * kGravThreads) {
         __syncthreads();  // the previous tile is consumed
         for (int t = threadIdx.x; t < 2 * kGravThreads; t += kGravThreads)
@@ -132,31 +251,27 @@ __global__ void __launch_bounds__(kGravThreads) k_gravity(BatchView b)
         __syncthreads();
         const int jn = (int)(jhi - j0 < 2 * kGravThreads ? jhi - j0 : 2 * kGravThreads);
 #pragma unroll 4
-        for (int k = 0; k < jn; ++k) {
-            const P q = tp[k];
-            const H hq = th[k];
-            grav_pair(x0.x, x0.y, x0.z, x0.w, h0.x, h0.y, q, hq, a0x, a0y, a0z);
-            grav_pair(x1.x, x1.y, x1.z, x1.w, h1.x, h1.y, q, hq, a1x, a1y, a1z);
-        }
+        for (int k = 0; k < jn; ++k) two.pair(tp[k], th[k]);
     }
-    auto store = [&](long long i, const TwoSumAcc<T> &ax, const TwoSumAcc<T> &ay, const TwoSumAcc<T> &az) {
+    auto store = [&](long long i, int k) {
+        const double F[3] = {two.sum(0, k), two.sum(1, k), two.sum(2, k)};
         if (b.block_on && ((const T *)b.slev)[i] < T(0)) return;  // block step: not this particle's force pass
         if (C > 1) {  // partial of range ch, layout [ch][axis][ntot]
             double *g = b.gpart + (long long)ch * 3 * b.ntot + i;
-            g[0] = (double)ax.s + (double)ax.c;
-            g[b.ntot] = (double)ay.s + (double)ay.c;
-            g[2 * b.ntot] = (double)az.s + (double)az.c;
+            g[0] = F[0];
+            g[b.ntot] = F[1];
+            g[2 * b.ntot] = F[2];
             return;
         }
         const long long io = (long long)b.perm[i] - ps.base;
         const double minv = ps.uniform_m ? ps.inv_m_uniform : 1.0 / ps.m[io];
         const double Gm = ps.ph.G * minv;
-        ps.ax[io] += Gm * ((double)ax.s + (double)ax.c);
-        ps.ay[io] += Gm * ((double)ay.s + (double)ay.c);
-        ps.az[io] += Gm * ((double)az.s + (double)az.c);
+        ps.ax[io] += Gm * F[0];
+        ps.ay[io] += Gm * F[1];
+        ps.az[io] += Gm * F[2];
     };
-    if (i0 < end) store(i0, a0x, a0y, a0z);
-    if (i1 < end) store(i1, a1x, a1y, a1z);
+    if (i0 < end) store(i0, 0);
+    if (i1 < end) store(i1, 1);
 }
 
 // Sum the partials of split problems in range order: a_i += G/m_i sum_ch F_i,ch.
@@ -693,15 +808,23 @@ __global__ void __launch_bounds__(256) k_grav_dt(BatchView b)
 
 }  // namespace
 
-// C partner ranges for N particles: enough blocks to fill the GPU (about 8 per
-// SM), at most 16 ranges and at least 4096 partners per range.
+// C partner ranges for N particles: four waves of blocks (8 per SM), of at
+// least 128 partners each.  The kernel's time was its slowest block's: blocks
+// near their own particles' diagonal take the softened branch.  One wave,
+// two, three and four, 20001 particles (three evaluations, the whole pass):
+// 3.43, 3.03, 2.94, 2.90 ms; 65536: 21.0, 19.9, 19.0, 18.7 ms (with ranges of
+// 4096 partners and scalar pairs 5.78 and 28 ms).
 int gravity_chunks(long long n, double theta)
 {
     if (theta > 0) return 0;  // the tree walk serves this problem
     const long long ib = (n + 2 * kGravThreads - 1) / (2 * kGravThreads);
-    long long c = ib > 0 ? (1216 + ib - 1) / ib : 1;
-    if (c > 16) c = 16;
-    if (c > n / 4096) c = n / 4096;
+    long long c = ib > 0 ? kGravBlocks / ib : 1;
+    if (c > kGravMaxChunks) c = kGravMaxChunks;
+    if (c > n / kGravMinSpan) c = n / kGravMinSpan;
+    if (n > 0 && n <= kGravFixedN) {
+        const long long fit = (kGravFixedBytes - kGravFixedRest * n) / (24 * n);
+        if (c > fit) c = fit;
+    }
     return c < 1 ? 1 : (int)c;
 }
 
