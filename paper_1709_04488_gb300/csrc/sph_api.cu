@@ -273,6 +273,11 @@ PhysParams phys_of(const sph_params *p)
         ph.box_inv[a] = p->periodic ? 1.0 / ph.box_len[a] : 0.0;
         ph.box_inv_f[a] = p->periodic ? 1.0f / ph.box_len_f[a] : 0.f;
     }
+    if (p->periodic)
+        for (int a = 0; a < 3; ++a) {
+            const float m = 2.f * (float)(std::fabs(p->box_lo[a]) + p->box_len[a]);
+            ph.coord_max = m > ph.coord_max ? m : ph.coord_max;
+        }
     ph.gamma = p->gamma;
     ph.cs_iso = p->cs_iso;
     ph.eta = p->eta;

@@ -72,6 +72,7 @@ struct PhysParams {
     int kernel;          // SPH_KERNEL_M4 or SPH_KERNEL_M6
     float box_len_f[3];  // box_len as float (node tests run in FP32)
     float kr_f;          // support radius in units of h: 2 (M4) or 3 (M6)
+    float coord_max;     // periodic: bound of the particles' and boxes' |coordinates|
     double kr;
     double box_inv[3];   // 1 / box_len (periodic), for minimum-image wraps
     float box_inv_f[3];
@@ -138,7 +139,7 @@ struct ProbDyn {
     int node_off[kMaxLevels + 1];  // global index of this problem's first node per level
     int node_cnt[kMaxLevels + 1];  // nodes per level (level 0 = leaves)
     int lists_stale;     // some leaf's final h exceeds what its recorded candidate groups cover
-    int pad_;
+    float coord_max;     // isolated: bound of |coordinates| (twice those of the last sort's domain)
 };
 
 // 32-byte vector of four doubles (FP64 staging)

@@ -209,102 +209,185 @@ __device__ __forceinline__ double bits_as_t(int v, double) { return (double)v; }
 __device__ __forceinline__ int t_as_bits(float v) { return __float_as_int(v); }
 __device__ __forceinline__ int t_as_bits(double v) { return (int)v; }
 
-// Separating-axis test of two boxes grown by R, periodic aware, conservative
-// for the FP32 rounding of the box coordinates.
-__device__ __forceinline__ bool axis_overlap(float alo, float ahi, float blo, float bhi, float R,
-                                             int periodic, float L)
+// The query box of a walk, in the warp's scratch (read back at each node
+// test as broadcast vectors).  The leaves that pass decide the slots of the
+// staged candidates, hence (at several lanes per particle) the order of the
+// sums, so their test has one definition (leaf_within, leaf_overlap).  It
+// takes about 15 operations per axis; node_gap takes 7 and agrees with it to
+// within s, 1e-5 of the problem's coordinates and the reach (five times the
+// definition's own slack), so that only boxes within s of the boundary, well
+// under one test in ten, are decided by the definition, and the nodes above
+// the leaves, which only have to pass what holds such a leaf, never are.
+// (With the definition at the leaves and a one-sided test above: cloud 8e6
+// 62.3 ms for two evaluations, M6 lattice of 37^3 3.84 ms for five; with
+// this 57.9 and 3.47 ms.)
+struct QueryBox {
+    float4 ax[3];  // per axis: lo + hi, hi - lo, 2 L (infinity if isolated)
+    // squared distances (of doubled coordinates) below which a box is within
+    // R for sure and above which it is not; s doubled; R^2 of the definition
+    float in2, out2, s2, R2;
+};
+__device__ __forceinline__ void set_query(QueryBox &qb, const float4 &lo, const float4 &hi, float R, const PhysParams &ph,
+                                          const ProbDyn &d)
 {
-    float ca = 0.5f * (alo + ahi), ha = 0.5f * (ahi - alo);
-    float cb = 0.5f * (blo + bhi), hb = 0.5f * (bhi - blo);
-    float reach = ha + hb + R;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < 3) {
+        const float l = lane == 0 ? lo.x : lane == 1 ? lo.y : lo.z, h = lane == 0 ? hi.x : lane == 1 ? hi.y : hi.z;
+        qb.ax[lane] = make_float4(l + h, h - l, ph.periodic ? 2.f * ph.box_len_f[lane] : INFINITY, 0.f);
+    } else if (lane == 3) {
+        const float s = 1e-5f * ((ph.periodic ? ph.coord_max : d.coord_max) + R) + 1e-29f;
+        const float in = 2.f * (R - 2.f * s), out = 2.f * (R + 2.f * s);
+        qb.in2 = in > 0.f ? in * in : -1.f;
+        qb.out2 = out * out;
+        qb.s2 = 2.f * s;
+        qb.R2 = R * R * 1.00001f;
+    }
+    __syncwarp();
+}
+
+// twice the gap between the query box and [blo, bhi] along one axis (minimum
+// image if periodic), negative where they overlap
+__device__ __forceinline__ float node_gap(const float4 &qa, float blo, float bhi)
+{
+    const float d = qa.x - (blo + bhi);
+    return fminf(fabsf(d), fabsf(qa.z - fabsf(d))) - (qa.y + (bhi - blo));
+}
+__device__ __forceinline__ float node_dist2(const QueryBox &qb, const float4 &blo, const float4 &bhi)
+{
+    const float gx = fmaxf(node_gap(qb.ax[0], blo.x, bhi.x), 0.f);
+    const float gy = fmaxf(node_gap(qb.ax[1], blo.y, bhi.y), 0.f);
+    const float gz = fmaxf(node_gap(qb.ax[2], blo.z, bhi.z), 0.f);
+    return gx * gx + gy * gy + gz * gz;
+}
+__device__ __forceinline__ float node_sep(const QueryBox &qb, const float4 &blo, const float4 &bhi)
+{
+    return fmaxf(node_gap(qb.ax[0], blo.x, bhi.x),
+                 fmaxf(node_gap(qb.ax[1], blo.y, bhi.y), node_gap(qb.ax[2], blo.z, bhi.z)));
+}
+
+// The definition, along one axis: the centres' distance and the reach of the
+// two boxes, grown for the FP32 rounding of the box coordinates; overlap in
+// every image where the reach spans half the box.
+__device__ __forceinline__ bool axis_dist(const float4 &qa, float blo, float bhi, int periodic, float L, float &d,
+                                          float &reach)
+{
+    const float ca = 0.5f * qa.x, ha = 0.5f * qa.y;
+    const float cb = 0.5f * (blo + bhi), hb = 0.5f * (bhi - blo);
+    reach = ha + hb;
     reach += 2e-6f * (fabsf(ca) + fabsf(cb) + reach) + 1e-30f;
-    float d = fabsf(ca - cb);
+    d = fabsf(ca - cb);
     if (periodic) {
         if (reach >= 0.5f * L) return true;
         if (d > L) d -= L;
         d = fminf(d, L - d);
     }
-    return d <= reach;
+    return false;
 }
-
-__device__ __forceinline__ bool box_overlap(const float4 &alo, const float4 &ahi, const float4 &blo,
-                                            const float4 &bhi, float R, const PhysParams &ph)
+__device__ __forceinline__ float axis_gap(const float4 &qa, float blo, float bhi, int periodic, float L)
 {
-    return axis_overlap(alo.x, ahi.x, blo.x, bhi.x, R, ph.periodic, ph.box_len_f[0]) &&
-           axis_overlap(alo.y, ahi.y, blo.y, bhi.y, R, ph.periodic, ph.box_len_f[1]) &&
-           axis_overlap(alo.z, ahi.z, blo.z, bhi.z, R, ph.periodic, ph.box_len_f[2]);
+    float d, reach;
+    return axis_dist(qa, blo, bhi, periodic, L, d, reach) ? 0.f : fmaxf(d - reach, 0.f);
 }
-
-// Gap between the two boxes' extents along one axis (minimum image if
-// periodic), shrunk for the FP32 rounding of the box coordinates.
-__device__ __forceinline__ float axis_gap(float alo, float ahi, float blo, float bhi, int periodic, float L)
+__device__ __forceinline__ bool axis_overlap(const float4 &qa, float blo, float bhi, int periodic, float L)
 {
-    float ca = 0.5f * (alo + ahi), ha = 0.5f * (ahi - alo);
-    float cb = 0.5f * (blo + bhi), hb = 0.5f * (bhi - blo);
-    float reach = ha + hb;
-    reach += 2e-6f * (fabsf(ca) + fabsf(cb) + reach) + 1e-30f;
-    float d = fabsf(ca - cb);
-    if (periodic) {
-        if (reach >= 0.5f * L) return 0.f;
-        if (d > L) d -= L;
-        d = fminf(d, L - d);
-    }
-    return fmaxf(d - reach, 0.f);
+    float d, reach;
+    return axis_dist(qa, blo, bhi, periodic, L, d, reach) || d <= reach;
 }
-
 // Do two boxes come within (Euclidean) distance R of each other?  Tighter
 // than growing one box by R along each axis: the grown box's corners, where
 // no point is within R, are left out.
-__device__ __forceinline__ bool box_within(const float4 &alo, const float4 &ahi, const float4 &blo,
-                                           const float4 &bhi, float R, const PhysParams &ph)
+__device__ __forceinline__ bool leaf_within(const QueryBox &qb, const float4 &blo, const float4 &bhi, const PhysParams &ph)
 {
-    const float gx = axis_gap(alo.x, ahi.x, blo.x, bhi.x, ph.periodic, ph.box_len_f[0]);
-    const float gy = axis_gap(alo.y, ahi.y, blo.y, bhi.y, ph.periodic, ph.box_len_f[1]);
-    const float gz = axis_gap(alo.z, ahi.z, blo.z, bhi.z, ph.periodic, ph.box_len_f[2]);
-    return gx * gx + gy * gy + gz * gz <= R * R * 1.00001f;
+    const float gx = axis_gap(qb.ax[0], blo.x, bhi.x, ph.periodic, ph.box_len_f[0]);
+    const float gy = axis_gap(qb.ax[1], blo.y, bhi.y, ph.periodic, ph.box_len_f[1]);
+    const float gz = axis_gap(qb.ax[2], blo.z, bhi.z, ph.periodic, ph.box_len_f[2]);
+    return gx * gx + gy * gy + gz * gz <= qb.R2;
+}
+__device__ __forceinline__ bool leaf_overlap(const QueryBox &qb, const float4 &blo, const float4 &bhi, const PhysParams &ph)
+{
+    return axis_overlap(qb.ax[0], blo.x, bhi.x, ph.periodic, ph.box_len_f[0]) &&
+           axis_overlap(qb.ax[1], blo.y, bhi.y, ph.periodic, ph.box_len_f[1]) &&
+           axis_overlap(qb.ax[2], blo.z, bhi.z, ph.periodic, ph.box_len_f[2]);
+}
+
+// Tests of one node per lane, called by the whole warp: the position box
+// within R (up_within: nodes above the leaves), the smoothing-sphere box
+// overlapping the query.
+__device__ __forceinline__ bool up_within(const QueryBox &qb, const NodeBox &nb)
+{
+    return node_dist2(qb, nb.plo, nb.phi) <= qb.out2;
+}
+__device__ __forceinline__ bool up_overlap(const QueryBox &qb, const NodeBox &nb) { return node_sep(qb, nb.slo, nb.shi) <= qb.s2; }
+__device__ __forceinline__ bool box_within(const QueryBox &qb, const NodeBox &nb, const PhysParams &ph)
+{
+    const float g2 = node_dist2(qb, nb.plo, nb.phi);
+    bool ok = g2 <= qb.in2;
+    const bool edge = !ok && g2 <= qb.out2;
+    if (__any_sync(FULL, edge) && edge) ok = leaf_within(qb, nb.plo, nb.phi, ph);
+    return ok;
+}
+__device__ __forceinline__ bool box_overlap(const QueryBox &qb, const NodeBox &nb, const PhysParams &ph)
+{
+    const float g = node_sep(qb, nb.slo, nb.shi);
+    bool ok = g <= -qb.s2;
+    const bool edge = !ok && g <= qb.s2;
+    if (__any_sync(FULL, edge) && edge) ok = leaf_overlap(qb, nb.slo, nb.shi, ph);
+    return ok;
 }
 
 // Warp-cooperative depth-first walk of one problem's tree.  At the leaf level
 // visit(mask, first) is called (warp-uniformly) with the ballot of the up to
 // 32 sibling leaves first..first+31 whose boxes pass test(box), so that a
-// whole group of candidate leaves is staged in one round of memory accesses.
-template <class Test, class Visit>
-__device__ __forceinline__ void walk(const BatchView &b, const ProbDyn &d, Test &&test, Visit &&visit)
+// whole group of candidate leaves is staged in one round of memory accesses;
+// the nodes above them are opened where up(box) passes.
+// The nodes still to open of each level above the current one are kept in
+// the lanes (lane l: level l's), not in an array a run-time level indexes.
+template <class Up, class Test, class Visit>
+__device__ __forceinline__ void walk(const BatchView &b, const ProbDyn &d, Up &&up, Test &&test, Visit &&visit)
 {
     const int lane = threadIdx.x & 31;
     const int top = d.top_level;
-    unsigned mask[kMaxLevels + 1];
-    int base[kMaxLevels + 1];
-    {
-        bool ok = lane < d.node_cnt[top] && test(b.nodes[top][d.node_off[top] + lane]);
-        unsigned m = __ballot_sync(FULL, ok);
-        if (top == 0) {
-            if (m) visit(m, d.node_off[0]);
-            return;
-        }
-        mask[top] = m;
-        base[top] = 0;
+    const int off0 = d.node_off[0], cnt0 = d.node_cnt[0];
+    const NodeBox *leaves = b.nodes[0] + off0;
+    bool ok = false;
+    if (top == 0) {
+        ok = test(leaves[lane < cnt0 ? lane : 0]) && lane < cnt0;
+        const unsigned lm = __ballot_sync(FULL, ok);
+        if (lm) visit(lm, off0);
+        return;
     }
-    int lvl = top;
+    if (lane < d.node_cnt[top]) ok = up(b.nodes[top][d.node_off[top] + lane]);
+    unsigned m = __ballot_sync(FULL, ok);
+    unsigned sm = 0u;
+    int sb = 0, lvl = top, base = 0;
     for (;;) {
-        unsigned m = mask[lvl];
-        if (m == 0u) {
-            if (++lvl > top) break;
+        while (m == 0u) {
+            if (lvl == top) return;
+            ++lvl;
+            m = __shfl_sync(FULL, sm, lvl);
+            base = __shfl_sync(FULL, sb, lvl);
+        }
+        const int node = base + __ffs(m) - 1;
+        m &= m - 1u;
+        const int ch = node * kBranch + lane;
+        ok = false;
+        if (lvl == 1) {  // (every lane tests a leaf of the node: test votes)
+            ok = test(leaves[ch < cnt0 ? ch : node * kBranch]) && ch < cnt0;
+            const unsigned cm = __ballot_sync(FULL, ok);
+            if (cm) visit(cm, off0 + node * kBranch);
             continue;
         }
-        int c = __ffs(m) - 1;
-        mask[lvl] = m & (m - 1u);
-        int node = base[lvl] + c;
-        int ch = node * kBranch + lane;
-        bool ok = ch < d.node_cnt[lvl - 1] && test(b.nodes[lvl - 1][d.node_off[lvl - 1] + ch]);
-        unsigned cm = __ballot_sync(FULL, ok);
-        if (lvl == 1) {
-            if (cm) visit(cm, d.node_off[0] + node * kBranch);
-            continue;
+        if (ch < d.node_cnt[lvl - 1]) ok = up(b.nodes[lvl - 1][d.node_off[lvl - 1] + ch]);
+        const unsigned cm = __ballot_sync(FULL, ok);
+        if (cm == 0u) continue;
+        if (lane == lvl) {
+            sm = m;
+            sb = base;
         }
         --lvl;
-        base[lvl] = node * kBranch;
-        mask[lvl] = cm;
+        m = cm;
+        base = node * kBranch;
     }
 }
 
@@ -323,27 +406,15 @@ __device__ __forceinline__ int warp_incl_scan(int v)
 // Per-warp scratch for staging one group of up to 32 candidate leaves.
 template <typename T>
 struct StageScratch {
-    int first[32];             // group element index of each candidate leaf's first particle
-    int start[32];             // sorted index of each candidate leaf's first particle
-    T dx[32], dy[32], dz[32];  // leaf shift (FP64 difference of reference points, cast)
+    // per candidate leaf, in order: its shift (FP64 difference of reference
+    // points, cast) and (w) its first sorted index less its first element
+    typename Vec4<T>::type leaf[32];
     T L[3], Li[3];             // box lengths and their inverses (periodic wraps)
     T C[3];                    // centre of the query leaf's box (in its frame)
+    QueryBox qb;               // the walk's query
     float ihl[3];              // 2 / box length
     float thr[3];              // candidate extents (packed units) from which a leaf pair is ambiguous
 };
-
-// candidate leaf (lane of the group) holding group element e: the last lane
-// whose first element is <= e (lanes without particles share the next
-// lane's first element and are passed over)
-template <typename T>
-__device__ __forceinline__ int owner_of(const StageScratch<T> &sc, int e)
-{
-    int k = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1)
-        if (sc.first[k + step] <= e) k += step;
-    return k;
-}
 
 // Periodic minimum images.  A pair vector is formed as (o_i - o_j) - D from
 // the particles' offsets o from their leaves' reference points (at most E_A,
@@ -416,6 +487,15 @@ __device__ __forceinline__ bool ambiguous(float eb, const StageScratch<T> &sc)
            (float)((b >> 20) & 1023u) >= sc.thr[2];
 }
 
+// bits of `m` (lanes of a group), renumbered by the order of the lanes set in
+// `mask`
+__device__ __forceinline__ unsigned by_order(unsigned m, unsigned mask)
+{
+    if (m == 0u) return 0u;
+    const int lane = threadIdx.x & 31;
+    return __reduce_or_sync(FULL, (m >> lane) & 1u ? 1u << __popc(mask & ((1u << lane) - 1u)) : 0u);
+}
+
 // largest h (plo.w) and largest leaf offset extent (slo.w) of a problem,
 // carried up to its top nodes
 __device__ __forceinline__ void problem_top_max(const BatchView &b, const ProbDyn &dy, float &hmax, float &extmax)
@@ -467,16 +547,33 @@ __device__ __forceinline__ T box_dist2(const V &q, const V &lo, const V &hi)
     return dx * dx + dy * dy + dz * dz;
 }
 
+// shift of candidate leaf B's reference point from the query leaf A's: FP64
+// difference, minimum image (min_image's, decided on the bit pattern of |d|:
+// the comparisons would run on the narrow FP64 pipe), cast
+template <typename T>
+__device__ __forceinline__ T leaf_shift(double cb, double ca, double L, int periodic)
+{
+    double d = cb - ca;
+    if (periodic) {
+        const long long ad = __double_as_longlong(d) & 0x7fffffffffffffffll;
+        if (ad > __double_as_longlong(0.5 * L)) d += __longlong_as_double(__double_as_longlong(L) | (~__double_as_longlong(d) & (1ll << 63)));
+    }
+    return (T)d;
+}
+
 // Stage the particles of the leaves first + k (bit k of mask) that keep()
 // accepts, compacted into slots [nbuf, ...) of the warp's candidate buffer of
 // capacity CH; flush() runs first whenever fewer than 32 slots are free.
 // The particles are read 32 at a time, one per lane, through load(j) (j the
 // sorted index) and moved into the query leaf A's frame by the leaf shift
-// (FP64 difference of the reference points, minimum image, cast) before
-// keep(q, k) sees them (k: the lane of the particle's leaf; keep may move q
-// to another periodic image).  group(has, B, stB, D) runs on every lane once
-// per call (lane k: candidate leaf first + k if has); store(slot, q, k, idx)
-// writes a kept particle (idx: its index within its leaf).
+// before keep(q, o) sees them (o: which candidate leaf of the group, in
+// order; keep may move q to another periodic image).  group(has, B, stB, o,
+// D) runs on every lane once per call (lane k: candidate leaf first + k if
+// has); store(slot, q, o, idx) writes a kept particle (idx: its index within
+// its leaf).  The leaf of element e follows from the leaves' first elements
+// that fall into the chunk, one bit each, gathered by one warp reduction
+// (a binary search over the first elements took five dependent shared-memory
+// reads per chunk).
 template <typename T, int CH, class Group, class Load, class Keep, class Store, class Flush>
 __device__ __forceinline__ void stage_group(const BatchView &b, int A, unsigned mask, int first, const PhysParams &ph,
                                             int &nbuf, StageScratch<T> &sc, Group &&group, Load &&load,
@@ -485,57 +582,64 @@ __device__ __forceinline__ void stage_group(const BatchView &b, int A, unsigned 
     using V = typename Vec4<T>::type;
     const int lane = threadIdx.x & 31;
     const bool has = (mask >> lane) & 1u;
+    const unsigned below = (1u << lane) - 1u;
+    const int ord = __popc(mask & below);
     int stB = 0, nB = 0;
-    T Dx = T(0), Dy = T(0), Dz = T(0);
+    V D{};
     if (has) {
         const int B = first + lane;
         stB = b.leaf_start[B];
         nB = b.leaf_start[B + 1] - stB;
         const double *cb = b.leaf_c + 3LL * B, *ca = b.leaf_c + 3LL * A;
-        Dx = (T)min_image(cb[0] - ca[0], ph.box_len[0], ph.periodic);
-        Dy = (T)min_image(cb[1] - ca[1], ph.box_len[1], ph.periodic);
-        Dz = (T)min_image(cb[2] - ca[2], ph.box_len[2], ph.periodic);
+        D.x = leaf_shift<T>(cb[0], ca[0], ph.box_len[0], ph.periodic);
+        D.y = leaf_shift<T>(cb[1], ca[1], ph.box_len[1], ph.periodic);
+        D.z = leaf_shift<T>(cb[2], ca[2], ph.box_len[2], ph.periodic);
     }
-    group(has, first + lane, stB, Dx, Dy, Dz);
+    group(has, first + lane, stB, ord, D);
     const int incl = warp_incl_scan<T>(nB);
     const int tot = __shfl_sync(FULL, incl, 31);
+    // first element of this lane's leaf (beyond every chunk without one)
+    const int fe = has ? incl - nB : 0x40000000;
     __syncwarp();  // earlier readers of the scratch are done
-    sc.first[lane] = incl - nB;
-    sc.start[lane] = stB;
-    sc.dx[lane] = Dx;
-    sc.dy[lane] = Dy;
-    sc.dz[lane] = Dz;
+    if (has) {
+        D.w = bits_as_t(stB - fe, T(0));
+        sc.leaf[ord] = D;
+    }
     __syncwarp();
-    const unsigned below = (1u << lane) - 1u;
+    // element e0 + lane of the chunk at e0: which leaf, its index there, its
+    // staged vector; `started` leaves begin before the chunk, the last of
+    // them `into` elements before it
+    int started = 0, into = 0;
+    V qn{}, sn{};
+    int on = 0, idxn = 0;
+    auto fetch = [&](int e0) {
+        const unsigned x = (unsigned)(fe - e0);
+        const unsigned M = __reduce_or_sync(FULL, x < 32u ? 1u << x : 0u);
+        const unsigned le = M & (below | (1u << lane));
+        if (e0 + lane < tot) {
+            on = started + __popc(le) - 1;
+            idxn = le ? lane - (31 - __clz(le)) : lane + into;
+            sn = sc.leaf[on];
+            qn = load(e0 + lane + t_as_bits(sn.w));
+        }
+        started += __popc(M);
+        into = M ? __clz(M) + 1 : into + 32;
+    };
     // the particles are loaded one chunk of 32 ahead: a chunk's load (an L2
     // round trip) overlaps the filtering, storing and flushing of the chunk
     // before it (flush() leaves the scratch and the loaded arrays alone)
-    V qn{};
-    int kn = 0, idxn = 0;
-    if (lane < tot) {
-        kn = owner_of(sc, lane);
-        idxn = lane - sc.first[kn];
-        qn = load(sc.start[kn] + idxn);
-    }
+    fetch(0);
     for (int e0 = 0; e0 < tot; e0 += 32) {
-        const int e = e0 + lane;
         V q = qn;
-        const int k = kn, idx = idxn;
-        if (e + 32 < tot) {
-            kn = owner_of(sc, e + 32);
-            idxn = e + 32 - sc.first[kn];
-            qn = load(sc.start[kn] + idxn);
-        }
+        q.x += sn.x;
+        q.y += sn.y;
+        q.z += sn.z;
+        const int o = on, idx = idxn;
+        if (e0 + 32 < tot) fetch(e0 + 32);
         if (nbuf > CH - 32) flush();
-        bool ok = false;
-        if (e < tot) {
-            q.x += sc.dx[k];
-            q.y += sc.dy[k];
-            q.z += sc.dz[k];
-            ok = keep(q, k);
-        }
+        const bool ok = e0 + lane < tot && keep(q, o);
         const unsigned bal = __ballot_sync(FULL, ok);
-        if (ok) store(nbuf + __popc(bal & below), q, k, idx);
+        if (ok) store(nbuf + __popc(bal & below), q, o, idx);
         nbuf += __popc(bal);
     }
 }
@@ -614,7 +718,9 @@ struct DCfg {
     static constexpr int MINB = LPP == 1 ? SPH_DENS_MINB1 : SPH_DENS_MINB;  // blocks per SM the registers allow
     static constexpr int LW = UM ? 1 : 2;  // list words per entry: r^2 (and m_j unless masses are equal)
     static constexpr size_t scratch = (sizeof(StageScratch<T>) + 31) & ~(size_t)31;
-    static constexpr size_t per_warp = CH * sizeof(V) + (size_t)LCAP * 32 * LW * sizeof(T) + scratch;
+    // (a row beyond the capacity takes the entries that no longer fit)
+    static constexpr size_t lists = (size_t)(LCAP + 1) * 32 * LW * sizeof(T);
+    static constexpr size_t per_warp = CH * sizeof(V) + lists + scratch;
     static constexpr size_t smem = WPB * per_warp;
 };
 
@@ -760,8 +866,8 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     const int lane = threadIdx.x & 31;
     V *cand = reinterpret_cast<V *>(mine);
     T *lr = reinterpret_cast<T *>(mine + C::CH * sizeof(V));  // r_ij^2 per entry
-    T *lm = lr + C::LCAP * 32;  // used only when masses differ
-    StageScratch<T> &sc = *reinterpret_cast<StageScratch<T> *>(lr + C::LCAP * 32 * C::LW);
+    T *lm = lr + (C::LCAP + 1) * 32;  // used only when masses differ
+    StageScratch<T> &sc = *reinterpret_cast<StageScratch<T> *>(mine + C::CH * sizeof(V) + C::lists);
     const int pp = lane / LPP, sub = lane % LPP;
     const V *pm = (const V *)b.pm;
     const int p = b.leaf_pid[leaf];
@@ -824,26 +930,26 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         const bool wrap2 = WRAP && half_width(flo, fhi) + Rq >= halfL;  // staged vectors may still need a wrap
         ng = 0;
         cnt = 0;
-        int gcnt = 0;
+        int gcnt = 0, at = lane;  // at: where this lane's next entry goes
+        const T R2t = active && !fail ? R2 : T(-1);
         bool ovf = false;
         int nbuf = 0;
         auto flush = [&]() {
             __syncwarp();  // staged candidates visible to every lane
             if (LPP == 1 || !bal) {
+                // (an entry beyond the capacity goes to the spare row: no
+                // branch on the append path)
 #pragma unroll 4
                 for (int k = sub; k < nbuf; k += LPP) {
                     V c = cand[k];
                     T dx = pi.x - c.x, dyy = pi.y - c.y, dz = pi.z - c.z;
                     if (wrap2) wrap3s<T>(sc, dx, dyy, dz);
                     T r2 = dx * dx + dyy * dyy + dz * dz;
-                    if (active && !fail && r2 < R2) {
-                        if (cnt < C::LCAP) {
-                            lr[cnt * 32 + lane] = r2;  // (its root where the lists are read: off the append path)
-                            if (!UM) lm[cnt * 32 + lane] = c.w;
-                            ++cnt;
-                        } else {
-                            ovf = true;
-                        }
+                    const int o = min(at, C::LCAP * 32 + lane);
+                    if (r2 < R2t) {
+                        lr[o] = r2;  // (its root where the lists are read: off the append path)
+                        if (!UM) lm[o] = c.w;
+                        at += 32;
                     }
                 }
             } else {
@@ -880,6 +986,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             nbuf = 0;
         };
         const T Rq2 = (T)Rq * (T)Rq;
+        set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, dy);
         // visit leaves within Rq (gather) or whose predicted smoothing
         // spheres reach this leaf (what the force pass will need); stage
         // only the former
@@ -887,8 +994,11 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         walk(
             b, dy,
             [&](const NodeBox &nb) {
-                near = box_within(boxA.plo, boxA.phi, nb.plo, nb.phi, Rq, ph);
-                return near || (record && box_overlap(boxA.plo, boxA.phi, nb.slo, nb.shi, 0.f, ph));
+                return up_within(sc.qb, nb) || (record && up_overlap(sc.qb, nb));
+            },
+            [&](const NodeBox &nb) {
+                near = box_within(sc.qb, nb, ph);
+                return record ? box_overlap(sc.qb, nb, ph) || near : near;
             },
             [&](unsigned mask, int first) {
                 if (lane == ng) {
@@ -905,17 +1015,23 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                                 : 0u;
                 if (!WRAP && am) to_wrap = true;
                 if (!WRAP && to_wrap) return;
+                const unsigned amo = WRAP ? by_order(am, gm) : 0u;
                 stage_group<T, C::CH>(
-                    b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, T, T, T) {},
+                    b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, int, const V &) {},
                     [&](int j) { return pm[j]; },
-                    [&](V &q, int k) {
-                        if (WRAP && ((am >> k) & 1u)) wrap_near<T>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
+                    [&](V &q, int o) {
+                        if (WRAP && ((amo >> o) & 1u)) wrap_near<T>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
                         return box_dist2<T>(q, flo, fhi) < Rq2;
                     },
                     [&](int slot, const V &q, int, int) { cand[slot] = q; }, flush);
             });
         flush();
         if (!WRAP && to_wrap) break;
+        if (LPP == 1 || !bal) {
+            cnt = at >> 5;
+            ovf = cnt > C::LCAP;
+            cnt = min(cnt, C::LCAP);
+        }
         if (LPP > 1 && bal) {
             const int mine_n = gcnt > sub ? (gcnt - sub - 1) / LPP + 1 : 0;
             cnt = mine_n < C::LCAP ? mine_n : C::LCAP;
@@ -1173,6 +1289,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
         // leaves; fn(r2, m_j) sees one candidate per lane
         auto visit_all = [&](float Rq, auto &&fn) {
             const T Rq2 = (T)Rq * (T)Rq;
+            set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, dy);
             int nbuf = 0;
             auto flush = [&]() {
                 __syncwarp();
@@ -1185,10 +1302,11 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
                 nbuf = 0;
             };
             walk(
-                b, dy, [&](const NodeBox &nb) { return box_within(boxA.plo, boxA.phi, nb.plo, nb.phi, Rq, ph); },
+                b, dy, [&](const NodeBox &nb) { return up_within(sc.qb, nb); },
+                [&](const NodeBox &nb) { return box_within(sc.qb, nb, ph); },
                 [&](unsigned mask, int first) {
                     stage_group<T, kFbCH>(
-                        b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, T, T, T) {},
+                        b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const V &) {},
                         [&](int j) { return pm[j]; },
                         [&](V &q, int) {
                             if (per) wrap_near<T>(sc, q, pi.x, pi.y, pi.z);  // then pi - q is the minimum image
@@ -1389,7 +1507,6 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     unsigned short *code = reinterpret_cast<unsigned short *>(mine + (C::CH + C::TAB) * sizeof(V) + C::scratch);
     unsigned short *lst = code + C::CH;
     const int pp = lane / LPP, sub = lane % LPP;
-    const unsigned below = (1u << lane) - 1u;
     const V *gph = (const V *)b.ph, *gvc = (const V *)b.vc, *gth = (const V *)b.th;
     const int p = b.leaf_pid[leaf];
     const ProbStatic &ps = b.prob[p];
@@ -1455,7 +1572,7 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     const bool wrap2 = WRAP && half_width(flo, fhi) + Rall >= halfL;  // staged vectors may still need a wrap
     bool to_wrap = false;  // (plain variant) met an ambiguous leaf pair: the wrapping variant takes the leaf
     int nbuf = 0, cnt = 0, ntab = 0, tA = -1;
-    unsigned gmask = 0u, am = 0u;
+    unsigned am = 0u;
     // table entry of a candidate leaf: its shift and first sorted index,
     // stored as ~index for an ambiguous leaf pair (whose pair vectors the
     // evaluation wraps)
@@ -1563,9 +1680,10 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         __syncwarp();
         nbuf = 0;
     };
+    set_query(sc.qb, boxA.plo, boxA.phi, R, ph, dy);
     auto node_test = [&](const NodeBox &nb) {
-        return box_within(boxA.plo, boxA.phi, nb.plo, nb.phi, R, ph) ||
-               box_overlap(boxA.plo, boxA.phi, nb.slo, nb.shi, 0.f, ph);
+        const bool near = box_within(sc.qb, nb, ph);
+        return box_overlap(sc.qb, nb, ph) || near;
     };
     auto visit = [&](unsigned mask, int first) {
             if (ntab + __popc(mask) > C::TAB) {
@@ -1579,30 +1697,27 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
                              : 0u;
             if (!WRAP && am) to_wrap = true;
             if (!WRAP && to_wrap) return;
+            const unsigned amo = WRAP ? by_order(am, mask) : 0u;
             stage_group<T, C::CH>(
                 b, leaf, mask, first, ph, nbuf, sc,
-                [&](bool has, int B, int stB, T Dx, T Dy, T Dz) {
-                    gmask = mask;
+                [&](bool has, int B, int stB, int ord, const V &D) {
                     if (has) {
-                        V t;
-                        t.x = Dx;
-                        t.y = Dy;
-                        t.z = Dz;
+                        V t = D;
                         t.w = bits_as_t((am >> lane) & 1u ? ~stB : stB, T(0));
-                        table[ntab + __popc(mask & below)] = t;
+                        table[ntab + ord] = t;
                     }
-                    const unsigned sm = __ballot_sync(FULL, has && B == leaf);
-                    if (sm) tA = ntab + __popc(mask & ((1u << (__ffs(sm) - 1)) - 1u));
+                    const unsigned ka = (unsigned)(leaf - first);  // the query leaf itself in this group
+                    if (ka < 32u && ((mask >> ka) & 1u)) tA = ntab + __popc(mask & ((1u << ka) - 1u));
                 },
                 [&](int j) { return gph[j]; },
-                [&](V &q, int k) {
-                    if (WRAP && ((am >> k) & 1u)) wrap_near<T>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
+                [&](V &q, int o) {
+                    if (WRAP && ((amo >> o) & 1u)) wrap_near<T>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
                     const T d2 = box_dist2<T>(q, flo, fhi);
                     return d2 < RA2 || d2 * q.w * q.w < T(KF::R * KF::R * 1.0001);
                 },
-                [&](int slot, const V &q, int k, int idx) {
+                [&](int slot, const V &q, int o, int idx) {
                     cand[slot] = q;
-                    code[slot] = (unsigned short)(((ntab + __popc(gmask & ((1u << k) - 1u))) << 5) | idx);
+                    code[slot] = (unsigned short)(((ntab + o) << 5) | idx);
                 },
                 test);
             ntab += __popc(mask);
@@ -1615,13 +1730,16 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         for (int g = 0; g < ngl; ++g) {
             const int2 e = b.group_pool[gofs + g];
             const unsigned mask = (unsigned)e.y;
-            bool ok = false;
-            if ((mask >> lane) & 1u) ok = node_test(b.nodes[0][e.x + lane]);
-            const unsigned fm = __ballot_sync(FULL, ok);
+            const bool in = (mask >> lane) & 1u;
+            const bool ok = node_test(b.nodes[0][e.x + (in ? lane : __ffs(mask) - 1)]);
+            const unsigned fm = __ballot_sync(FULL, ok && in);
             if (fm) visit(fm, e.x);
         }
     } else {
-        walk(b, dy, node_test, visit);
+        walk(
+            b, dy,
+            [&](const NodeBox &nb) { return up_within(sc.qb, nb) || up_overlap(sc.qb, nb); },
+            node_test, visit);
     }
     test();
     eval_lists();
