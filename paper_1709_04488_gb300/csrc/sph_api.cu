@@ -1135,7 +1135,7 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     CU(launch_build_leaves(b, c->prm.precision, st));
     CU(launch_set_sorted_h(b, h_in, st));
     CU(launch_refit(b, c->prm.precision, st));
-    CU(launch_neighbour_export(b, kind, h_in, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
+    CU(launch_neighbour_export(b, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
     CU(cudaStreamSynchronize(st));
     long long tot = 0;
     CU(cudaMemcpy(&tot, b.scratch64, sizeof tot, cudaMemcpyDeviceToHost));

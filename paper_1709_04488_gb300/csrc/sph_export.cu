@@ -1,42 +1,16 @@
-// Exact FP64 neighbour lists (CSR, ids ascending) for one problem: the
-// per-leaf tree walk retrieves the candidates (Sec. 4.2), membership is
-// decided on absolute FP64 positions with the periodic minimum image and
-// r^2 = dx*dx + dy*dy + dz*dz formed without fused multiply-add, compared
-// with (R_K h)^2 (gather list) or (R_K max(h_i,h_j))^2 (force list), R_K the
-// kernel's support in units of h (2 for M4, 3 for M6).  Used by
-// the tests to compare neighbour sets bit for bit with the CPU oracle.
-#include "sph_internal.cuh"
+// Exact FP64 neighbour lists (CSR, ids ascending) for one problem: a tree
+// walk per leaf retrieves the candidates (Sec. 4.2); membership is
+// r^2 = dx*dx + dy*dy + dz*dz < (R_K h_i)^2 (gather list) or < (R_K
+// max(h_i,h_j))^2 (force list) on absolute FP64 positions with the periodic
+// minimum image, formed without fused multiply-add, R_K the kernel's support
+// in units of h (2 for M4, 3 for M6).
+#include "sph_pairs.cuh"
 
 namespace sph {
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
 constexpr int kExportCap = 1024;  // neighbours one particle may have in the export
-
-__device__ __forceinline__ bool axis_overlap_x(float alo, float ahi, float blo, float bhi, float R, int periodic,
-                                               float L)
-{
-    float ca = 0.5f * (alo + ahi), ha = 0.5f * (ahi - alo);
-    float cb = 0.5f * (blo + bhi), hb = 0.5f * (bhi - blo);
-    float reach = ha + hb + R;
-    reach += 2e-6f * (fabsf(ca) + fabsf(cb) + reach) + 1e-30f;
-    float d = fabsf(ca - cb);
-    if (periodic) {
-        if (reach >= 0.5f * L) return true;
-        if (d > L) d -= L;
-        d = fminf(d, L - d);
-    }
-    return d <= reach;
-}
-
-__device__ __forceinline__ bool overlap_x(const float4 &alo, const float4 &ahi, const float4 &blo, const float4 &bhi,
-                                          float R, const PhysParams &ph)
-{
-    return axis_overlap_x(alo.x, ahi.x, blo.x, bhi.x, R, ph.periodic, (float)ph.box_len[0]) &&
-           axis_overlap_x(alo.y, ahi.y, blo.y, bhi.y, R, ph.periodic, (float)ph.box_len[1]) &&
-           axis_overlap_x(alo.z, ahi.z, blo.z, bhi.z, R, ph.periodic, (float)ph.box_len[2]);
-}
 
 __global__ void k_set_sorted_h(BatchView b, const double *h_in)
 {
@@ -49,121 +23,261 @@ __global__ void k_set_sorted_h(BatchView b, const double *h_in)
     b.hf[s] = __double2float_ru(h);
 }
 
-// pass 0: count into cnt[i]; pass 1: write sorted ids at offsets[i]
-__global__ void __launch_bounds__(128) k_export(BatchView b, int kind, int pass, unsigned *cnt,
-                                                const long long *offsets, int *idx, long long cap)
+// the membership test's own arithmetic (i, j: sorted indices)
+__device__ __forceinline__ bool export_member(const BatchView &b, const PhysParams &ph, long long i, long long j, int kind)
 {
-    __shared__ int buf[4][kExportCap];
-    __shared__ int sorted[4][kExportCap];
+    const double dx = min_image(__dsub_rn(b.sx[i], b.sx[j]), ph.box_len[0], ph.periodic);
+    const double dy = min_image(__dsub_rn(b.sy[i], b.sy[j]), ph.box_len[1], ph.periodic);
+    const double dz = min_image(__dsub_rn(b.sz[i], b.sz[j]), ph.box_len[2], ph.periodic);
+    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    const double hh = kind == 1 ? fmax(b.sh[i], b.sh[j]) : b.sh[i];
+    const double Rk = __dmul_rn(ph.kr, hh);  // R_K h, rounded as the oracle's
+    return r2 < __dmul_rn(Rk, Rk);
+}
+
+// One warp per leaf, as in the pair kernels: the leaf's candidates are staged
+// in FP32 in its frame, and each lane tests them for its particle.  A pair
+// within the rounding of the staged coordinates of the boundary (a few in
+// 1e4) is decided in FP64 (export_member); the others are decided by FP32.
+// (One walk per particle with every candidate tested in FP64, the first form
+// of this kernel, was bound by the FP64 pipe, 1/64 of the FP32 rate: 3.04 ms
+// per pass for 103823 particles; this form: 94-114 us.)  The pairs found wait in
+// a short list per lane, so that the lanes write them together.
+// FILL false: counts into cnt[i]; true: ids, in any order, at offsets[i].
+struct ExportCfg {
+    static constexpr int CH = 64, LC = 32, SB = 16, WPB = 4;
+    static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
+    static constexpr size_t per_warp = CH * (sizeof(float4) + sizeof(int)) + (size_t)LC * 32 * sizeof(int) + scratch;
+};
+template <typename V, bool FILL>
+__global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int kind, unsigned *cnt,
+                                                                const long long *offsets, int *idx, long long cap)
+{
+    using C = ExportCfg;
+    __shared__ __align__(32) unsigned char smem[C::WPB * C::per_warp];
+    __shared__ int wrote[C::WPB][32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    unsigned char *mine = smem + wib * C::per_warp;
+    float4 *cand = reinterpret_cast<float4 *>(mine);  // staged (x, y, z, R_K h rounded up)
+    StageScratch<float> &sc = *reinterpret_cast<StageScratch<float> *>(cand + C::CH);
+    int *code = reinterpret_cast<int *>(mine + C::CH * sizeof(float4) + C::scratch);  // sorted index per candidate
+    int *lst = code + C::CH;  // 2 x sorted index + (decided in FP64)
     const ProbStatic &ps = b.prob[0];
     const ProbDyn &d = b.dyn[0];
     const PhysParams &ph = ps.ph;
-    for (long long s = w; s < b.ntot; s += nw) {
-        const double xi = b.sx[s], yi = b.sy[s], zi = b.sz[s], hi = b.sh[s];
+    const V *pm = (const V *)b.pm;
+    const int lpp = ps.lpp, pp = lane / lpp, sub = lane % lpp;
+    // bound of a staged coordinate's error: each of the two offsets and the
+    // shift rounded once, the sums once more
+    const float err = 1e-6f * (ph.periodic ? ph.coord_max : d.coord_max) + 1e-30f;
+    const int nleaf = b.counters[0];
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int leaf = w; leaf < nleaf; leaf += nw) {
+        const NodeBox boxA = b.nodes[0][leaf];
+        const int st = b.leaf_start[leaf], nA = b.leaf_start[leaf + 1] - st;
+        const bool active = pp < nA;
+        const int s = st + (active ? pp : 0);
+        const V o = pm[s];
+        const float4 pi = make_float4((float)o.x, (float)o.y, (float)o.z, __fmul_ru(ph.kr_f, b.hf[s]));
+        float4 flo, fhi;
+        frame_box<float4, float>(pi, active, flo, fhi);
+        const float R = __fmul_ru(ph.kr_f, boxA.plo.w) * 1.0001f + 4.f * err;
+        const float R2 = R * R;
+        // the largest reach of a pair of this leaf, for the image handling
+        float Rall = R, extmax;
+        if (kind == 1) problem_top_max(b, d, Rall, extmax), Rall = __fmul_ru(ph.kr_f, Rall) * 1.0001f;
+        if (ph.periodic) load_box(sc, ph, flo, fhi);
+        const bool wrap2 = ph.periodic && half_width(flo, fhi) + Rall >= half_box(ph);
+        set_query(sc.qb, boxA.plo, boxA.phi, R, ph, d);
+        int nbuf = 0, n = 0;
         const long long i = (long long)b.perm[s] - ps.base;
-        float4 qlo = make_float4(__double2float_rd(xi), __double2float_rd(yi), __double2float_rd(zi), 0.f);
-        float4 qhi = make_float4(__double2float_ru(xi), __double2float_ru(yi), __double2float_ru(zi), 0.f);
-        const float R = __double2float_ru(ph.kr * hi) * 1.0001f;
-        int n = 0;
-        // walk (same structure as the pair kernels)
-        const int top = d.top_level;
-        unsigned mask[kMaxLevels + 1];
-        int base[kMaxLevels + 1];
-        auto test = [&](const NodeBox &nb) {
-            bool t = overlap_x(qlo, qhi, nb.plo, nb.phi, R, ph);
-            if (kind == 1) t = t || overlap_x(qlo, qhi, nb.slo, nb.shi, 0.f, ph);
-            return t;
+        const long long at = FILL ? offsets[i] : 0;
+        int total = 0;
+        if (FILL) wrote[wib][lane] = 0;
+        __syncwarp();
+        auto drain = [&]() {
+            for (int e = 0; e < n; ++e) {
+                const int c = lst[e * 32 + lane], j = c >> 1;
+                if ((c & 1) && !export_member(b, ph, s, j, kind)) continue;
+                ++total;
+                if (FILL) {
+                    const long long k = at + atomicAdd(&wrote[wib][pp], 1);
+                    if (k < cap) idx[k] = (int)((long long)b.perm[j] - ps.base);
+                }
+            }
+            n = 0;
         };
-        int lvl = top;
-        base[top] = 0;
-        mask[top] = __ballot_sync(FULL, lane < d.node_cnt[top] && test(b.nodes[top][d.node_off[top] + lane]));
-        for (;;) {
-            unsigned m = mask[lvl];
-            if (m == 0u) {
-                if (++lvl > top) break;
-                continue;
-            }
-            int c = __ffs(m) - 1;
-            mask[lvl] = m & (m - 1u);
-            int node = base[lvl] + c;
-            if (lvl == 0) {
-                int B = d.node_off[0] + node;
-                int stB = b.leaf_start[B], nB = b.leaf_start[B + 1] - stB;
-                bool hit = false;
-                int jid = 0;
-                if (lane < nB) {
-                    long long j = stB + lane;
-                    double dx = min_image(__dsub_rn(xi, b.sx[j]), ph.box_len[0], ph.periodic);
-                    double dy = min_image(__dsub_rn(yi, b.sy[j]), ph.box_len[1], ph.periodic);
-                    double dz = min_image(__dsub_rn(zi, b.sz[j]), ph.box_len[2], ph.periodic);
-                    double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-                    double hh = kind == 1 ? fmax(hi, b.sh[j]) : hi;
-                    const double Rk = __dmul_rn(ph.kr, hh);  // R_K h, rounded as the oracle's
-                    double R2 = __dmul_rn(Rk, Rk);
-                    hit = r2 < R2 && !(kind == 1 && j == s);
-                    jid = (int)((long long)b.perm[j] - ps.base);
+        auto test = [&]() {
+            __syncwarp();  // staged candidates visible to every lane
+            for (int k0 = 0; k0 < nbuf; k0 += C::SB) {
+                if (__any_sync(FULL, n > C::LC - C::SB)) drain();
+                const int ke = min(k0 + C::SB, nbuf);
+                for (int k = k0 + sub; k < ke; k += lpp) {
+                    const float4 c = cand[k];
+                    float rx = pi.x - c.x, ry = pi.y - c.y, rz = pi.z - c.z;
+                    if (wrap2) wrap3s<float>(sc, rx, ry, rz);
+                    const float r2 = rx * rx + ry * ry + rz * rz;
+                    const float Rk = kind == 1 ? fmaxf(pi.w, c.w) : pi.w;
+                    const float gap = r2 - Rk * Rk, tol = Rk * (8.f * err + 1e-5f * Rk) + err * err;
+                    const int j = code[k];
+                    if (active && gap < tol && !(kind == 1 && j == s))
+                        lst[n++ * 32 + lane] = 2 * j + (gap > -tol);
                 }
-                unsigned hm = __ballot_sync(FULL, hit);
-                if (pass == 1 && hit) {
-                    int pos = n + __popc(hm & ((1u << lane) - 1u));
-                    if (pos < kExportCap) buf[wib][pos] = jid;
-                }
-                n += __popc(hm);
-                continue;
             }
-            int ch = node * kBranch + lane;
-            bool ok = ch < d.node_cnt[lvl - 1] && test(b.nodes[lvl - 1][d.node_off[lvl - 1] + ch]);
-            --lvl;
-            base[lvl] = node * kBranch;
-            mask[lvl] = __ballot_sync(FULL, ok);
+            __syncwarp();
+            nbuf = 0;
+        };
+        auto node = [&](const NodeBox &nb) {
+            return up_within(sc.qb, nb) || (kind == 1 && up_overlap(sc.qb, nb));
+        };
+        walk(b, d, node, node, [&](unsigned mask, int first) {
+            int j = 0;
+            float Rj = 0.f;
+            stage_group<float, C::CH>(
+                b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
+                [&](int jj) {
+                    const V v = pm[jj];
+                    return make_float4((float)v.x, (float)v.y, (float)v.z, __int_as_float(jj));
+                },
+                [&](float4 &q, int) {
+                    j = __float_as_int(q.w);
+                    Rj = __fmul_ru(ph.kr_f, b.hf[j]);
+                    if (ph.periodic) wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
+                    const float d2 = box_dist2<float>(q, flo, fhi), Rjj = Rj + 4.f * err;
+                    return d2 < R2 || (kind == 1 && d2 < Rjj * Rjj * 1.0001f);
+                },
+                [&](int slot, const float4 &q, int, int) {
+                    cand[slot] = make_float4(q.x, q.y, q.z, Rj);
+                    code[slot] = j;
+                },
+                test);
+        });
+        test();
+        drain();
+        if (!FILL) {
+            for (int x = 1; x < lpp; x <<= 1) total += __shfl_xor_sync(FULL, total, x);
+            if (active && sub == 0) cnt[i] = (unsigned)total;
         }
-        if (pass == 0) {
-            if (lane == 0) cnt[i] = (unsigned)n;
-            continue;
-        }
-        __syncwarp();
-        int nn = n < kExportCap ? n : kExportCap;
-        if (n > kExportCap && lane == 0) atomicOr(&ps.diag->status, ST_OVERFLOW);
-        // rank sort (ids are distinct)
-        for (int e = lane; e < nn; e += 32) {
-            int v = buf[wib][e], r = 0;
-            for (int f = 0; f < nn; ++f) r += buf[wib][f] < v;
-            sorted[wib][r] = v;
-        }
-        __syncwarp();
-        long long o = offsets[i];
-        for (int e = lane; e < nn; e += 32)
-            if (o + e < cap) idx[o + e] = sorted[wib][e];
         __syncwarp();
     }
 }
 
-// exclusive scan of n counts into int64 offsets (one block; test-sized inputs)
-__global__ void k_offsets(const unsigned *cnt, long long n, long long *offsets, long long *total)
+// Sorts each particle's ids (one warp per particle; ids are distinct, so an
+// id's place is the number of smaller ones).  A particle whose list crosses
+// cap is left to k_export_cut.
+__global__ void __launch_bounds__(128) k_export_sort(BatchView b, const long long *offsets, int *idx, long long cap)
 {
-    __shared__ long long part[1024];
-    long long per = (n + blockDim.x - 1) / blockDim.x;
-    long long lo = threadIdx.x * per, hi = lo + per < n ? lo + per : n;
-    long long s = 0;
-    for (long long k = lo; k < hi; ++k) s += cnt[k];
-    part[threadIdx.x] = s;
+    __shared__ int buf[4][kExportCap];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (long long i = w; i < b.ntot; i += nw) {
+        const long long o = offsets[i], end = offsets[i + 1];
+        const int n = (int)(end - o);
+        if (n > kExportCap) {
+            if (lane == 0) atomicOr(&b.prob[0].diag->status, ST_OVERFLOW);
+            continue;
+        }
+        if (end > cap) continue;
+        for (int e = lane; e < n; e += 32) buf[wib][e] = idx[o + e];
+        __syncwarp();
+        for (int e = lane; e < n; e += 32) {
+            const int v = buf[wib][e];
+            int r = 0;
+#pragma unroll 4
+            for (int f = 0; f < n; ++f) r += buf[wib][f] < v;
+            idx[o + r] = v;
+        }
+        __syncwarp();
+    }
+}
+
+// The particle whose list crosses cap, if there is one (one block): its ids
+// are gathered again from all particles and those below cap written in order.
+__global__ void __launch_bounds__(1024) k_export_cut(BatchView b, int kind, const long long *offsets, int *idx, long long cap)
+{
+    __shared__ int buf[kExportCap];
+    __shared__ int s_pos, s_n;
+    if (offsets[b.ntot] <= cap) return;
+    const ProbStatic &ps = b.prob[0];
+    long long lo = 0, hi = b.ntot - 1;  // the last particle that starts below cap
+    while (lo < hi) {
+        const long long mid = (lo + hi + 1) >> 1;
+        if (offsets[mid] < cap) lo = mid;
+        else hi = mid - 1;
+    }
+    const long long i = lo, o = offsets[i];
+    const long long n = offsets[i + 1] - o;
+    if (!(o < cap && cap < o + n) || n > kExportCap) return;
+    if (threadIdx.x == 0) s_n = 0;
+    for (long long t = threadIdx.x; t < b.ntot; t += blockDim.x)
+        if ((long long)b.perm[t] - ps.base == i) s_pos = (int)t;
     __syncthreads();
-    for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-        long long t = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0;
-        __syncthreads();
-        part[threadIdx.x] += t;
-        __syncthreads();
+    const long long s = s_pos;
+    for (long long t = threadIdx.x; t < b.ntot; t += blockDim.x)
+        if (!(kind == 1 && t == s) && export_member(b, ps.ph, s, t, kind)) {
+            const int k = atomicAdd(&s_n, 1);
+            if (k < kExportCap) buf[k] = (int)((long long)b.perm[t] - ps.base);
+        }
+    __syncthreads();
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+        const int v = buf[e];
+        int r = 0;
+        for (int f = 0; f < n; ++f) r += buf[f] < v;
+        if (o + r < cap) idx[o + r] = v;
     }
-    long long run = part[threadIdx.x] - s;
-    for (long long k = lo; k < hi; ++k) {
-        offsets[k] = run;
-        run += cnt[k];
+}
+
+// Exclusive scan of n counts into int64 offsets: the sum of each block's
+// share, then each block's scan of its share from the sums before it.
+constexpr int kScanThreads = 1024, kScanBlocks = 1024;
+__device__ __forceinline__ long long scan_share(long long n)
+{
+    const long long per = (n + kScanBlocks - 1) / kScanBlocks;
+    return (per + kScanThreads - 1) / kScanThreads * kScanThreads;
+}
+__device__ __forceinline__ long long block_sum(long long v, long long *red)
+{
+    v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    long long t = 0;
+    for (int k = 0; k < kScanThreads / 32; ++k) t += red[k];
+    return t;
+}
+__global__ void __launch_bounds__(kScanThreads) k_count_sums(const unsigned *cnt, long long n, long long *part)
+{
+    __shared__ long long red[kScanThreads / 32];
+    const long long per = scan_share(n), lo = blockIdx.x * per, hi = lo + per < n ? lo + per : n;
+    long long s = 0;
+    for (long long k = lo + threadIdx.x; k < hi; k += kScanThreads) s += cnt[k];
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+__global__ void __launch_bounds__(kScanThreads) k_offsets(const unsigned *cnt, long long n, const long long *part,
+                                                          long long *offsets, long long *total)
+{
+    __shared__ long long red[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const long long per = scan_share(n), lo = blockIdx.x * per, hi = lo + per < n ? lo + per : n;
+    long long run = block_sum(threadIdx.x < blockIdx.x ? part[threadIdx.x] : 0, red);
+    for (long long k0 = lo; k0 < hi; k0 += kScanThreads) {
+        const long long k = k0 + threadIdx.x;
+        const int c = k < hi ? (int)cnt[k] : 0, incl = warp_incl_scan<int>(c);
+        __syncthreads();
+        if (lane == 31) red[wib] = incl;
+        __syncthreads();
+        long long before = run, all = 0;
+        for (int v = 0; v < kScanThreads / 32; ++v) {
+            if (v < wib) before += red[v];
+            all += red[v];
+        }
+        if (k < hi) offsets[k] = before + incl - c;
+        run += all;
     }
-    if (threadIdx.x == blockDim.x - 1) {
-        offsets[n] = part[threadIdx.x];
-        *total = part[threadIdx.x];
+    if (hi == n && lo < n && threadIdx.x == 0) {
+        offsets[n] = run;
+        *total = run;
     }
 }
 
@@ -176,20 +290,28 @@ cudaError_t launch_set_sorted_h(const BatchView &b, const double *h_in, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t launch_neighbour_export(const BatchView &b, int kind, const double *h_in, long long *offsets,
-                                    int *idx, long long cap, long long *total_dev, cudaStream_t st)
+cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind, long long *offsets, int *idx,
+                                    long long cap, long long *total_dev, cudaStream_t st)
 {
-    (void)h_in;
     if (b.ntot == 0) {
         cudaMemsetAsync(offsets, 0, sizeof(long long), st);
         cudaMemsetAsync(total_dev, 0, sizeof(long long), st);
         return cudaGetLastError();
     }
-    unsigned *cnt = b.flag;  // reuse: the leaf flags are no longer needed
-    int grid = dev_info().sm_count * 4;
-    k_export<<<grid, 128, 0, st>>>(b, kind, 0, cnt, offsets, idx, cap);
-    k_offsets<<<1, 1024, 0, st>>>(cnt, b.ntot, offsets, total_dev);
-    k_export<<<grid, 128, 0, st>>>(b, kind, 1, cnt, offsets, idx, cap);
+    unsigned *cnt = b.flag;                        // reuse: the leaf flags are no longer needed,
+    long long *part = (long long *)b.keys[1];      // nor the sort's second key buffer
+    const int sms = dev_info().sm_count, grid = sms * 8;
+    const long long n = b.ntot, share = (n + kScanBlocks - 1) / kScanBlocks;
+    const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
+                         ((share + kScanThreads - 1) / kScanThreads * kScanThreads));
+    const auto count = precision == SPH_PREC_FP64 ? k_export<dbl4, false> : k_export<float4, false>;
+    const auto fill = precision == SPH_PREC_FP64 ? k_export<dbl4, true> : k_export<float4, true>;
+    count<<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
+    k_count_sums<<<nb, kScanThreads, 0, st>>>(cnt, n, part);
+    k_offsets<<<nb, kScanThreads, 0, st>>>(cnt, n, part, offsets, total_dev);
+    fill<<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
+    k_export_sort<<<grid, 128, 0, st>>>(b, offsets, idx, cap);
+    k_export_cut<<<1, 1024, 0, st>>>(b, kind, offsets, idx, cap);
     return cudaGetLastError();
 }
 
