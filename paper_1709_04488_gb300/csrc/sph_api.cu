@@ -68,6 +68,7 @@ void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precis
     for (double **p : sd) *p = c.take<double>(n);
     void **st[] = {&b.pm, &b.ph, &b.vc, &b.th};
     for (void **p : st) *p = c.take<char>(v4 * n);
+    b.pmf = precision == SPH_PREC_FP64 ? c.take<float4>(n) : (float4 *)b.pm;
     b.sal = c.take<char>(v4 / 4 * n);
     b.scd = c.take<char>(v4 / 4 * n);
     b.divv = c.take<float>(n);
@@ -173,7 +174,11 @@ static int choose_lpp(long long n, int precision, int requested, int kernel)
     if (l != 1 && l != 2 && l != 4 && l != 8) l = 4;
     if (kernel == SPH_KERNEL_M6 && requested == 0) l = l >= 4 ? 8 : 2 * l;
     if (kernel == SPH_KERNEL_M6 && l < 2) l = 2;
-    if (precision == SPH_PREC_FP64) l = (l >= 4) ? 4 : 2;
+    // FP64 pair kernels run 2 or 4 lanes; 4 where leaves of 16 particles would
+    // not fill one wave of warps (12 per SM): lattice 4096, two evaluations and
+    // three steps: 2.74 ms with 2 lanes, 1.66 with 4; from about 1e4 particles
+    // on the two differ by the last wave's fill only
+    if (precision == SPH_PREC_FP64) l = l >= 4 || (requested == 0 && n <= 8000) ? 4 : 2;
     return l;
 }
 
@@ -1135,7 +1140,7 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     CU(launch_build_leaves(b, c->prm.precision, st));
     CU(launch_set_sorted_h(b, h_in, st));
     CU(launch_refit(b, c->prm.precision, st));
-    CU(launch_neighbour_export(b, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
+    CU(launch_neighbour_export(b, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
     CU(cudaStreamSynchronize(st));
     long long tot = 0;
     CU(cudaMemcpy(&tot, b.scratch64, sizeof tot, cudaMemcpyDeviceToHost));

@@ -49,7 +49,7 @@ struct ExportCfg {
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
     static constexpr size_t per_warp = CH * (sizeof(float4) + sizeof(int)) + (size_t)LC * 32 * sizeof(int) + scratch;
 };
-template <typename V, bool FILL>
+template <bool FILL>
 __global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int kind, unsigned *cnt,
                                                                 const long long *offsets, int *idx, long long cap)
 {
@@ -65,7 +65,6 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int
     const ProbStatic &ps = b.prob[0];
     const ProbDyn &d = b.dyn[0];
     const PhysParams &ph = ps.ph;
-    const V *pm = (const V *)b.pm;
     const int lpp = ps.lpp, pp = lane / lpp, sub = lane % lpp;
     // bound of a staged coordinate's error: each of the two offsets and the
     // shift rounded once, the sums once more
@@ -77,8 +76,8 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int
         const int st = b.leaf_start[leaf], nA = b.leaf_start[leaf + 1] - st;
         const bool active = pp < nA;
         const int s = st + (active ? pp : 0);
-        const V o = pm[s];
-        const float4 pi = make_float4((float)o.x, (float)o.y, (float)o.z, __fmul_ru(ph.kr_f, b.hf[s]));
+        float4 pi = b.pmf[s];
+        pi.w = __fmul_ru(ph.kr_f, b.hf[s]);
         float4 flo, fhi;
         frame_box<float4, float>(pi, active, flo, fhi);
         const float R = __fmul_ru(ph.kr_f, boxA.plo.w) * 1.0001f + 4.f * err;
@@ -136,8 +135,9 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int
             stage_group<float, C::CH>(
                 b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
                 [&](int jj) {
-                    const V v = pm[jj];
-                    return make_float4((float)v.x, (float)v.y, (float)v.z, __int_as_float(jj));
+                    float4 q = b.pmf[jj];
+                    q.w = __int_as_float(jj);
+                    return q;
                 },
                 [&](float4 &q, int) {
                     j = __float_as_int(q.w);
@@ -290,8 +290,8 @@ cudaError_t launch_set_sorted_h(const BatchView &b, const double *h_in, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind, long long *offsets, int *idx,
-                                    long long cap, long long *total_dev, cudaStream_t st)
+cudaError_t launch_neighbour_export(const BatchView &b, int kind, long long *offsets, int *idx, long long cap,
+                                    long long *total_dev, cudaStream_t st)
 {
     if (b.ntot == 0) {
         cudaMemsetAsync(offsets, 0, sizeof(long long), st);
@@ -304,12 +304,10 @@ cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind,
     const long long n = b.ntot, share = (n + kScanBlocks - 1) / kScanBlocks;
     const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
                          ((share + kScanThreads - 1) / kScanThreads * kScanThreads));
-    const auto count = precision == SPH_PREC_FP64 ? k_export<dbl4, false> : k_export<float4, false>;
-    const auto fill = precision == SPH_PREC_FP64 ? k_export<dbl4, true> : k_export<float4, true>;
-    count<<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
+    k_export<false><<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
     k_count_sums<<<nb, kScanThreads, 0, st>>>(cnt, n, part);
     k_offsets<<<nb, kScanThreads, 0, st>>>(cnt, n, part, offsets, total_dev);
-    fill<<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
+    k_export<true><<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
     k_export_sort<<<grid, 128, 0, st>>>(b, offsets, idx, cap);
     k_export_cut<<<1, 1024, 0, st>>>(b, kind, offsets, idx, cap);
     return cudaGetLastError();

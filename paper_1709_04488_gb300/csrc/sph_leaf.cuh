@@ -151,6 +151,7 @@ __device__ __forceinline__ void leaf_props_one(const BatchView &b, int leaf)
             v.z = (decltype(v.z))d[2];
             v.w = ps.uniform_m ? (decltype(v.w))ps.m_uniform : (decltype(v.w))b.sm[st + lane];
             ((T4 *)b.pm)[st + lane] = v;
+            if (sizeof(v.x) == 8) b.pmf[st + lane] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
             const float o[3] = {offset_f(v.x), offset_f(v.y), offset_f(v.z)};
             for (int a = 0; a < 3; ++a) ex[a] = fabsf(o[a]);
             // predicted smoothing spheres: 1.1 x the guessed h (the h the

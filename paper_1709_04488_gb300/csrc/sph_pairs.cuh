@@ -10,6 +10,14 @@
 // differenced in FP64, then cast), and each lane keeps its own list of
 // in-range candidates so that the arithmetic runs without divergence.
 //
+// FP64 problems (SPH_PREC_FP64): this GPU runs FP64 at 1/64 of the FP32 rate,
+// so the walk, the staging and the tests of the candidates run in FP32 with
+// the rounding of the staged coordinates to spare, and only the pairs that
+// pass take FP64: their distance from the FP64 positions, the exact
+// membership, the sums.  The FP64 pipe is 72-75 % busy (k_forces 947 -> 660 us,
+// k_density 626 -> 510 us at 36864 particles of the Sod tube, two lanes per
+// particle; smaller problems 1.7-4 times faster).
+//
 //  k_density   Eqs. SPHRHO, HRHO, OMEGA: Newton-Raphson on
 //              F(h) = rho(h) - m (eta/h)^3 over the cached list of (r^2, m_j)
 //              with the same bracketing fallback as the oracle; the list is
@@ -27,6 +35,8 @@
 #include "sph_internal.cuh"
 #include "sph_leaf.cuh"
 #include "sph_tuned.h"
+
+#include <type_traits>
 
 namespace sph {
 
@@ -47,6 +57,11 @@ __device__ __forceinline__ float tinf<float>() { return INFINITY; }
 template <>
 __device__ __forceinline__ double tinf<double>() { return INFINITY; }
 
+// a < b for a >= 0 (or -1) and b > 0: in FP64 on the bit patterns, which keeps
+// the comparison off the FP64 pipe
+__device__ __forceinline__ bool lt_pos(float a, float b) { return a < b; }
+__device__ __forceinline__ bool lt_pos(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+
 // Smoothing kernels of Sec. 2, W(r, h) = sigma f(q) / h^3 with q = r / h and
 // support q < R: fdf(q) gives f and f', df(q) f' alone.
 template <int K>
@@ -60,13 +75,13 @@ struct Kern<SPH_KERNEL_M4> {
     template <typename T>
     static __device__ __forceinline__ void fdf(T q, T &f, T &df)
     {
-        T t = q < T(2) ? T(2) - q : T(0);
+        T t = lt_pos(q, T(2)) ? T(2) - q : T(0);
         T t2 = t * t;
         T f2 = T(0.25) * t2 * t, df2 = T(-0.75) * t2;
         T q2 = q * q;
         T f1 = T(1) + q2 * (T(0.75) * q - T(1.5));
         T df1 = q * (T(2.25) * q - T(3));
-        bool in = q < T(1);
+        bool in = lt_pos(q, T(1));
         f = in ? f1 : f2;
         df = in ? df1 : df2;
     }
@@ -86,14 +101,14 @@ struct Kern<SPH_KERNEL_M6> {
     template <typename T>
     static __device__ __forceinline__ void fdf(T q, T &f, T &df)
     {
-        T a = q < T(3) ? T(3) - q : T(0);
-        T c = q < T(2) ? T(2) - q : T(0);
+        T a = lt_pos(q, T(3)) ? T(3) - q : T(0);
+        T c = lt_pos(q, T(2)) ? T(2) - q : T(0);
         T a4 = (a * a) * (a * a), c4 = (c * c) * (c * c);
         T f2 = a4 * a - T(6) * (c4 * c), df2 = T(30) * c4 - T(5) * a4;
         T q2 = q * q;
         T f1 = T(66) + q2 * (T(-60) + q2 * (T(30) - T(10) * q));
         T df1 = q * (T(-120) + q2 * (T(120) - T(50) * q));
-        bool in = q < T(1);
+        bool in = lt_pos(q, T(1));
         f = in ? f1 : f2;
         df = in ? df1 : df2;
     }
@@ -177,21 +192,21 @@ __device__ __forceinline__ double fma_rn<double>(double a, double b, double c) {
 template <typename T>
 __device__ __forceinline__ T Kern<SPH_KERNEL_M4>::df(T q)
 {
-    const T t = q < T(2) ? sub_rn(T(2), q) : T(0);
+    const T t = lt_pos(q, T(2)) ? sub_rn(T(2), q) : T(0);
     const T df2 = mul_rn(mul_rn(T(-0.75), t), t);
     const T df1 = mul_rn(q, fma_rn(T(2.25), q, T(-3)));
-    return q < T(1) ? df1 : df2;
+    return lt_pos(q, T(1)) ? df1 : df2;
 }
 
 template <typename T>
 __device__ __forceinline__ T Kern<SPH_KERNEL_M6>::df(T q)
 {
-    const T a = q < T(3) ? sub_rn(T(3), q) : T(0);
-    const T c = q < T(2) ? sub_rn(T(2), q) : T(0);
+    const T a = lt_pos(q, T(3)) ? sub_rn(T(3), q) : T(0);
+    const T c = lt_pos(q, T(2)) ? sub_rn(T(2), q) : T(0);
     const T a2 = mul_rn(a, a), c2 = mul_rn(c, c);
     const T df2 = fma_rn(T(30), mul_rn(c2, c2), mul_rn(T(-5), mul_rn(a2, a2)));
     const T df1 = mul_rn(q, fma_rn(mul_rn(q, q), fma_rn(T(-50), q, T(120)), T(-120)));
-    return q < T(1) ? df1 : df2;
+    return lt_pos(q, T(1)) ? df1 : df2;
 }
 
 // 2/(rho_i + rho_j): a deterministic function of the commutative sum, so
@@ -547,18 +562,22 @@ __device__ __forceinline__ T box_dist2(const V &q, const V &lo, const V &hi)
     return dx * dx + dy * dy + dz * dz;
 }
 
-// shift of candidate leaf B's reference point from the query leaf A's: FP64
-// difference, minimum image (min_image's, decided on the bit pattern of |d|:
-// the comparisons would run on the narrow FP64 pipe), cast
-template <typename T>
-__device__ __forceinline__ T leaf_shift(double cb, double ca, double L, int periodic)
+// min_image, decided on the bit pattern of |d|: the comparisons would run on
+// the FP64 pipe, 1/64 of the FP32 rate
+__device__ __forceinline__ double min_image_bits(double d, double L, int periodic)
 {
-    double d = cb - ca;
     if (periodic) {
         const long long ad = __double_as_longlong(d) & 0x7fffffffffffffffll;
         if (ad > __double_as_longlong(0.5 * L)) d += __longlong_as_double(__double_as_longlong(L) | (~__double_as_longlong(d) & (1ll << 63)));
     }
-    return (T)d;
+    return d;
+}
+// shift of candidate leaf B's reference point from the query leaf A's: FP64
+// difference, minimum image, cast
+template <typename T>
+__device__ __forceinline__ T leaf_shift(double cb, double ca, double L, int periodic)
+{
+    return (T)min_image_bits(cb - ca, L, periodic);
 }
 
 // Stage the particles of the leaves first + k (bit k of mask) that keep()
@@ -705,22 +724,42 @@ __device__ __forceinline__ bool nr_update(T &h, T &lo, T &hi, T rho, T drho, T m
     return conv;
 }
 
+// The items of a pair kernel's warp: one by position first, the first warp of
+// every block before the second ones, so that a launch of fewer items than
+// warps spreads over all SMs (tickets alone went to the warps of the blocks
+// that started first, four to an SM, and left the other SMs idle); tickets
+// after that.
+__device__ __forceinline__ int first_item() { return (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x); }
+__device__ __forceinline__ int next_item(int *ticket)
+{
+    int t = 0;
+    if ((threadIdx.x & 31) == 0) t = atomicAdd(ticket, 1);
+    return (int)(gridDim.x * (blockDim.x >> 5)) + __shfl_sync(FULL, t, 0);
+}
+
 template <typename T, int LPP, bool UM, int K>
 struct DCfg {
     using V = typename Vec4<T>::type;
     // list entries per lane: room for ~2x the mean neighbour count per
     // particle within the list radius (M4 at eta = 1.2: ~63; M6 at eta = 1.0:
     // ~123, served by 2 or more lanes per particle)
-    static constexpr int LCAP = K == SPH_KERNEL_M6 ? (LPP <= 2 ? 96 : LPP == 4 ? 64 : 32)
-                                                   : LPP == 1 ? SPH_DENS_LCAP1 : LPP == 2 ? 64 : LPP == 4 ? 40 : 24;
+    static constexpr bool D64 = sizeof(T) == 8;
+    // (FP64 deals its entries to the lanes by rank, so that they fill evenly:
+    // room for 120 (M6: 192) per particle)
+    static constexpr int LCAP = D64 ? (K == SPH_KERNEL_M6 ? 192 : 120) / LPP
+                                : K == SPH_KERNEL_M6 ? (LPP <= 2 ? 96 : LPP == 4 ? 64 : 32)
+                                                     : LPP == 1 ? SPH_DENS_LCAP1 : LPP == 2 ? 64 : LPP == 4 ? 40 : 24;
     static constexpr int CH = SPH_DENS_CH;
-    static constexpr int WPB = 4;
-    static constexpr int MINB = LPP == 1 ? SPH_DENS_MINB1 : SPH_DENS_MINB;  // blocks per SM the registers allow
+    static constexpr int WPB = D64 ? 2 : 4;
+    static constexpr int MINB = D64 ? 4 : LPP == 1 ? SPH_DENS_MINB1 : SPH_DENS_MINB;  // blocks per SM the registers allow
+    // FP64: rows of pairs waiting for their FP64 distance, candidates per room check
+    static constexpr int LC = 32, SB = 32;
+    static constexpr size_t wait = D64 ? (size_t)LC * 32 * sizeof(int) + CH * sizeof(int) : 0;
     static constexpr int LW = UM ? 1 : 2;  // list words per entry: r^2 (and m_j unless masses are equal)
-    static constexpr size_t scratch = (sizeof(StageScratch<T>) + 31) & ~(size_t)31;
+    static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
     // (a row beyond the capacity takes the entries that no longer fit)
     static constexpr size_t lists = (size_t)(LCAP + 1) * 32 * LW * sizeof(T);
-    static constexpr size_t per_warp = CH * sizeof(V) + lists + scratch;
+    static constexpr size_t per_warp = CH * sizeof(float4) + lists + scratch + wait;
     static constexpr size_t smem = WPB * per_warp;
 };
 
@@ -850,6 +889,54 @@ __device__ __forceinline__ void density_epilogue(const BatchView &b, const ProbS
         atomicOr(&ps.diag->status, ST_NONFINITE);
 }
 
+// FP64 density: Newton-Raphson on the FP64 lists in FP32 arithmetic, as far
+// as FP32 resolves h, so that the FP64 iteration that follows (same stopping
+// rule, FP64 sums) starts within ~1e-7 of the root and needs two passes over
+// the list where the previous step's h needs four; h stays as it is where
+// it is that close already, or where the FP32 steps leave [0.8, 1.25] of it.
+template <int LPP, bool UM, int K, typename T>
+__device__ __forceinline__ void presolve_f32(const T *lr, const T *lm, int cnt, bool on, T mi, T mu_all, T eta3, T hs, T &h)
+{
+    using KF = Kern<K>;
+    const int lane = threadIdx.x & 31;
+    const float m = (float)mi, e3 = (float)eta3, sigma = (float)KF::sigma, mu = (float)mu_all;
+    const float h0 = (float)h, hlim = fminf(1.25f * h0, (float)hs * 0.9999f);
+    float x = h0;
+    bool go = on, moved = false;
+    for (int it = 0; it < 6 && __any_sync(FULL, go); ++it) {
+        float S0 = 0.f, S1 = 0.f;
+        const float xi = 1.f / x;
+        if (go)
+            for (int e = 0; e < cnt; ++e) {
+                const float q = (float)lr[e * 32 + lane] * xi;
+                const float mj = UM ? mu : (float)lm[e * 32 + lane];
+                float f, df;
+                KF::fdf(q, f, df);
+                S0 += mj * f;
+                S1 += mj * q * df;
+            }
+        S0 = group_sum<LPP>(S0);
+        S1 = group_sum<LPP>(S1);
+        if (go) {
+            const float x3 = xi * xi * xi;
+            const float F = sigma * S0 * x3 - m * e3 * x3;
+            const float dF = -sigma * x3 * xi * (3.f * S0 + S1) + 3.f * m * e3 * x3 * xi;
+            const float xn = dF > 0.f ? x - F / dF : -1.f;
+            const float step = fabsf(xn - x);
+            if (!(xn >= 0.8f * h0) || !(xn <= hlim)) {
+                go = moved = false;
+            } else if (it == 0 && step < 1e-5f * x) {
+                go = false;
+            } else {
+                go = step >= 1e-6f * x;
+                x = xn;
+                moved = true;
+            }
+        }
+    }
+    if (moved) h = (T)x;
+}
+
 // One query leaf of the density pass.  WRAP: pair vectors are wrapped to
 // the minimum image where they may miss it (see the wrap helpers).  Returns
 // false, having written nothing, when the plain variant meets an ambiguous
@@ -864,10 +951,13 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     const T sigma = T(KF::sigma);
     using V = typename C::V;
     const int lane = threadIdx.x & 31;
-    V *cand = reinterpret_cast<V *>(mine);
-    T *lr = reinterpret_cast<T *>(mine + C::CH * sizeof(V));  // r_ij^2 per entry
+    constexpr bool D64 = C::D64;
+    float4 *cand = reinterpret_cast<float4 *>(mine);
+    T *lr = reinterpret_cast<T *>(mine + C::CH * sizeof(float4));  // r_ij^2 per entry (FP64: r_ij)
     T *lm = lr + (C::LCAP + 1) * 32;  // used only when masses differ
-    StageScratch<T> &sc = *reinterpret_cast<StageScratch<T> *>(mine + C::CH * sizeof(V) + C::lists);
+    StageScratch<float> &sc = *reinterpret_cast<StageScratch<float> *>(mine + C::CH * sizeof(float4) + C::lists);
+    // FP64: the staged candidates' sorted indices, and the pairs that wait
+    int *code = reinterpret_cast<int *>(mine + C::CH * sizeof(float4) + C::lists + C::scratch), *lst = code + C::CH;
     const int pp = lane / LPP, sub = lane % LPP;
     const V *pm = (const V *)b.pm;
     const int p = b.leaf_pid[leaf];
@@ -881,12 +971,17 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     const bool active = task_member<T>(b, st, nA, k0, pp, pos);
     const long long s = st + (active ? pos : 0);
     const V pi = pm[s];
+    const float4 pf = b.pmf[s];  // (FP32: pi)
     const T mi = pi.w;
+    // FP64: bound of a staged coordinate's error (its offset and shift rounded
+    // once each, their sum once more), and the particle's position
+    const float err = D64 ? 1e-6f * (ps.ph.periodic ? ps.ph.coord_max : b.dyn[p].coord_max) + 1e-30f : 0.f;
+    const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles (the others
     // of the leaf keep their last solve, restaged by k_block_restage)
     if (k0 >= 0) task_box(b, leaf, pi, active, boxA.plo.w, boxA);
-    V flo, fhi;
-    frame_box<V, T>(pi, active, flo, fhi);
+    float4 flo, fhi;
+    frame_box<float4, float>(pf, active, flo, fhi);
     const float halfL = ph.periodic ? half_box(ph) : INFINITY;
     const T eta3 = (T)(ph.eta * ph.eta * ph.eta);
     const T tol = (T)ph.h_tol;
@@ -926,25 +1021,74 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         float Rq = warp_max((active && !fail) ? __fmul_ru(KR_f, (float)hs) : 0.f) * 1.0001f;
         const T R2 = (T(KF::R) * hs) * (T(KF::R) * hs);
         Rq_last = Rq;
-        if (ph.periodic) set_thr(sc, boxA.slo.w, Rq);
-        const bool wrap2 = WRAP && half_width(flo, fhi) + Rq >= halfL;  // staged vectors may still need a wrap
+        if (!D64 && ph.periodic) set_thr(sc, boxA.slo.w, Rq);
+        const bool wrap2 = (WRAP || D64) && half_width(flo, fhi) + Rq >= halfL;  // staged vectors may still need a wrap
         ng = 0;
         cnt = 0;
         int gcnt = 0, at = lane;  // at: where this lane's next entry goes
-        const T R2t = active && !fail ? R2 : T(-1);
+        const float Rs = KR_f * (float)hs;
+        const float R2t = active && !fail ? D64 ? Rs * (Rs * 1.00002f + 8.f * err) + err * err : (float)R2 : -1.f;
         bool ovf = false;
         int nbuf = 0;
+        // FP64: the waiting pairs' distances, from the FP64 positions
+        auto drain = [&]() {
+            __syncwarp();
+            const int n = gcnt > sub ? (gcnt - sub - 1) / LPP + 1 : 0;
+            for (int e = 0; e < n; ++e) {
+                const int j = lst[e * 32 + lane];
+                const T dx = (T)min_image_bits(X[0] - b.sx[j], ph.box_len[0], ph.periodic);
+                const T dyy = (T)min_image_bits(X[1] - b.sy[j], ph.box_len[1], ph.periodic);
+                const T dz = (T)min_image_bits(X[2] - b.sz[j], ph.box_len[2], ph.periodic);
+                const T r2 = dx * dx + dyy * dyy + dz * dz;
+                if (lt_pos(r2, R2)) {
+                    if (cnt < C::LCAP) {
+                        lr[cnt * 32 + lane] = sqrt(r2);
+                        if (!UM) lm[cnt * 32 + lane] = (T)b.sm[j];
+                        ++cnt;
+                    } else {
+                        ovf = true;
+                    }
+                }
+            }
+            gcnt = 0;
+            __syncwarp();
+        };
         auto flush = [&]() {
             __syncwarp();  // staged candidates visible to every lane
-            if (LPP == 1 || !bal) {
+            if constexpr (D64) {
+                // tested in FP32 with the coordinates' error to spare; the hits
+                // are dealt to the particle's lanes by rank
+                const unsigned below = (1u << sub) - 1u;
+                for (int kb = 0; kb < nbuf; kb += C::SB) {
+                    if (__any_sync(FULL, gcnt > C::LC * LPP - C::SB)) drain();
+                    const int ke = min(kb + C::SB, nbuf);
+#pragma unroll 4
+                    for (int kk = kb; kk < ke; kk += LPP) {
+                        const int k = kk + sub;
+                        bool hit = false;
+                        if (k < ke) {
+                            const float4 c = cand[k];
+                            float dx = pf.x - c.x, dyy = pf.y - c.y, dz = pf.z - c.z;
+                            if (wrap2) wrap3s<float>(sc, dx, dyy, dz);
+                            hit = dx * dx + dyy * dyy + dz * dz < R2t;
+                        }
+                        const unsigned gm = (__ballot_sync(FULL, hit) >> (pp * LPP)) & ((1u << LPP) - 1u);
+                        if (hit) {
+                            const int e = gcnt + __popc(gm & below);
+                            lst[(e / LPP) * 32 + pp * LPP + e % LPP] = code[k];
+                        }
+                        gcnt += __popc(gm);
+                    }
+                }
+            } else if (LPP == 1 || !bal) {
                 // (an entry beyond the capacity goes to the spare row: no
                 // branch on the append path)
 #pragma unroll 4
                 for (int k = sub; k < nbuf; k += LPP) {
-                    V c = cand[k];
-                    T dx = pi.x - c.x, dyy = pi.y - c.y, dz = pi.z - c.z;
-                    if (wrap2) wrap3s<T>(sc, dx, dyy, dz);
-                    T r2 = dx * dx + dyy * dyy + dz * dz;
+                    const float4 c = cand[k];
+                    float dx = pf.x - c.x, dyy = pf.y - c.y, dz = pf.z - c.z;
+                    if (wrap2) wrap3s<float>(sc, dx, dyy, dz);
+                    const float r2 = dx * dx + dyy * dyy + dz * dz;
                     const int o = min(at, C::LCAP * 32 + lane);
                     if (r2 < R2t) {
                         lr[o] = r2;  // (its root where the lists are read: off the append path)
@@ -959,11 +1103,11 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                     bool hit = false;
                     T r = T(0), mj = T(0);  // (r: r_ij^2)
                     if (k < nbuf) {
-                        V c = cand[k];
-                        T dx = pi.x - c.x, dyy = pi.y - c.y, dz = pi.z - c.z;
-                        if (wrap2) wrap3s<T>(sc, dx, dyy, dz);
-                        T r2 = dx * dx + dyy * dyy + dz * dz;
-                        hit = active && !fail && r2 < R2;
+                        const float4 c = cand[k];
+                        float dx = pf.x - c.x, dyy = pf.y - c.y, dz = pf.z - c.z;
+                        if (wrap2) wrap3s<float>(sc, dx, dyy, dz);
+                        const float r2 = dx * dx + dyy * dyy + dz * dz;
+                        hit = r2 < R2t;
                         r = r2;
                         mj = c.w;
                     }
@@ -985,7 +1129,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             __syncwarp();
             nbuf = 0;
         };
-        const T Rq2 = (T)Rq * (T)Rq;
+        const float Rq2 = (Rq + 4.f * err) * (Rq + 4.f * err);
         set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, dy);
         // visit leaves within Rq (gather) or whose predicted smoothing
         // spheres reach this leaf (what the force pass will need); stage
@@ -1010,38 +1154,53 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                 const unsigned gm = __ballot_sync(FULL, near && ((mask >> lane) & 1u));
                 if (gm == 0u) return;
                 // candidate leaves that form an ambiguous pair with A (periodic)
+                // (FP64 takes its pairs' minimum images from the positions: every
+                // staged candidate moves to its image nearest the query box)
                 const unsigned am =
-                    ph.periodic ? __ballot_sync(FULL, ((gm >> lane) & 1u) && ambiguous(b.nodes[0][first + lane].slo.w, sc))
-                                : 0u;
+                    !D64 && ph.periodic ? __ballot_sync(FULL, ((gm >> lane) & 1u) && ambiguous(b.nodes[0][first + lane].slo.w, sc))
+                                        : 0u;
                 if (!WRAP && am) to_wrap = true;
                 if (!WRAP && to_wrap) return;
                 const unsigned amo = WRAP ? by_order(am, gm) : 0u;
-                stage_group<T, C::CH>(
-                    b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, int, const V &) {},
-                    [&](int j) { return pm[j]; },
-                    [&](V &q, int o) {
-                        if (WRAP && ((amo >> o) & 1u)) wrap_near<T>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
-                        return box_dist2<T>(q, flo, fhi) < Rq2;
+                stage_group<float, C::CH>(
+                    b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
+                    [&](int j) {
+                        float4 q = b.pmf[j];
+                        if (D64) q.w = __int_as_float(j);
+                        return q;
                     },
-                    [&](int slot, const V &q, int, int) { cand[slot] = q; }, flush);
+                    [&](float4 &q, int o) {
+                        if (D64 ? ph.periodic != 0 : WRAP && ((amo >> o) & 1u))
+                            wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
+                        return box_dist2<float>(q, flo, fhi) < Rq2;
+                    },
+                    [&](int slot, const float4 &q, int, int) {
+                        cand[slot] = q;
+                        if (D64) code[slot] = __float_as_int(q.w);
+                    },
+                    flush);
             });
         flush();
+        if (D64) drain();
         if (!WRAP && to_wrap) break;
-        if (LPP == 1 || !bal) {
+        if (D64) {
+        } else if (LPP == 1 || !bal) {
             cnt = at >> 5;
             ovf = cnt > C::LCAP;
             cnt = min(cnt, C::LCAP);
         }
-        if (LPP > 1 && bal) {
+        if (!D64 && LPP > 1 && bal) {
             const int mine_n = gcnt > sub ? (gcnt - sub - 1) / LPP + 1 : 0;
             cnt = mine_n < C::LCAP ? mine_n : C::LCAP;
         }
-        if (LPP > 1 && !bal && __any_sync(FULL, ovf)) {
+        if (!D64 && LPP > 1 && !bal && __any_sync(FULL, ovf)) {
             bal = true;  // same radius again, dealt by rank
             --attempt;
             continue;
         }
         if (group_any<LPP>(ovf) && active && !fail) fail = true;
+        if constexpr (D64)
+            if (attempt == 0 && maxit >= 16 && tol < T(1e-9)) presolve_f32<LPP, UM, K>(lr, lm, cnt, active && !fail, mi, mu_all, eta3, hs, h);
         // Newton-Raphson on the cached lists
         for (;;) {
             bool go = active && !conv && !fail && !need;
@@ -1051,13 +1210,13 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             if (go) {
                 const T hinv = T(1) / h;
                 for (int e = 0; e < cnt; ++e) {
-                    T q = sqrt(lr[e * 32 + lane]) * hinv;
+                    T q = (D64 ? lr[e * 32 + lane] : sqrt(lr[e * 32 + lane])) * hinv;
                     T mj = UM ? mu_all : lm[e * 32 + lane];
                     T f, df;
                     KF::fdf(q, f, df);
                     S0 += mj * f;
                     S1 += mj * q * df;
-                    nn += q < T(KF::R);
+                    nn += lt_pos(q, T(KF::R));
                 }
             }
             S0 = group_sum<LPP>(S0);
@@ -1125,13 +1284,13 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         if (redo) {
             const T hinv = T(1) / h;
             for (int e = 0; e < cnt; ++e) {
-                T q = sqrt(lr[e * 32 + lane]) * hinv;
+                T q = (D64 ? lr[e * 32 + lane] : sqrt(lr[e * 32 + lane])) * hinv;
                 T mj = UM ? mu_all : lm[e * 32 + lane];
                 T f, df;
                 KF::fdf(q, f, df);
                 R0 += mj * f;
                 R1 += mj * q * df;
-                rn += q < T(KF::R);
+                rn += lt_pos(q, T(KF::R));
             }
         }
         R0 = group_sum<LPP>(R0);
@@ -1149,7 +1308,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         if (fin) {
             const T hinv = T(1) / h;
             for (int e = 0; e < cnt; ++e)
-                Z += (UM ? mu_all : lm[e * 32 + lane]) * grav_psi_plus_mq(sqrt(lr[e * 32 + lane]) * hinv);
+                Z += (UM ? mu_all : lm[e * 32 + lane]) * grav_psi_plus_mq((D64 ? lr[e * 32 + lane] : sqrt(lr[e * 32 + lane])) * hinv);
         }
         Z = group_sum<LPP>(Z);
     }
@@ -1207,21 +1366,18 @@ __global__ void __launch_bounds__(DCfg<T, LPP, UM, K>::WPB * 32, DCfg<T, LPP, UM
     const bool tasks = WRAP && b.block_on && b.block_tasks;
     const int nleaf = tasks ? b.counters[kBlockTasks] : WRAP ? b.counters[kDensWrapList] : b.counters[0];
     const int cls = lpp_log2(LPP) + (UM ? 4 : 0) + 8 * K;
-    for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(&b.counters[(WRAP ? kDensityWrapCounter : kDensityCounter) + cls], 1);
-        item = __shfl_sync(FULL, item, 0);
+    for (int item = first_item();; item = next_item(&b.counters[(WRAP ? kDensityWrapCounter : kDensityCounter) + cls])) {
         if (item >= nleaf) break;
-        if (WRAP) item = tasks ? b.btask[item] : b.wrap_list[item];
-        const int leaf = tasks ? item >> 5 : item, k0 = tasks ? item & 31 : -1;
+        const int what = !WRAP ? item : tasks ? b.btask[item] : b.wrap_list[item];
+        const int leaf = tasks ? what >> 5 : what, k0 = tasks ? what & 31 : -1;
         const ProbStatic &ps = b.prob[b.leaf_pid[leaf]];
         if ((tasks ? b.block_lanes : ps.lpp) != LPP || (ps.uniform_m != 0) != UM || ps.ph.kernel != K) continue;
         if (!WRAP && ps.ph.gravity) {  // gravity's zeta runs in the wrap-list launch only
-            if (lane == 0) b.wrap_list[atomicAdd(&b.counters[kDensWrapList], 1)] = item;
+            if (lane == 0) b.wrap_list[atomicAdd(&b.counters[kDensWrapList], 1)] = leaf;
             continue;
         }
         if (!density_leaf<T, LPP, UM, K, WRAP>(b, leaf, k0, mine, use_pred) && lane == 0) {
-            b.wrap_list[atomicAdd(&b.counters[kDensWrapList], 1)] = item;
+            b.wrap_list[atomicAdd(&b.counters[kDensWrapList], 1)] = leaf;
             atomicAdd(&ps.diag->wrap_leaves, 1);
         }
     }
@@ -1430,17 +1586,19 @@ template <typename T, int LPP>
 struct FCfg {
     using V = typename Vec4<T>::type;
     static constexpr int CH = SPH_FORCE_CH;
+    static constexpr bool D64 = sizeof(T) == 8;
     // list entries per lane, and candidates tested per list-room check: at
     // one lane per particle a lane holds all of its particle's ~60 pairs
     static constexpr int LC = LPP == 1 ? SPH_FORCE_LC1 : SPH_FORCE_LC;
     static constexpr int SB = LPP == 1 ? SPH_FORCE_SB1 : SPH_FORCE_SB;
-    static constexpr int TAB = SPH_FORCE_TAB;  // candidate leaves per table fill (<= 2048)
-    static constexpr int WPB = 4;
-    static constexpr int MINB = LPP == 1 ? SPH_FORCE_MINB1 : SPH_FORCE_MINB;  // blocks per SM the registers allow
+    static constexpr int TAB = D64 ? 0 : SPH_FORCE_TAB;  // candidate leaves per table fill (<= 2048)
+    static constexpr int WPB = D64 ? 2 : 4;
+    static constexpr int MINB = D64 ? 4 : LPP == 1 ? SPH_FORCE_MINB1 : SPH_FORCE_MINB;  // blocks per SM the registers allow
+    using Code = std::conditional_t<D64, int, unsigned short>;  // (FP64: the sorted index itself)
     static_assert(TAB <= 2048 && LC >= 2 * SB / LPP, "force list layout");
-    static constexpr size_t scratch = (sizeof(StageScratch<T>) + 31) & ~(size_t)31;
-    static constexpr size_t codes = ((size_t)(CH + LC * 32) * 2 + 31) & ~(size_t)31;
-    static constexpr size_t per_warp = (CH + TAB) * sizeof(V) + scratch + codes;
+    static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
+    static constexpr size_t codes = ((size_t)(CH + LC * 32) * sizeof(Code) + 31) & ~(size_t)31;
+    static constexpr size_t per_warp = (CH + TAB) * sizeof(float4) + scratch + codes;
     static constexpr size_t smem = WPB * per_warp;
 };
 
@@ -1501,11 +1659,13 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     constexpr float KR_f = (float)KF::R;
     using V = typename C::V;
     const int lane = threadIdx.x & 31;
-    V *cand = reinterpret_cast<V *>(mine);  // staged (offset + leaf shift, 1/h)
-    V *table = cand + C::CH;                // per candidate leaf: (leaf shift, first sorted index)
-    StageScratch<T> &sc = *reinterpret_cast<StageScratch<T> *>(table + C::TAB);
-    unsigned short *code = reinterpret_cast<unsigned short *>(mine + (C::CH + C::TAB) * sizeof(V) + C::scratch);
-    unsigned short *lst = code + C::CH;
+    constexpr bool D64 = C::D64;
+    float4 *cand = reinterpret_cast<float4 *>(mine);  // staged (offset + leaf shift, 1/h; FP64: R_K h)
+    float4 *table = cand + C::CH;                     // per candidate leaf: (leaf shift, first sorted index)
+    StageScratch<float> &sc = *reinterpret_cast<StageScratch<float> *>(table + C::TAB);
+    using Code = typename C::Code;
+    Code *code = reinterpret_cast<Code *>(mine + (C::CH + C::TAB) * sizeof(float4) + C::scratch);
+    Code *lst = code + C::CH;
     const int pp = lane / LPP, sub = lane % LPP;
     const V *gph = (const V *)b.ph, *gvc = (const V *)b.vc, *gth = (const V *)b.th;
     const int p = b.leaf_pid[leaf];
@@ -1518,6 +1678,17 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     const bool active = task_member<T>(b, st, nA, k0, pp, pos);
     const int s = st + (active ? pos : 0);
     const V xi = gph[s], vi = gvc[s], ti = gth[s];
+    // the walk's copy of the particle, its membership data (FP64: R_K h and the
+    // bound of a staged coordinate's error) and its position
+    float4 xf;
+    if constexpr (D64) {
+        xf = b.pmf[s];
+        xf.w = __fmul_ru(KR_f, b.hf[s]);
+    } else {
+        xf = xi;
+    }
+    const float err = D64 ? 1e-6f * (ps.ph.periodic ? ps.ph.coord_max : b.dyn[p].coord_max) + 1e-30f : 0.f;
+    const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles, whose
     // largest h sets the gather reach
     if (k0 >= 0) task_box(b, leaf, xi, active, warp_max(active ? b.hf[s] : 0.f), boxA);
@@ -1561,48 +1732,67 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     T du = T(0), vs = T(-1);
     int pairs = 0, tested = 0;
     const float R = __fmul_ru(KR_f, boxA.plo.w) * 1.0001f;
-    const T RA2 = (T)R * (T)R;
-    V flo, fhi;
-    frame_box<V, T>(xi, active, flo, fhi);
+    const float RA2 = (R + 4.f * err) * (R + 4.f * err);
+    float4 flo, fhi;
+    frame_box<float4, float>(xf, active, flo, fhi);
     const float halfL = ph.periodic ? half_box(ph) : INFINITY;
     if (ph.periodic) {
         load_box(sc, ph, flo, fhi);
-        set_thr(sc, boxA.slo.w, Rall);
+        if (!D64) set_thr(sc, boxA.slo.w, Rall);
     }
-    const bool wrap2 = WRAP && half_width(flo, fhi) + Rall >= halfL;  // staged vectors may still need a wrap
+    const bool wrap2 = (WRAP || D64) && half_width(flo, fhi) + Rall >= halfL;  // staged vectors may still need a wrap
     bool to_wrap = false;  // (plain variant) met an ambiguous leaf pair: the wrapping variant takes the leaf
-    int nbuf = 0, cnt = 0, ntab = 0, tA = -1;
+    int nbuf = 0, cnt = 0, ntab = 0, tA = -1, gcnt = 0;  // gcnt (FP64): hits dealt to the particle's lanes
     unsigned am = 0u;
     // table entry of a candidate leaf: its shift and first sorted index,
     // stored as ~index for an ambiguous leaf pair (whose pair vectors the
     // evaluation wraps)
-    auto fetch = [&](int e, V &tb, V &a0, V &a1, V &a2, int &j) {
-        const unsigned cd = lst[e * 32 + lane];
-        tb = table[cd >> 5];
-        const int tv = t_as_bits(tb.w);
-        j = (WRAP && tv < 0 ? ~tv : tv) + (int)(cd & 31u);
-        a0 = ld_ro(gph + j);
+    auto fetch = [&](int e, T &rx, T &ry, T &rz, T &hinv_j, V &a1, V &a2, int &j) {
+        if constexpr (D64) {
+            // the minimum image of the FP64 positions' difference: odd, so
+            // particle j forms exactly -r_ij
+            j = lst[e * 32 + lane];
+            rx = min_image_bits(X[0] - b.sx[j], ph.box_len[0], ph.periodic);
+            ry = min_image_bits(X[1] - b.sy[j], ph.box_len[1], ph.periodic);
+            rz = min_image_bits(X[2] - b.sz[j], ph.box_len[2], ph.periodic);
+            hinv_j = gph[j].w;
+        } else {
+            const unsigned cd = lst[e * 32 + lane];
+            const float4 tb = table[cd >> 5];
+            const int tv = __float_as_int(tb.w);
+            j = (WRAP && tv < 0 ? ~tv : tv) + (int)(cd & 31u);
+            const V a0 = ld_ro(gph + j);
+            // r_ij = (o_i - o_j) - D_AB: IEEE subtraction is sign-symmetric and
+            // D_BA = -D_AB exactly, so particle j forms exactly -r_ij
+            rx = sub_rn(sub_rn(xi.x, a0.x), tb.x);
+            ry = sub_rn(sub_rn(xi.y, a0.y), tb.y);
+            rz = sub_rn(sub_rn(xi.z, a0.z), tb.z);
+            if (WRAP && tv < 0) wrap3s<float>(sc, rx, ry, rz);
+            hinv_j = a0.w;
+        }
         a1 = ld_ro(gvc + j);
         a2 = ld_ro(gth + j);
     };
     auto eval_lists = [&]() {
         __syncwarp();
+        if (D64) cnt = gcnt > sub ? (gcnt - sub - 1) / LPP + 1 : 0;
         for (int e = 0; e < cnt; ++e) {
-            V tb, a0, a1, a2;
+            V a1, a2;
+            T rx, ry, rz, hinv_j;
             int j;
-            fetch(e, tb, a0, a1, a2, j);
-            // r_ij = (o_i - o_j) - D_AB: IEEE subtraction is sign-symmetric and
-            // D_BA = -D_AB exactly, so particle j forms exactly -r_ij
-            T rx = sub_rn(sub_rn(xi.x, a0.x), tb.x), ry = sub_rn(sub_rn(xi.y, a0.y), tb.y),
-              rz = sub_rn(sub_rn(xi.z, a0.z), tb.z);
-            if (WRAP && t_as_bits(tb.w) < 0) wrap3s<T>(sc, rx, ry, rz);
+            fetch(e, rx, ry, rz, hinv_j, a1, a2, j);
             // every operation below up to m_i a_i with fixed rounding (odd
             // in r where it must be: particle j forms exactly the negatives)
             const T r2 = fma_rn(rz, rz, fma_rn(ry, ry, mul_rn(rx, rx)));
+            if constexpr (D64) {  // tested in FP32 with room to spare until here
+                const T hm = lt_pos(xi.w, hinv_j) ? xi.w : hinv_j;
+                if (!lt_pos(r2 * hm * hm, T(KF::R * KF::R))) continue;
+                ++pairs;
+            }
             const T rinv = rsqrt_t(r2);
             const T r = mul_rn(r2, rinv);
-            const T qi = mul_rn(r, xi.w), qj = mul_rn(r, a0.w);
-            const T hj2 = mul_rn(a0.w, a0.w);
+            const T qi = mul_rn(r, xi.w), qj = mul_rn(r, hinv_j);
+            const T hj2 = mul_rn(hinv_j, hinv_j);
             const T gi = mul_rn(mul_rn(sigma, KF::df(qi)), hi4);
             const T gj = mul_rn(mul_rn(sigma, KF::df(qj)), mul_rn(hj2, hj2));
             const T pterm = add_rn(mul_rn(Ai_g, gi), mul_rn(grav ? add_rn(a2.x, szg[j]) : a2.x, gj));
@@ -1644,15 +1834,15 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
             if (adi)
                 du += a2.z * (ti.x * vdr * gi +
                               rhob_inv * gbar * (T(-0.5) * al * vsig * mu * mu + aac * ac_speed(vdr, ti, a2, gm1_price, rhob_inv) * (ti.w - a2.w)));
-            vs = vsig > vs ? vsig : vs;
+            vs = lt_pos(vs, vsig) ? vsig : vs;
             if (blk) {
                 const T lj = slev[j], aj = fabs(lj);
                 mlev = aj > mlev ? aj : mlev;
                 if (due && lj < T(0) && aj < li1 - lgap) atomicMax(&b.breq[b.perm[j]], (int)(li1 - lgap) - 1);
             }
         }
-        pairs += cnt;
-        cnt = 0;
+        if (!D64) pairs += cnt;
+        cnt = gcnt = 0;
         __syncwarp();  // table and lists free for reuse
     };
     // membership: r_ij < R_K max(h_i, h_j), decided on the staged
@@ -1662,18 +1852,46 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         __syncwarp();  // staged candidates visible to every lane
         const int self = tA >= 0 ? ((tA << 5) | pos) : -1;
         for (int k0 = 0; k0 < nbuf; k0 += C::SB) {
-            if (__any_sync(FULL, cnt > C::LC - C::SB / LPP)) eval_lists();
             const int ke = k0 + C::SB < nbuf ? k0 + C::SB : nbuf;
+            if constexpr (D64) {
+                // FP32, with the coordinates' error to spare; the hits are dealt
+                // to the particle's lanes by rank
+                if (__any_sync(FULL, gcnt > C::LC * LPP - C::SB)) eval_lists();
+                const unsigned below = (1u << sub) - 1u;
+#pragma unroll 4
+                for (int kk = k0; kk < ke; kk += LPP) {
+                    const int k = kk + sub;
+                    bool hit = false;
+                    int j = 0;
+                    if (k < ke) {
+                        const float4 c = cand[k];
+                        float rx = xf.x - c.x, ry = xf.y - c.y, rz = xf.z - c.z;
+                        if (wrap2) wrap3s<float>(sc, rx, ry, rz);
+                        const float Rm = fmaxf(xf.w, c.w);
+                        j = code[k];
+                        hit = active && j != s &&
+                              rx * rx + ry * ry + rz * rz < Rm * (Rm * 1.00002f + 8.f * err) + err * err;
+                    }
+                    const unsigned gm = (__ballot_sync(FULL, hit) >> (pp * LPP)) & ((1u << LPP) - 1u);
+                    if (hit) {
+                        const int e = gcnt + __popc(gm & below);
+                        lst[(e / LPP) * 32 + pp * LPP + e % LPP] = j;
+                    }
+                    gcnt += __popc(gm);
+                }
+                continue;
+            }
+            if (__any_sync(FULL, cnt > C::LC - C::SB / LPP)) eval_lists();
 #pragma unroll 4
             for (int k = k0 + sub; k < ke; k += LPP) {
-                const V c = cand[k];
-                T rx = xi.x - c.x, ry = xi.y - c.y, rz = xi.z - c.z;
-                if (wrap2) wrap3s<T>(sc, rx, ry, rz);
-                T r2 = rx * rx + ry * ry + rz * rz;
-                T hm = xi.w < c.w ? xi.w : c.w;
+                const float4 c = cand[k];
+                float rx = xf.x - c.x, ry = xf.y - c.y, rz = xf.z - c.z;
+                if (wrap2) wrap3s<float>(sc, rx, ry, rz);
+                const float r2 = rx * rx + ry * ry + rz * rz;
+                const float hm = xf.w < c.w ? xf.w : c.w;
                 const int cd = code[k];
-                if (active && cd != self && r2 * hm * hm < T(KF::R * KF::R))
-                    lst[cnt++ * 32 + lane] = (unsigned short)cd;
+                if (active && cd != self && r2 * hm * hm < (float)(KF::R * KF::R))
+                    lst[cnt++ * 32 + lane] = (Code)cd;
             }
         }
         tested += (nbuf - sub + LPP - 1) / LPP;
@@ -1686,38 +1904,56 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         return box_overlap(sc.qb, nb, ph) || near;
     };
     auto visit = [&](unsigned mask, int first) {
-            if (ntab + __popc(mask) > C::TAB) {
+            int jq = 0;  // (FP64) the staged particle's sorted index
+            if (!D64 && ntab + __popc(mask) > C::TAB) {
                 test();
                 eval_lists();
                 ntab = 0;
                 tA = -1;
             }
             // candidate leaves that form an ambiguous pair with A (periodic)
-            am = ph.periodic ? __ballot_sync(FULL, ((mask >> lane) & 1u) && ambiguous(b.nodes[0][first + lane].slo.w, sc))
-                             : 0u;
+            // (FP64: see the density pass)
+            am = !D64 && ph.periodic ? __ballot_sync(FULL, ((mask >> lane) & 1u) && ambiguous(b.nodes[0][first + lane].slo.w, sc))
+                                     : 0u;
             if (!WRAP && am) to_wrap = true;
             if (!WRAP && to_wrap) return;
             const unsigned amo = WRAP ? by_order(am, mask) : 0u;
-            stage_group<T, C::CH>(
+            stage_group<float, C::CH>(
                 b, leaf, mask, first, ph, nbuf, sc,
-                [&](bool has, int B, int stB, int ord, const V &D) {
+                [&](bool has, int B, int stB, int ord, const float4 &D) {
+                    if (D64) return;
                     if (has) {
-                        V t = D;
-                        t.w = bits_as_t((am >> lane) & 1u ? ~stB : stB, T(0));
+                        float4 t = D;
+                        t.w = __int_as_float((am >> lane) & 1u ? ~stB : stB);
                         table[ntab + ord] = t;
                     }
                     const unsigned ka = (unsigned)(leaf - first);  // the query leaf itself in this group
                     if (ka < 32u && ((mask >> ka) & 1u)) tA = ntab + __popc(mask & ((1u << ka) - 1u));
                 },
-                [&](int j) { return gph[j]; },
-                [&](V &q, int o) {
-                    if (WRAP && ((amo >> o) & 1u)) wrap_near<T>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
-                    const T d2 = box_dist2<T>(q, flo, fhi);
-                    return d2 < RA2 || d2 * q.w * q.w < T(KF::R * KF::R * 1.0001);
+                [&](int j) {
+                    if constexpr (D64) {
+                        float4 q = b.pmf[j];
+                        q.w = __int_as_float(j);
+                        return q;
+                    } else {
+                        return gph[j];
+                    }
                 },
-                [&](int slot, const V &q, int o, int idx) {
+                [&](float4 &q, int o) {
+                    if (D64 ? ph.periodic != 0 : WRAP && ((amo >> o) & 1u))
+                        wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
+                    const float d2 = box_dist2<float>(q, flo, fhi);
+                    if constexpr (D64) {
+                        jq = __float_as_int(q.w);
+                        q.w = __fmul_ru(KR_f, b.hf[jq]);
+                        const float Rj = q.w * 1.0001f + 4.f * err;
+                        return d2 < RA2 || d2 < Rj * Rj;
+                    }
+                    return d2 < RA2 || d2 * q.w * q.w < (float)(KF::R * KF::R * 1.0001);
+                },
+                [&](int slot, const float4 &q, int o, int idx) {
                     cand[slot] = q;
-                    code[slot] = (unsigned short)(((ntab + o) << 5) | idx);
+                    code[slot] = (Code)(D64 ? jq : (((ntab + o) << 5) | idx));
                 },
                 test);
             ntab += __popc(mask);
@@ -1837,13 +2073,11 @@ __global__ void __launch_bounds__(FCfg<T, LPP>::WPB * 32, FCfg<T, LPP>::MINB) k_
     const int cls = lpp_log2(LPP) + 4 * K;
     int last_p = -1;
     float Rall = 0.f;  // periodic: pairs reach R_K x the problem's largest h
-    for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(&b.counters[(CD ? kForceCdCounter : WRAP ? kForceWrapCounter : kForceCounter) + cls], 1);
-        item = __shfl_sync(FULL, item, 0);
+    for (int item = first_item();;
+         item = next_item(&b.counters[(CD ? kForceCdCounter : WRAP ? kForceWrapCounter : kForceCounter) + cls])) {
         if (item >= nleaf) break;
-        if (WRAP) item = tasks ? b.btask[item] : b.wrap_list[item];
-        const int leaf = tasks ? item >> 5 : item, k0 = tasks ? item & 31 : -1;
+        const int what = !WRAP ? item : tasks ? b.btask[item] : b.wrap_list[item];
+        const int leaf = tasks ? what >> 5 : what, k0 = tasks ? what & 31 : -1;
         const int p = b.leaf_pid[leaf];
         const ProbStatic &ps = b.prob[p];
         if ((tasks ? b.block_lanes : ps.lpp) != LPP || ps.ph.kernel != K) continue;  // served by another launch
