@@ -50,7 +50,7 @@ struct ExportCfg {
     static constexpr size_t per_warp = CH * (sizeof(float4) + sizeof(int)) + (size_t)LC * 32 * sizeof(int) + scratch;
 };
 template <bool FILL>
-__global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int kind, unsigned *cnt,
+__global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, int kind, unsigned *cnt,
                                                                 const long long *offsets, int *idx, long long cap)
 {
     using C = ExportCfg;
@@ -129,10 +129,18 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int
         auto node = [&](const NodeBox &nb) {
             return up_within(sc.qb, nb) || (kind == 1 && up_overlap(sc.qb, nb));
         };
-        walk(b, d, node, node, [&](unsigned mask, int first) {
-            int j = 0;
-            float Rj = 0.f;
-            stage_group<float, C::CH>(
+        int j = 0;
+        float Rj = 0.f;
+        Walk wk;
+        wk.start(d);
+        for (;;) {
+            const int nd = wk.next(b, d, node);
+            if (nd < 0) break;
+            const int first = d.node_off[0] + nd * kBranch;
+            const bool in = (leaf_lanes(d.node_cnt[0], nd) >> lane) & 1u;
+            const unsigned mask = __ballot_sync(FULL, node(b.nodes[0][first + (in ? lane : 0)]) && in);
+            if (mask)
+                stage_group<float, C::CH>(
                 b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
                 [&](int jj) {
                     float4 q = b.pmf[jj];
@@ -151,7 +159,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32) k_export(BatchView b, int
                     code[slot] = j;
                 },
                 test);
-        });
+        }
         test();
         drain();
         if (!FILL) {

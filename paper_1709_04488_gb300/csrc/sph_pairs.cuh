@@ -351,59 +351,59 @@ __device__ __forceinline__ bool box_overlap(const QueryBox &qb, const NodeBox &n
     return ok;
 }
 
-// Warp-cooperative depth-first walk of one problem's tree.  At the leaf level
-// visit(mask, first) is called (warp-uniformly) with the ballot of the up to
-// 32 sibling leaves first..first+31 whose boxes pass test(box), so that a
-// whole group of candidate leaves is staged in one round of memory accesses;
-// the nodes above them are opened where up(box) passes.
-// The nodes still to open of each level above the current one are kept in
-// the lanes (lane l: level l's), not in an array a run-time level indexes.
-template <class Up, class Test, class Visit>
-__device__ __forceinline__ void walk(const BatchView &b, const ProbDyn &d, Up &&up, Test &&test, Visit &&visit)
-{
-    const int lane = threadIdx.x & 31;
-    const int top = d.top_level;
-    const int off0 = d.node_off[0], cnt0 = d.node_cnt[0];
-    const NodeBox *leaves = b.nodes[0] + off0;
-    bool ok = false;
-    if (top == 0) {
-        ok = test(leaves[lane < cnt0 ? lane : 0]) && lane < cnt0;
-        const unsigned lm = __ballot_sync(FULL, ok);
-        if (lm) visit(lm, off0);
-        return;
+// Warp-cooperative depth-first walk of one problem's tree, one step at a time:
+// next() returns the next level-1 node (up to 32 sibling leaves, in order) that
+// lies under nodes whose boxes pass up(box), or -1.  The caller tests its
+// leaves, one per lane, and stages the ones that pass in one round of memory
+// accesses.  (A step function, so that the caller's staging has one call site:
+// each inlined one is a copy, and the instruction cache was the second
+// largest stall of the wrap-list force launch.)  The nodes still to open of
+// each level are kept in the lanes (lane l: level l's), not in an array a
+// run-time level indexes.
+struct Walk {
+    unsigned m, sm;
+    int base, sb, lvl, top;
+    __device__ __forceinline__ void start(const ProbDyn &d)
+    {
+        top = lvl = d.top_level + 1;  // (one node above the top level holds it; top level 0: the leaves' only node)
+        m = 1u;
+        sm = 0u;
+        base = sb = 0;
     }
-    if (lane < d.node_cnt[top]) ok = up(b.nodes[top][d.node_off[top] + lane]);
-    unsigned m = __ballot_sync(FULL, ok);
-    unsigned sm = 0u;
-    int sb = 0, lvl = top, base = 0;
-    for (;;) {
-        while (m == 0u) {
-            if (lvl == top) return;
-            ++lvl;
-            m = __shfl_sync(FULL, sm, lvl);
-            base = __shfl_sync(FULL, sb, lvl);
-        }
-        const int node = base + __ffs(m) - 1;
-        m &= m - 1u;
-        const int ch = node * kBranch + lane;
-        ok = false;
-        if (lvl == 1) {  // (every lane tests a leaf of the node: test votes)
-            ok = test(leaves[ch < cnt0 ? ch : node * kBranch]) && ch < cnt0;
+    template <class Up>
+    __device__ __forceinline__ int next(const BatchView &b, const ProbDyn &d, Up &&up)
+    {
+        const int lane = threadIdx.x & 31;
+        for (;;) {
+            while (m == 0u) {
+                if (lvl == top) return -1;
+                ++lvl;
+                m = __shfl_sync(FULL, sm, lvl);
+                base = __shfl_sync(FULL, sb, lvl);
+            }
+            const int node = base + __ffs(m) - 1;
+            m &= m - 1u;
+            if (lvl == 1) return node;
+            const int ch = node * kBranch + lane;
+            bool ok = false;
+            if (ch < d.node_cnt[lvl - 1]) ok = up(b.nodes[lvl - 1][d.node_off[lvl - 1] + ch]);
             const unsigned cm = __ballot_sync(FULL, ok);
-            if (cm) visit(cm, off0 + node * kBranch);
-            continue;
+            if (cm == 0u) continue;
+            if (lane == lvl) {
+                sm = m;
+                sb = base;
+            }
+            --lvl;
+            m = cm;
+            base = node * kBranch;
         }
-        if (ch < d.node_cnt[lvl - 1]) ok = up(b.nodes[lvl - 1][d.node_off[lvl - 1] + ch]);
-        const unsigned cm = __ballot_sync(FULL, ok);
-        if (cm == 0u) continue;
-        if (lane == lvl) {
-            sm = m;
-            sb = base;
-        }
-        --lvl;
-        m = cm;
-        base = node * kBranch;
     }
+};
+// lanes of a level-1 node that hold a leaf
+__device__ __forceinline__ unsigned leaf_lanes(int cnt0, int node)
+{
+    const int n = cnt0 - node * kBranch;
+    return n >= 32 ? FULL : (1u << n) - 1u;
 }
 
 template <typename T>
@@ -1135,51 +1135,54 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         // spheres reach this leaf (what the force pass will need); stage
         // only the former
         bool near = false;  // this lane's last tested node is within Rq
-        walk(
-            b, dy,
-            [&](const NodeBox &nb) {
+        Walk wk;
+        wk.start(dy);
+        for (;;) {
+            const int node = wk.next(b, dy, [&](const NodeBox &nb) {
                 return up_within(sc.qb, nb) || (record && up_overlap(sc.qb, nb));
-            },
-            [&](const NodeBox &nb) {
-                near = box_within(sc.qb, nb, ph);
-                return record ? box_overlap(sc.qb, nb, ph) || near : near;
-            },
-            [&](unsigned mask, int first) {
-                if (lane == ng) {
-                    g_first = first;
-                    g_mask = mask;
-                }
-                ++ng;
-                // the leaf-level tests just made: stage the leaves within Rq
-                const unsigned gm = __ballot_sync(FULL, near && ((mask >> lane) & 1u));
-                if (gm == 0u) return;
-                // candidate leaves that form an ambiguous pair with A (periodic)
-                // (FP64 takes its pairs' minimum images from the positions: every
-                // staged candidate moves to its image nearest the query box)
-                const unsigned am =
-                    !D64 && ph.periodic ? __ballot_sync(FULL, ((gm >> lane) & 1u) && ambiguous(b.nodes[0][first + lane].slo.w, sc))
-                                        : 0u;
-                if (!WRAP && am) to_wrap = true;
-                if (!WRAP && to_wrap) return;
-                const unsigned amo = WRAP ? by_order(am, gm) : 0u;
-                stage_group<float, C::CH>(
-                    b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
-                    [&](int j) {
-                        float4 q = b.pmf[j];
-                        if (D64) q.w = __int_as_float(j);
-                        return q;
-                    },
-                    [&](float4 &q, int o) {
-                        if (D64 ? ph.periodic != 0 : WRAP && ((amo >> o) & 1u))
-                            wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
-                        return box_dist2<float>(q, flo, fhi) < Rq2;
-                    },
-                    [&](int slot, const float4 &q, int, int) {
-                        cand[slot] = q;
-                        if (D64) code[slot] = __float_as_int(q.w);
-                    },
-                    flush);
             });
+            if (node < 0) break;
+            const int first = dy.node_off[0] + node * kBranch;
+            const bool in = (leaf_lanes(dy.node_cnt[0], node) >> lane) & 1u;
+            const NodeBox &nb = b.nodes[0][first + (in ? lane : 0)];
+            near = box_within(sc.qb, nb, ph);
+            const unsigned mask = __ballot_sync(FULL, (record ? box_overlap(sc.qb, nb, ph) || near : near) && in);
+            if (mask == 0u) continue;
+            if (lane == ng) {
+                g_first = first;
+                g_mask = mask;
+            }
+            ++ng;
+            // the leaf-level tests just made: stage the leaves within Rq
+            const unsigned gm = __ballot_sync(FULL, near && ((mask >> lane) & 1u));
+            if (gm == 0u) continue;
+            // candidate leaves that form an ambiguous pair with A (periodic)
+            // (FP64 takes its pairs' minimum images from the positions: every
+            // staged candidate moves to its image nearest the query box)
+            const unsigned am =
+                !D64 && ph.periodic ? __ballot_sync(FULL, ((gm >> lane) & 1u) && ambiguous(b.nodes[0][first + lane].slo.w, sc))
+                                    : 0u;
+            if (!WRAP && am) to_wrap = true;
+            if (!WRAP && to_wrap) break;
+            const unsigned amo = WRAP ? by_order(am, gm) : 0u;
+            stage_group<float, C::CH>(
+                b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
+                [&](int j) {
+                    float4 q = b.pmf[j];
+                    if (D64) q.w = __int_as_float(j);
+                    return q;
+                },
+                [&](float4 &q, int o) {
+                    if (D64 ? ph.periodic != 0 : WRAP && ((amo >> o) & 1u))
+                        wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
+                    return box_dist2<float>(q, flo, fhi) < Rq2;
+                },
+                [&](int slot, const float4 &q, int, int) {
+                    cand[slot] = q;
+                    if (D64) code[slot] = __float_as_int(q.w);
+                },
+                flush);
+        }
         flush();
         if (D64) drain();
         if (!WRAP && to_wrap) break;
@@ -1457,10 +1460,15 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
                 __syncwarp();
                 nbuf = 0;
             };
-            walk(
-                b, dy, [&](const NodeBox &nb) { return up_within(sc.qb, nb); },
-                [&](const NodeBox &nb) { return box_within(sc.qb, nb, ph); },
-                [&](unsigned mask, int first) {
+            Walk wk;
+            wk.start(dy);
+            for (;;) {
+                const int node = wk.next(b, dy, [&](const NodeBox &nb) { return up_within(sc.qb, nb); });
+                if (node < 0) break;
+                const int first = dy.node_off[0] + node * kBranch;
+                const bool in = (leaf_lanes(dy.node_cnt[0], node) >> lane) & 1u;
+                const unsigned mask = __ballot_sync(FULL, box_within(sc.qb, b.nodes[0][first + (in ? lane : 0)], ph) && in);
+                if (mask)
                     stage_group<T, kFbCH>(
                         b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const V &) {},
                         [&](int j) { return pm[j]; },
@@ -1469,7 +1477,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
                             return box_dist2<T>(q, pi, pi) < Rq2;
                         },
                         [&](int slot, const V &q, int, int) { cand[slot] = q; }, flush);
-                });
+            }
             flush();
         };
         bool direct = false;
@@ -1959,23 +1967,52 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
             ntab += __popc(mask);
     };
     // the candidate groups the density walk recorded cover every pair
-    // unless some final h outgrew them (then walk the tree again)
-    const int ngl = k0 < 0 ? b.leaf_ngroups[leaf] : -1;
-    if (!dy.lists_stale && ngl >= 0) {
-        const int gofs = b.leaf_gofs[leaf];
-        for (int g = 0; g < ngl; ++g) {
-            const int2 e = b.group_pool[gofs + g];
-            const unsigned mask = (unsigned)e.y;
-            const bool in = (mask >> lane) & 1u;
-            const bool ok = node_test(b.nodes[0][e.x + (in ? lane : __ffs(mask) - 1)]);
-            const unsigned fm = __ballot_sync(FULL, ok && in);
-            if (fm) visit(fm, e.x);
+    // unless some final h outgrew them (then walk the tree again).  One lane
+    // per particle: a loop of its own for either way, so that the walk's state
+    // takes no registers beside the recorded groups' (in one loop k_forces
+    // was 11 % slower at 1e6 particles); else one loop, so that the staging and
+    // the evaluation are there once, with lane g holding group g (at most 32
+    // are recorded)
+    const int ngl = k0 < 0 && !dy.lists_stale ? b.leaf_ngroups[leaf] : -1;
+    auto offer = [&](int first, unsigned in) {
+        const bool mine_in = (in >> lane) & 1u;
+        const bool ok = node_test(b.nodes[0][first + (mine_in ? lane : __ffs(in) - 1)]);
+        const unsigned fm = __ballot_sync(FULL, ok && mine_in);
+        if (fm) visit(fm, first);
+    };
+    auto next_node = [&](Walk &wk) {
+        return wk.next(b, dy, [&](const NodeBox &nb) { return up_within(sc.qb, nb) || up_overlap(sc.qb, nb); });
+    };
+    if constexpr ((LPP == 1 && !WRAP) || CD) {
+        if (ngl >= 0) {
+            const int2 *rec = b.group_pool + b.leaf_gofs[leaf];
+            for (int g = 0; g < ngl && !to_wrap; ++g) offer(rec[g].x, (unsigned)rec[g].y);
+        } else {
+            Walk wk;
+            wk.start(dy);
+            for (int node; !to_wrap && (node = next_node(wk)) >= 0;)
+                offer(dy.node_off[0] + node * kBranch, leaf_lanes(dy.node_cnt[0], node));
         }
     } else {
-        walk(
-            b, dy,
-            [&](const NodeBox &nb) { return up_within(sc.qb, nb) || up_overlap(sc.qb, nb); },
-            node_test, visit);
+        int2 rec = make_int2(0, 0);
+        if (lane < ngl) rec = b.group_pool[b.leaf_gofs[leaf] + lane];
+        Walk wk;
+        wk.start(dy);
+        for (int g = 0; !to_wrap; ++g) {
+            int first;
+            unsigned in;
+            if (ngl >= 0) {
+                if (g >= ngl) break;
+                first = __shfl_sync(FULL, rec.x, g);
+                in = (unsigned)__shfl_sync(FULL, rec.y, g);
+            } else {
+                const int node = next_node(wk);
+                if (node < 0) break;
+                first = dy.node_off[0] + node * kBranch;
+                in = leaf_lanes(dy.node_cnt[0], node);
+            }
+            offer(first, in);
+        }
     }
     test();
     eval_lists();

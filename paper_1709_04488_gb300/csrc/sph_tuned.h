@@ -15,7 +15,7 @@
 #define SPH_DENS_MINB 4
 #endif
 #ifndef SPH_DENS_MINB1
-#define SPH_DENS_MINB1 5
+#define SPH_DENS_MINB1 4
 #endif
 #ifndef SPH_DENS_LCAP1
 #define SPH_DENS_LCAP1 96
