@@ -29,6 +29,7 @@ constexpr long long kTileSpinLimit = 1ll << 24;
 
 __global__ void k_gather(BatchView b)
 {
+    chain_entry();
     long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= b.ntot) return;
     int p = (int)(b.keys[0][s] >> kMortonTotal);
@@ -167,6 +168,7 @@ __device__ void problem_meta(const BatchView &b)
 // and clears the tile state for the next build.
 __global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b)
 {
+    chain_entry();
     __shared__ unsigned long long sk[kLeafTile + 2 * kHalo];
     __shared__ int wsum[kLeafThreads / 32];
     __shared__ unsigned s_tile, s_prefix;
@@ -266,6 +268,7 @@ __global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b)
 template <typename T4, bool WRAP>
 __global__ void k_leaf_props(BatchView b)
 {
+    chain_entry();
     const int nleaf = b.counters[0];
     if (blockIdx.x == 0)
         for (int p = threadIdx.x; p < b.nprob; p += blockDim.x) b.dyn[p].lists_stale = 0;
@@ -280,6 +283,7 @@ __global__ void k_leaf_props(BatchView b)
 template <typename T4>
 __global__ void k_leaf_refit(BatchView b)
 {
+    chain_entry();
     // a block-step tick with tasks: unless some particle's final h outgrew
     // the prediction the leaf pass boxed it with (lists_stale), those boxes
     // already hold every smoothing sphere (the kept particles' h unchanged)
@@ -360,7 +364,7 @@ int levels_needed(long long max_leaves)
 cudaError_t launch_gather(const BatchView &b, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
-    k_gather<<<(unsigned)((b.ntot + 255) / 256), 256, 0, st>>>(b);
+    launch_chain(SPH_DEP(b), k_gather, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b);
     return cudaGetLastError();
 }
 
@@ -368,10 +372,10 @@ cudaError_t launch_build_leaves(const BatchView &b, int precision, cudaStream_t 
 {
     if (b.ntot == 0) return cudaSuccess;
     const long long tiles = (b.ntot + kLeafTile - 1) / kLeafTile;
-    k_leaf_scan<<<(unsigned)tiles, kLeafThreads, 0, st>>>(b);
+    launch_chain(SPH_DEP(b), k_leaf_scan, (unsigned)tiles, kLeafThreads, 0, st, b);
     int pb = persistent_blocks(256);
-    if (precision == SPH_PREC_FP64) k_leaf_props<dbl4, false><<<pb, 256, 0, st>>>(b);
-    else k_leaf_props<float4, false><<<pb, 256, 0, st>>>(b);
+    if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_leaf_props<dbl4, false>, pb, 256, 0, st, b);
+    else launch_chain(SPH_DEP(b), k_leaf_props<float4, false>, pb, 256, 0, st, b);
     return cudaGetLastError();
 }
 
@@ -383,8 +387,8 @@ cudaError_t launch_update_leaves(const BatchView &b, int precision, cudaStream_t
 {
     if (b.ntot == 0) return cudaSuccess;
     int pb = persistent_blocks(256);
-    if (precision == SPH_PREC_FP64) k_leaf_props<dbl4, true><<<pb, 256, 0, st>>>(b);
-    else k_leaf_props<float4, true><<<pb, 256, 0, st>>>(b);
+    if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_leaf_props<dbl4, true>, pb, 256, 0, st, b);
+    else launch_chain(SPH_DEP(b), k_leaf_props<float4, true>, pb, 256, 0, st, b);
     return cudaGetLastError();
 }
 
@@ -392,8 +396,8 @@ cudaError_t launch_refit(const BatchView &b, int precision, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
     int pb = persistent_blocks(256);
-    if (precision == SPH_PREC_FP64) k_leaf_refit<dbl4><<<pb, 256, 0, st>>>(b);
-    else k_leaf_refit<float4><<<pb, 256, 0, st>>>(b);
+    if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_leaf_refit<dbl4>, pb, 256, 0, st, b);
+    else launch_chain(SPH_DEP(b), k_leaf_refit<float4>, pb, 256, 0, st, b);
     return cudaGetLastError();
 }
 

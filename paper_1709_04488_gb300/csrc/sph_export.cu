@@ -14,6 +14,7 @@ constexpr int kExportCap = 1024;  // neighbours one particle may have in the exp
 
 __global__ void k_set_sorted_h(BatchView b, const double *h_in)
 {
+    chain_entry();
     long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= b.ntot) return;
     int p = (int)(b.keys[0][s] >> kMortonTotal);
@@ -53,6 +54,7 @@ template <bool FILL>
 __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, int kind, unsigned *cnt,
                                                                 const long long *offsets, int *idx, long long cap)
 {
+    chain_entry();
     using C = ExportCfg;
     __shared__ __align__(32) unsigned char smem[C::WPB * C::per_warp];
     __shared__ int wrote[C::WPB][32];
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
 // cap is left to k_export_cut.
 __global__ void __launch_bounds__(128) k_export_sort(BatchView b, const long long *offsets, int *idx, long long cap)
 {
+    chain_entry();
     __shared__ int buf[4][kExportCap];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -203,6 +206,7 @@ __global__ void __launch_bounds__(128) k_export_sort(BatchView b, const long lon
 // are gathered again from all particles and those below cap written in order.
 __global__ void __launch_bounds__(1024) k_export_cut(BatchView b, int kind, const long long *offsets, int *idx, long long cap)
 {
+    chain_entry();
     __shared__ int buf[kExportCap];
     __shared__ int s_pos, s_n;
     if (offsets[b.ntot] <= cap) return;
@@ -255,6 +259,7 @@ __device__ __forceinline__ long long block_sum(long long v, long long *red)
 }
 __global__ void __launch_bounds__(kScanThreads) k_count_sums(const unsigned *cnt, long long n, long long *part)
 {
+    chain_entry();
     __shared__ long long red[kScanThreads / 32];
     const long long per = scan_share(n), lo = blockIdx.x * per, hi = lo + per < n ? lo + per : n;
     long long s = 0;
@@ -265,6 +270,7 @@ __global__ void __launch_bounds__(kScanThreads) k_count_sums(const unsigned *cnt
 __global__ void __launch_bounds__(kScanThreads) k_offsets(const unsigned *cnt, long long n, const long long *part,
                                                           long long *offsets, long long *total)
 {
+    chain_entry();
     __shared__ long long red[kScanThreads / 32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long per = scan_share(n), lo = blockIdx.x * per, hi = lo + per < n ? lo + per : n;
@@ -294,7 +300,7 @@ __global__ void __launch_bounds__(kScanThreads) k_offsets(const unsigned *cnt, l
 cudaError_t launch_set_sorted_h(const BatchView &b, const double *h_in, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
-    k_set_sorted_h<<<(unsigned)((b.ntot + 255) / 256), 256, 0, st>>>(b, h_in);
+    launch_chain(SPH_DEP(b), k_set_sorted_h, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b, h_in);
     return cudaGetLastError();
 }
 
@@ -312,12 +318,12 @@ cudaError_t launch_neighbour_export(const BatchView &b, int kind, long long *off
     const long long n = b.ntot, share = (n + kScanBlocks - 1) / kScanBlocks;
     const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
                          ((share + kScanThreads - 1) / kScanThreads * kScanThreads));
-    k_export<false><<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
-    k_count_sums<<<nb, kScanThreads, 0, st>>>(cnt, n, part);
-    k_offsets<<<nb, kScanThreads, 0, st>>>(cnt, n, part, offsets, total_dev);
-    k_export<true><<<grid, ExportCfg::WPB * 32, 0, st>>>(b, kind, cnt, offsets, idx, cap);
-    k_export_sort<<<grid, 128, 0, st>>>(b, offsets, idx, cap);
-    k_export_cut<<<1, 1024, 0, st>>>(b, kind, offsets, idx, cap);
+    launch_chain(SPH_DEP(b), k_export<false>, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
+    launch_chain(SPH_DEP(b), k_count_sums, nb, kScanThreads, 0, st, cnt, n, part);
+    launch_chain(SPH_DEP(b), k_offsets, nb, kScanThreads, 0, st, cnt, n, part, offsets, total_dev);
+    launch_chain(SPH_DEP(b), k_export<true>, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
+    launch_chain(SPH_DEP(b), k_export_sort, grid, 128, 0, st, b, offsets, idx, cap);
+    launch_chain(SPH_DEP(b), k_export_cut, 1, 1024, 0, st, b, kind, offsets, idx, cap);
     return cudaGetLastError();
 }
 

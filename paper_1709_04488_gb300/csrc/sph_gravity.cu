@@ -205,6 +205,7 @@ struct GravTwo<float> {
 template <typename T>
 __global__ void __launch_bounds__(kGravThreads, sizeof(T) == 4 ? kGravBlocksPerSM : 1) k_gravity(BatchView b)
 {
+    chain_entry();
     using P = typename GravVec<T>::P;
     using H = typename GravVec<T>::H;
     __shared__ P tp[2 * kGravThreads];
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(kGravThreads, sizeof(T) == 4 ? kGravBlocksPerS
 template <typename T>
 __global__ void __launch_bounds__(256) k_gravity_reduce(BatchView b)
 {
+    chain_entry();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= b.ntot) return;
     if (b.block_on && ((const T *)b.slev)[i] < T(0)) return;  // block step: not this particle's force pass
@@ -447,6 +449,7 @@ __device__ void form_groups(double M, const double (&x)[3], const double (&q)[6]
 template <typename T>
 __global__ void __launch_bounds__(256) k_grav_moments(BatchView b)
 {
+    chain_entry();
     using V4 = typename Vec4<T>::type;
     const int lane = threadIdx.x & 31;
     const int nleaf = b.counters[0];
@@ -565,6 +568,7 @@ __device__ __forceinline__ void multipole_acc(T rx, T ry, T rz, T M, const T (&Q
 template <typename T>
 __global__ void __launch_bounds__(kTreeThreads) k_gravity_tree(BatchView b)
 {
+    chain_entry();
     using V4 = typename Vec4<T>::type;
     using P = typename GravVec<T>::P;
     using H = typename GravVec<T>::H;
@@ -783,6 +787,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_gravity_tree(BatchView b)
 // joins the CFL minimum of the force pass.
 __global__ void __launch_bounds__(256) k_grav_dt(BatchView b)
 {
+    chain_entry();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int p = -1;
     double dt = INFINITY;
@@ -837,25 +842,25 @@ void launch_gravity(const BatchView &b, int precision, cudaStream_t st)
 {
     if (!b.any_gravity) return;
     if (b.grav_blocks > 0) {
-        if (precision == SPH_PREC_FP64) k_gravity<double><<<(unsigned)b.grav_blocks, kGravThreads, 0, st>>>(b);
-        else k_gravity<float><<<(unsigned)b.grav_blocks, kGravThreads, 0, st>>>(b);
+        if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_gravity<double>, (unsigned)b.grav_blocks, kGravThreads, 0, st, b);
+        else launch_chain(SPH_DEP(b), k_gravity<float>, (unsigned)b.grav_blocks, kGravThreads, 0, st, b);
     }
     if (b.grav_split) {
-        if (precision == SPH_PREC_FP64) k_gravity_reduce<double><<<(unsigned)((b.ntot + 255) / 256), 256, 0, st>>>(b);
-        else k_gravity_reduce<float><<<(unsigned)((b.ntot + 255) / 256), 256, 0, st>>>(b);
+        if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_gravity_reduce<double>, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b);
+        else launch_chain(SPH_DEP(b), k_gravity_reduce<float>, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b);
     }
     if (b.any_grav_tree) {
         static int sms = 0;
         if (!sms) sms = dev_info().sm_count;
         if (precision == SPH_PREC_FP64) {
-            k_grav_moments<double><<<sms * 8, 256, 0, st>>>(b);
-            k_gravity_tree<double><<<sms * 8, kTreeThreads, 0, st>>>(b);
+            launch_chain(SPH_DEP(b), k_grav_moments<double>, sms * 8, 256, 0, st, b);
+            launch_chain(SPH_DEP(b), k_gravity_tree<double>, sms * 8, kTreeThreads, 0, st, b);
         } else {
-            k_grav_moments<float><<<sms * 8, 256, 0, st>>>(b);
-            k_gravity_tree<float><<<sms * 8, kTreeThreads, 0, st>>>(b);
+            launch_chain(SPH_DEP(b), k_grav_moments<float>, sms * 8, 256, 0, st, b);
+            launch_chain(SPH_DEP(b), k_gravity_tree<float>, sms * 8, kTreeThreads, 0, st, b);
         }
     }
-    if (b.ntot > 0) k_grav_dt<<<(unsigned)((b.ntot + 255) / 256), 256, 0, st>>>(b);
+    if (b.ntot > 0) launch_chain(SPH_DEP(b), k_grav_dt, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b);
 }
 
 }  // namespace sph

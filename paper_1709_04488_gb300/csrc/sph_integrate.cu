@@ -18,6 +18,7 @@ constexpr int kCloseItems = 8;  // most particles per thread in the closing kern
 
 __global__ void k_reset_step(BatchView b, int mode)
 {
+    chain_entry();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     reset_counters(b, mode);
     if (p < b.nprob) reset_diag(b, p, mode);
@@ -33,6 +34,7 @@ __device__ __forceinline__ double step_dt(const ProbDiag *d, double dt_host)
 // 0 also selects each problem's step and resets its diagnostics.
 __global__ void k_kick_drift(BatchView b, double dt_host)
 {
+    chain_entry();
     reset_counters(b, 1);
     if (blockIdx.x == 0) {
         for (int p = threadIdx.x; p < b.nprob; p += blockDim.x) {
@@ -109,6 +111,7 @@ __device__ __forceinline__ void add_diag(ProbDiag *d, const double *v)
 // this kernel writes.
 __global__ void k_kick_close(BatchView b, int do_kick, int forces_ran, int items)
 {
+    chain_entry();
     __shared__ double red[9][kRedThreads / 32];
     __shared__ int pfirst, plast;
     if (blockIdx.x == 0) {
@@ -225,14 +228,14 @@ __global__ void k_kick_close(BatchView b, int do_kick, int forces_ran, int items
 
 cudaError_t launch_reset_step(const BatchView &b, int mode, cudaStream_t st)
 {
-    k_reset_step<<<(b.nprob + 127) / 128, 128, 0, st>>>(b, mode);
+    launch_chain(SPH_DEP(b), k_reset_step, (b.nprob + 127) / 128, 128, 0, st, b, mode);
     return cudaGetLastError();
 }
 
 cudaError_t launch_kick_drift(const BatchView &b, double dt_host, cudaStream_t st)
 {
     const long long blocks = b.ntot > 0 ? (b.ntot + 255) / 256 : 1;
-    k_kick_drift<<<(unsigned)blocks, 256, 0, st>>>(b, dt_host);
+    launch_chain(SPH_DEP(b), k_kick_drift, (unsigned)blocks, 256, 0, st, b, dt_host);
     return cudaGetLastError();
 }
 
@@ -244,7 +247,7 @@ cudaError_t launch_kick_close(const BatchView &b, int do_kick, int forces_ran, c
     items = items < 1 ? 1 : items > kCloseItems ? kCloseItems : items;
     const long long per = (long long)kRedThreads * items;
     const long long blocks = b.ntot > 0 ? (b.ntot + per - 1) / per : 1;
-    k_kick_close<<<(unsigned)blocks, kRedThreads, 0, st>>>(b, do_kick, forces_ran, (int)items);
+    launch_chain(SPH_DEP(b), k_kick_close, (unsigned)blocks, kRedThreads, 0, st, b, do_kick, forces_ran, (int)items);
     return cudaGetLastError();
 }
 

@@ -40,16 +40,16 @@ cudaError_t launch_density(const BatchView &b, int precision, int use_pred, cuda
 cudaError_t launch_block_tasks(const BatchView &b, int precision, cudaStream_t st)
 {
     const unsigned grid = (unsigned)dev_info().sm_count * 4;
-    if (precision == SPH_PREC_FP64) k_block_tasks<double><<<grid, 256, 0, st>>>(b, 1);
-    else k_block_tasks<float><<<grid, 256, 0, st>>>(b, 1);
+    if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_block_tasks<double>, grid, 256, 0, st, b, 1);
+    else launch_chain(SPH_DEP(b), k_block_tasks<float>, grid, 256, 0, st, b, 1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_block_leaf_tick(const BatchView &b, int precision, cudaStream_t st)
 {
     const unsigned grid = (unsigned)dev_info().sm_count * 8;
-    if (precision == SPH_PREC_FP64) k_block_leaf_tick<double, dbl4><<<grid, 256, 0, st>>>(b, 1);
-    else k_block_leaf_tick<float, float4><<<grid, 256, 0, st>>>(b, 1);
+    if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_block_leaf_tick<double, dbl4>, grid, 256, 0, st, b, 1);
+    else launch_chain(SPH_DEP(b), k_block_leaf_tick<float, float4>, grid, 256, 0, st, b, 1);
     return cudaGetLastError();
 }
 

@@ -751,7 +751,7 @@ struct DCfg {
                                                      : LPP == 1 ? SPH_DENS_LCAP1 : LPP == 2 ? 64 : LPP == 4 ? 40 : 24;
     static constexpr int CH = SPH_DENS_CH;
     static constexpr int WPB = D64 ? 2 : 4;
-    static constexpr int MINB = D64 ? 4 : LPP == 1 ? SPH_DENS_MINB1 : SPH_DENS_MINB;  // blocks per SM the registers allow
+    static constexpr int MINB = D64 ? 4 : K == SPH_KERNEL_M6 ? SPH_MINB_M6 : LPP == 1 ? SPH_DENS_MINB1 : SPH_DENS_MINB;  // blocks per SM the registers allow
     // FP64: rows of pairs waiting for their FP64 distance, candidates per room check
     static constexpr int LC = 32, SB = 32;
     static constexpr size_t wait = D64 ? (size_t)LC * 32 * sizeof(int) + CH * sizeof(int) : 0;
@@ -1360,6 +1360,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
 template <typename T, int LPP, bool UM, int K, bool WRAP>
 __global__ void __launch_bounds__(DCfg<T, LPP, UM, K>::WPB * 32, DCfg<T, LPP, UM, K>::MINB) k_density(BatchView b, int use_pred)
 {
+    chain_entry();
     using C = DCfg<T, LPP, UM, K>;
     extern __shared__ __align__(32) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1409,6 +1410,7 @@ struct FbCfg {
 template <typename T>
 __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchView b, int use_pred)
 {
+    chain_entry();
     using C = FbCfg<T>;
     using V = typename C::V;
     extern __shared__ __align__(32) unsigned char smem[];
@@ -1590,7 +1592,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
 // index within that leaf); the lists are evaluated, reading the partner's
 // data from global memory, when one of them or the table fills and at the end,
 // so that every lane evaluates about the same number of pairs.
-template <typename T, int LPP>
+template <typename T, int LPP, int K>
 struct FCfg {
     using V = typename Vec4<T>::type;
     static constexpr int CH = SPH_FORCE_CH;
@@ -1601,7 +1603,7 @@ struct FCfg {
     static constexpr int SB = LPP == 1 ? SPH_FORCE_SB1 : SPH_FORCE_SB;
     static constexpr int TAB = D64 ? 0 : SPH_FORCE_TAB;  // candidate leaves per table fill (<= 2048)
     static constexpr int WPB = D64 ? 2 : 4;
-    static constexpr int MINB = D64 ? 4 : LPP == 1 ? SPH_FORCE_MINB1 : SPH_FORCE_MINB;  // blocks per SM the registers allow
+    static constexpr int MINB = D64 ? 4 : K == SPH_KERNEL_M6 ? SPH_MINB_M6 : LPP == 1 ? SPH_FORCE_MINB1 : SPH_FORCE_MINB;  // blocks per SM the registers allow
     using Code = std::conditional_t<D64, int, unsigned short>;  // (FP64: the sorted index itself)
     static_assert(TAB <= 2048 && LC >= 2 * SB / LPP, "force list layout");
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
@@ -1662,7 +1664,7 @@ __device__ __forceinline__ dbl4 ld_ro<dbl4>(const dbl4 *p)
 template <typename T, int LPP, int K, bool WRAP, bool CD>
 __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0, unsigned char *mine, float Rall)
 {
-    using C = FCfg<T, LPP>;
+    using C = FCfg<T, LPP, K>;
     using KF = Kern<K>;
     constexpr float KR_f = (float)KF::R;
     using V = typename C::V;
@@ -2097,9 +2099,10 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
 // WRAP: the launch that serves the wrap list (leaves whose pair vectors may
 // miss the minimum image); the other launch puts them there.
 template <typename T, int LPP, int K, bool WRAP, bool CD>
-__global__ void __launch_bounds__(FCfg<T, LPP>::WPB * 32, FCfg<T, LPP>::MINB) k_forces(BatchView b)
+__global__ void __launch_bounds__(FCfg<T, LPP, K>::WPB * 32, FCfg<T, LPP, K>::MINB) k_forces(BatchView b)
 {
-    using C = FCfg<T, LPP>;
+    chain_entry();
+    using C = FCfg<T, LPP, K>;
     extern __shared__ __align__(32) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     unsigned char *mine = smem + wib * C::per_warp;
@@ -2156,8 +2159,7 @@ cudaError_t run_density(const BatchView &b, int use_pred, cudaStream_t st)
     }
     // the wrap-list launch serves few leaves (mostly none) unless a problem
     // has gravity or the launch is a block-step tick's
-    k_density<T, LPP, UM, K, WRAP><<<dev_info().sm_count * (WRAP && !b.any_gravity && !(b.block_on && b.block_tasks) ? 1 : per_sm),
-                                     C::WPB * 32, C::smem, st>>>(b, use_pred);
+    launch_chain(SPH_DEP(b), k_density<T, LPP, UM, K, WRAP>, dev_info().sm_count * (WRAP && !b.any_gravity && !(b.block_on && b.block_tasks) ? 1 : per_sm), C::WPB * 32, C::smem, st, b, use_pred);
     return cudaGetLastError();
 }
 
@@ -2170,7 +2172,7 @@ void run_density_fallback(const BatchView &b, int use_pred, cudaStream_t st)
         set_smem(k_density_fallback<T>, C::smem);
         init = true;
     }
-    k_density_fallback<T><<<dev_info().sm_count * 4, C::WPB * 32, C::smem, st>>>(b, use_pred);
+    launch_chain(SPH_DEP(b), k_density_fallback<T>, dev_info().sm_count * 4, C::WPB * 32, C::smem, st, b, use_pred);
 }
 
 // Block-step ticks, after the leaves: each leaf with particles whose step
@@ -2199,6 +2201,7 @@ __device__ __forceinline__ void block_tasks_one(const BatchView &b, int leaf, in
 template <typename T>
 __global__ void __launch_bounds__(256) k_block_tasks(BatchView b, int use_pred)
 {
+    chain_entry();
     const int lane = threadIdx.x & 31;
     const int nleaf = b.counters[0];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -2218,6 +2221,7 @@ __global__ void __launch_bounds__(256) k_block_tasks(BatchView b, int use_pred)
 template <typename T, typename T4>
 __global__ void __launch_bounds__(256) k_block_leaf_tick(BatchView b, int use_pred)
 {
+    chain_entry();
     const int lane = threadIdx.x & 31;
     const int nleaf = b.counters[0];
     if (blockIdx.x == 0)
@@ -2256,7 +2260,7 @@ __global__ void __launch_bounds__(256) k_block_leaf_tick(BatchView b, int use_pr
 template <typename T, int LPP, int K, bool WRAP, bool CD = false>
 cudaError_t run_forces(const BatchView &b, cudaStream_t st)
 {
-    using C = FCfg<T, LPP>;
+    using C = FCfg<T, LPP, K>;
     static bool init = false;
     if (!init) {
         set_smem(k_forces<T, LPP, K, WRAP, CD>, C::smem);
@@ -2267,7 +2271,7 @@ cudaError_t run_forces(const BatchView &b, cudaStream_t st)
     if (per_sm < 1) per_sm = 1;
     // the wrap list is short unless a problem uses the viscosity switch or Price's conductivity
     int grid = dev_info().sm_count * (WRAP && !b.any_general ? 1 : per_sm);
-    k_forces<T, LPP, K, WRAP, CD><<<grid, C::WPB * 32, C::smem, st>>>(b);
+    launch_chain(SPH_DEP(b), k_forces<T, LPP, K, WRAP, CD>, grid, C::WPB * 32, C::smem, st, b);
     cudaError_t e = cudaGetLastError();
     // the Cullen & Dehnen problems' leaves on the wrap list: their own launch
     // (never with block steps, the only users of whole-warp particles)

@@ -53,6 +53,7 @@ __device__ __forceinline__ void warp_hist_add(unsigned *h, unsigned d, bool vali
 
 __global__ void k_reset_bbox(ProbDyn *dyn, int nprob)
 {
+    chain_entry();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= nprob) return;
     for (int a = 0; a < 3; ++a) {
@@ -76,6 +77,7 @@ __device__ __forceinline__ void bbox_flush(const BatchView &b, int p, const unsi
 
 __global__ void k_bbox(BatchView b, int items)
 {
+    chain_entry();
     __shared__ unsigned long long red[6][kBboxThreads / 32];
     __shared__ int pfirst, plast;
     const long long base = (long long)blockIdx.x * blockDim.x * items;
@@ -137,6 +139,7 @@ __global__ void k_bbox(BatchView b, int items)
 
 __global__ void k_domain(BatchView b)
 {
+    chain_entry();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= b.nprob) return;
     const PhysParams &ph = b.prob[p].ph;
@@ -198,6 +201,7 @@ __device__ __forceinline__ unsigned morton_key_code(const BatchView &b, int p, l
 // Keys of every particle, and the digit histograms of every pass.
 __global__ void k_keys_hist(BatchView b, unsigned long long *kout, unsigned *hist, int passes, int lo)
 {
+    chain_entry();
     __shared__ unsigned h[8][256];
     for (int k = threadIdx.x; k < 8 * 256; k += blockDim.x) (&h[0][0])[k] = 0u;
     __syncthreads();
@@ -224,6 +228,7 @@ __global__ void k_onesweep(const unsigned long long *kin, const unsigned *vin, u
                            unsigned *vout, long long n, int shift, const unsigned *hist, unsigned *status,
                            unsigned *tile_ctr, int identity_vals, unsigned *timeout_flag)
 {
+    chain_entry();
     constexpr int NW = kSortThreads / 32;
     constexpr int TILE = kSortThreads * ITEMS;
     __shared__ unsigned run[256];
@@ -336,14 +341,14 @@ cudaError_t launch_domain_and_keys(const BatchView &b, cudaStream_t st)
     // bounding boxes of isolated problems (periodic boxes need no pass)
     if (b.ntot == 0 || !b.any_isolated) return cudaSuccess;
     int pb = (b.nprob + 127) / 128;
-    k_reset_bbox<<<pb, 128, 0, st>>>(b.dyn, b.nprob);
+    launch_chain(SPH_DEP(b), k_reset_bbox, pb, 128, 0, st, b.dyn, b.nprob);
     // two blocks per SM of up to kBboxItems particles a thread
     const long long fill = 2LL * dev_info().sm_count * kBboxThreads;
     long long items = (b.ntot + fill - 1) / fill;
     items = items < 1 ? 1 : items > kBboxItems ? kBboxItems : items;
     const long long nb = (b.ntot + kBboxThreads * items - 1) / (kBboxThreads * items);
-    k_bbox<<<(unsigned)nb, kBboxThreads, 0, st>>>(b, (int)items);
-    k_domain<<<pb, 128, 0, st>>>(b);
+    launch_chain(SPH_DEP(b), k_bbox, (unsigned)nb, kBboxThreads, 0, st, b, (int)items);
+    launch_chain(SPH_DEP(b), k_domain, pb, 128, 0, st, b);
     return cudaGetLastError();
 }
 
@@ -369,12 +374,12 @@ cudaError_t launch_radix_sort(const BatchView &b, cudaStream_t st)
     // the passes ping-pong between the two key buffers: start in the one that
     // leaves the sorted keys in keys[0] for the leaf builder
     int src = passes & 1;
-    k_keys_hist<<<kb < cap ? kb : cap, 256, 0, st>>>(b, b.keys[src], hist, passes, b.key_lo);
+    launch_chain(SPH_DEP(b), k_keys_hist, kb < cap ? kb : cap, 256, 0, st, b, b.keys[src], hist, passes, b.key_lo);
     for (int pass = 0; pass < passes; ++pass) {
         const bool last = pass == passes - 1;
         unsigned *vdst = last ? (unsigned *)b.perm : b.vals[src ^ 1];
         auto kern = items == 1 ? k_onesweep<1> : items == 2 ? k_onesweep<2> : items == 4 ? k_onesweep<4> : k_onesweep<8>;
-        kern<<<ntile, kSortThreads, 0, st>>>(b.keys[src], b.vals[src], b.keys[src ^ 1], vdst, n, b.key_lo + 8 * pass,
+        launch_chain(SPH_DEP(b), kern, ntile, kSortThreads, 0, st, b.keys[src], b.vals[src], b.keys[src ^ 1], vdst, n, b.key_lo + 8 * pass,
                                              hist + pass * 256, status + (size_t)pass * ntile * 256, ctr + pass,
                                              pass == 0, (unsigned *)&b.counters[kTimeoutCounter]);
         src ^= 1;

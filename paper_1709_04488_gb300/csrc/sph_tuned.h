@@ -17,6 +17,11 @@
 #ifndef SPH_DENS_MINB1
 #define SPH_DENS_MINB1 4
 #endif
+// (both pair kernels with the M6 kernel, whose longer lists gain from a fifth
+// block more than its spills cost: M6 lattice 37^3 276 -> 258 us and 328 -> 317)
+#ifndef SPH_MINB_M6
+#define SPH_MINB_M6 5
+#endif
 #ifndef SPH_DENS_LCAP1
 #define SPH_DENS_LCAP1 96
 #endif
