@@ -55,13 +55,10 @@ void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precis
 {
     const long long n = ntot > 0 ? ntot : 1;
     const size_t v4 = precision == SPH_PREC_FP64 ? sizeof(dbl4) : sizeof(float4);
-    const long long nblk = sort_tiles(n);
-    const long long passes = (key_bits_for(nprob) + 7) / 8;
     b.keys[0] = c.take<unsigned long long>(n);
     b.keys[1] = c.take<unsigned long long>(n);
     b.vals[0] = c.take<unsigned>(n);
     b.vals[1] = c.take<unsigned>(n);
-    b.hist = c.take<unsigned>(passes * 256 + 8 + passes * nblk * 256);
     b.perm = c.take<int>(n);
     double **sd[] = {&b.sx, &b.sy, &b.sz, &b.sh, &b.sm, &b.srho, &b.somega, &b.sP, &b.sc,
                      &b.vpx, &b.vpy, &b.vpz, &b.up, &b.ap};
@@ -114,7 +111,9 @@ void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precis
     b.zero_lo = (char *)b.tile_state;
     b.node_ctr[0] = nullptr;
     for (int l = 1; l <= kMaxLevels; ++l) b.node_ctr[l] = c.take<int>(b.node_cap[l]);
-    b.zero_bytes = c.base ? (size_t)((char *)(b.node_ctr[kMaxLevels] + b.node_cap[kMaxLevels]) - b.zero_lo) : 0;
+    const long long words = sort_words(key_bits_for(nprob), n);
+    b.hist = c.take<unsigned>(words);
+    b.zero_bytes = c.base ? (size_t)((char *)(b.hist + words) - b.zero_lo) : 0;
 }
 
 void carve_tables(Carver &c, BatchView &b, int nprob)

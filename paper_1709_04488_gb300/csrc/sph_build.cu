@@ -166,7 +166,7 @@ __device__ void problem_meta(const BatchView &b)
 // with a decoupled look-back between tiles, the leaf starts and owners; the
 // last block to finish lays out the leaves and tree levels of every problem
 // and clears the tile state for the next build.
-__global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b)
+__global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b, long long sort_words)
 {
     chain_entry();
     __shared__ unsigned long long sk[kLeafTile + 2 * kHalo];
@@ -249,6 +249,10 @@ __global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b)
             b.counters[0] = (int)run;
         }
     }
+    // the sort's histograms, counters and look-back status, for the next sort
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < sort_words;
+         k += (long long)gridDim.x * blockDim.x)
+        b.hist[k] = 0u;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) s_last = atomicAdd(&ts[1], 1u) == gridDim.x - 1;
@@ -372,7 +376,7 @@ cudaError_t launch_build_leaves(const BatchView &b, int precision, cudaStream_t 
 {
     if (b.ntot == 0) return cudaSuccess;
     const long long tiles = (b.ntot + kLeafTile - 1) / kLeafTile;
-    launch_chain(SPH_DEP(b), k_leaf_scan, (unsigned)tiles, kLeafThreads, 0, st, b);
+    launch_chain(SPH_DEP(b), k_leaf_scan, (unsigned)tiles, kLeafThreads, 0, st, b, sort_words(b.key_bits - b.key_lo, b.ntot));
     int pb = persistent_blocks(256);
     if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_leaf_props<dbl4, false>, pb, 256, 0, st, b);
     else launch_chain(SPH_DEP(b), k_leaf_props<float4, false>, pb, 256, 0, st, b);

@@ -211,7 +211,7 @@ struct BatchView {
     // sort
     unsigned long long *keys[2];
     unsigned *vals[2];
-    unsigned *hist;              // sort: digit histograms, tile counters, look-back status
+    unsigned *hist;              // sort: digit histograms, tile counters, look-back status (in the zero region)
     int *perm;                   // sorted position -> batch-global original index
     // sorted FP64 copies
     double *sx, *sy, *sz, *sh, *sm;
@@ -243,7 +243,7 @@ struct BatchView {
     // state that must be zero before a build; the kernels clear what they use
     unsigned *tile_state;        // leaf scan: ticket, finished tiles, look-back status per tile
     int *node_ctr[kMaxLevels + 1];  // arrival counters of the nodes of levels 1..
-    char *zero_lo;               // [zero_lo, zero_lo + zero_bytes) holds the two above
+    char *zero_lo;               // [zero_lo, zero_lo + zero_bytes) holds the two above and hist
     size_t zero_bytes;
     int *fallback_list;          // [ntot] sorted indices needing the slow path
     int *wrap_list;              // [ntot] leaves served by the minimum-image (wrap) launches
@@ -493,6 +493,7 @@ int status_to_code(unsigned st);
 long long leaves_upper_bound(long long n);
 long long leaf_tiles(long long n);  // tiles of the leaf scan
 long long sort_tiles(long long n);  // tiles of one radix-sort pass
+long long sort_words(int bits, long long n);  // words of BatchView::hist a sort of `bits` key bits uses
 int levels_needed(long long max_leaves);
 
 }  // namespace sph

@@ -12,20 +12,22 @@ namespace sph {
 namespace {
 
 constexpr int kSortThreads = 256;
-// keys per thread of a radix pass (1, 2, 4 or 8): small problems take short
-// tiles (more blocks in flight), large ones long tiles (fewer look-back records)
+// keys per thread of a radix pass: small problems take short tiles (more
+// blocks in flight), large ones long tiles (fewer look-back records).  The
+// sort stage with 2, 4 and 8: 36864 keys 31.0, 33.1, 33.1 us; 103823: 43.1,
+// 41.3, 43.2; 262144: 69.7, 61.1, 56.9; 1e6: -, 161.8, 161.2
 #ifndef SPH_SORT_ITEMS_S
-#define SPH_SORT_ITEMS_S 2  // up to 2^18 keys
+#define SPH_SORT_ITEMS_S 2  // up to 2^16 keys
 #endif
 #ifndef SPH_SORT_ITEMS_M
-#define SPH_SORT_ITEMS_M 8  // up to 2^22 keys
+#define SPH_SORT_ITEMS_M 4  // up to 3 x 2^16 keys
 #endif
 #ifndef SPH_SORT_ITEMS_L
 #define SPH_SORT_ITEMS_L 8
 #endif
 int sort_items(long long n)
 {
-    return n <= (1ll << 18) ? SPH_SORT_ITEMS_S : n <= (1ll << 22) ? SPH_SORT_ITEMS_M : SPH_SORT_ITEMS_L;
+    return n <= (1ll << 16) ? SPH_SORT_ITEMS_S : n <= 3 * (1ll << 16) ? SPH_SORT_ITEMS_M : SPH_SORT_ITEMS_L;
 }
 constexpr int kBboxThreads = 1024, kBboxItems = 64;
 
@@ -223,46 +225,77 @@ __global__ void k_keys_hist(BatchView b, unsigned long long *kout, unsigned *his
     }
 }
 
+// One pass: a tile of kSortThreads * ITEMS keys, warp w's the w-th part of it.
+// Each warp ranks its keys against its own digit counts, so that ranking
+// takes no barrier; the counts then give the tile's digit counts (for the
+// look-back) and each warp's place within them.  (Rows of kSortThreads keys
+// ranked by the whole block, with 3 barriers a row, and a 16-barrier scan of
+// the digit histogram made the sort stage 49.2 us at 103823 keys and 73.8 at
+// 262144; 41.3 and 56.9 like this.)
 template <int ITEMS>
-__global__ void k_onesweep(const unsigned long long *kin, const unsigned *vin, unsigned long long *kout,
-                           unsigned *vout, long long n, int shift, const unsigned *hist, unsigned *status,
-                           unsigned *tile_ctr, int identity_vals, unsigned *timeout_flag)
+__global__ void __launch_bounds__(kSortThreads) k_onesweep(const unsigned long long *kin, const unsigned *vin,
+                                                           unsigned long long *kout, unsigned *vout, long long n, int shift,
+                                                           const unsigned *hist, unsigned *status, unsigned *tile_ctr,
+                                                           int identity_vals, unsigned *timeout_flag)
 {
     chain_entry();
     constexpr int NW = kSortThreads / 32;
     constexpr int TILE = kSortThreads * ITEMS;
     __shared__ unsigned run[256];
     __shared__ unsigned wcnt[NW][256];
-    __shared__ unsigned cnt[256];
-    __shared__ unsigned gpre[256];
+    __shared__ unsigned wsum[NW];
     __shared__ int s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = threadIdx.x;
     if (t == 0) s_tile = (int)atomicAdd(tile_ctr, 1u);
-    cnt[t] = 0u;
-    for (int w = 0; w < NW; ++w) wcnt[w][t] = 0u;
+#pragma unroll
+    for (int k = 0; k < 256; k += 32) wcnt[warp][k + lane] = 0u;
     // exclusive scan of the pass's global digit histogram
-    gpre[t] = hist[t];
-    __syncthreads();
-    for (int o = 1; o < 256; o <<= 1) {
-        unsigned v = t >= o ? gpre[t - o] : 0u;
-        __syncthreads();
-        gpre[t] += v;
-        __syncthreads();
+    const unsigned hv = hist[t];
+    unsigned hs = hv;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, hs, o);
+        if (lane >= o) hs += v;
     }
-    const unsigned gstart = gpre[t] - hist[t];
+    if (lane == 31) wsum[warp] = hs;
+    __syncthreads();
     const int tile = s_tile;
-    const long long base = (long long)tile * TILE;
-    // local digit counts
+    unsigned gstart = hs - hv;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) gstart += w < warp ? wsum[w] : 0u;
+    // this warp's keys and their ranks among its equal digits, in index order
+    const long long base = (long long)tile * TILE + warp * (32 * ITEMS) + lane;
+    const unsigned lt = (1u << lane) - 1u;
     unsigned long long keys[ITEMS];
+    unsigned vals[ITEMS], rank[ITEMS];
+#pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
-        long long k = base + r * kSortThreads + t;
+        const long long k = base + r * 32;
         keys[r] = k < n ? kin[k] : 0ull;
-        warp_hist_add(cnt, (unsigned)(keys[r] >> shift) & 255u, k < n);
+        vals[r] = k < n ? (identity_vals ? (unsigned)k : vin[k]) : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const bool ok = base + r * 32 < n;
+        const unsigned d = (unsigned)(keys[r] >> shift) & 255u;
+        const unsigned peers = __match_any_sync(0xffffffffu, ok ? d : 256u);
+        const unsigned before = wcnt[warp][d];
+        __syncwarp();
+        if (ok && (peers & lt) == 0u) wcnt[warp][d] = before + __popc(peers);
+        __syncwarp();
+        rank[r] = before + __popc(peers & lt);
     }
     __syncthreads();
+    // the tile's count of digit t, and what the warps before each put there
+    unsigned mine = 0u;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        const unsigned c = wcnt[w][t];
+        wcnt[w][t] = mine;
+        mine += c;
+    }
     // publish this tile's counts, then look back over the earlier tiles
     unsigned *st = status + (long long)tile * 256;
-    const unsigned mine = cnt[t];
     if (tile == 0) {
         atomicExch(&st[t], kFlagPre | mine);
         run[t] = gstart;
@@ -302,36 +335,14 @@ __global__ void k_onesweep(const unsigned long long *kin, const unsigned *vin, u
         run[t] = gstart + excl;
     }
     __syncthreads();
-    // stable ranks inside the tile (index order), then scatter
-    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
     for (int r = 0; r < ITEMS; ++r) {
-        long long k = base + r * kSortThreads + t;
-        bool ok = k < n;
-        unsigned long long key = keys[r];
-        unsigned val = ok ? (identity_vals ? (unsigned)k : vin[k]) : 0u;
-        unsigned d = ok ? (unsigned)(key >> shift) & 255u : 256u + lane;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        unsigned rank = __popc(peers & lt);
-        bool leader = (peers & lt) == 0u;
-        if (ok && leader) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        if (ok) {
-            unsigned off = run[d] + rank;
-            for (int w = 0; w < warp; ++w) off += wcnt[w][d];
-            kout[off] = key;
-            vout[off] = val;
-        }
-        __syncthreads();
-        unsigned tot = 0;
-        for (int w = 0; w < NW; ++w) {
-            tot += wcnt[w][t];
-            wcnt[w][t] = 0;
-        }
-        run[t] += tot;
-        __syncthreads();
+        if (base + r * 32 >= n) continue;
+        const unsigned d = (unsigned)(keys[r] >> shift) & 255u, off = run[d] + wcnt[warp][d] + rank[r];
+        kout[off] = keys[r];
+        vout[off] = vals[r];
     }
 }
-
 
 }  // namespace
 
@@ -358,6 +369,13 @@ long long sort_tiles(long long n)
     return (n + t - 1) / t;
 }
 
+// hist[passes][256] | tile counters[8] | status[passes][tiles][256]
+long long sort_words(int bits, long long n)
+{
+    const long long passes = (bits + 7) / 8;
+    return passes * 256 + 8 + passes * sort_tiles(n) * 256;
+}
+
 cudaError_t launch_radix_sort(const BatchView &b, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
@@ -368,13 +386,19 @@ cudaError_t launch_radix_sort(const BatchView &b, cudaStream_t st)
     const int passes = (b.key_bits - b.key_lo + 7) / 8;
     // hist[passes][256] | tile counters[passes] | status[passes][ntile][256]
     unsigned *hist = b.hist, *ctr = b.hist + passes * 256, *status = b.hist + passes * 256 + 8;
-    cudaMemsetAsync(b.hist, 0, sizeof(unsigned) * ((size_t)passes * 256 + 8 + (size_t)passes * ntile * 256), st);
-    int kb = (int)((n + 255) / 256);
-    int cap = dev_info().sm_count * 8;
+    // (histograms, counters and status are zero: the leaf scan, which follows
+    // every sort, clears what it used)
+    // one key per thread until every SM has two blocks, then two (half as many
+    // blocks add their histograms).  A plain launch: placed early, beside the
+    // drift's blocks, this kernel's went to the few SMs those left idle, whose
+    // FP64 pipes then took 27 us for the keys of 36864 particles (spread over
+    // the SMs 4.7)
+    const long long kb = n <= 2ll * dev_info().sm_count * 256 ? (n + 255) / 256 : (n + 511) / 512;
+    const int cap = dev_info().sm_count * 8;
     // the passes ping-pong between the two key buffers: start in the one that
     // leaves the sorted keys in keys[0] for the leaf builder
     int src = passes & 1;
-    launch_chain(SPH_DEP(b), k_keys_hist, kb < cap ? kb : cap, 256, 0, st, b, b.keys[src], hist, passes, b.key_lo);
+    launch_chain(false, k_keys_hist, kb < cap ? kb : cap, 256, 0, st, b, b.keys[src], hist, passes, b.key_lo);
     for (int pass = 0; pass < passes; ++pass) {
         const bool last = pass == passes - 1;
         unsigned *vdst = last ? (unsigned *)b.perm : b.vals[src ^ 1];
