@@ -277,6 +277,11 @@ PhysParams phys_of(const sph_params *p)
         ph.box_inv[a] = p->periodic ? 1.0 / ph.box_len[a] : 0.0;
         ph.box_inv_f[a] = p->periodic ? 1.0f / ph.box_len_f[a] : 0.f;
     }
+    if (p->periodic) {
+        const double ext = std::fmax(p->box_len[0], std::fmax(p->box_len[1], p->box_len[2]));
+        ph.key_inv = 1.0 / ext * (double)(1 << kMortonBits);
+        for (int a = 0; a < 3; ++a) ph.box_hi[a] = p->box_lo[a] + p->box_len[a];
+    }
     if (p->periodic)
         for (int a = 0; a < 3; ++a) {
             const float m = 2.f * (float)(std::fabs(p->box_lo[a]) + p->box_len[a]);
@@ -557,10 +562,10 @@ static int enqueue_density(const BatchView &b, int precision, int use_pred, cuda
         CU(launch_domain_and_keys(b, st));
         CU(launch_radix_sort(b, st));
     }
-    CU(launch_gather(b, st));
+    if (!rebuild) CU(launch_gather(b, st));
     mk.at(SPH_STAGE_TREE, st);
     mk.done(SPH_STAGE_SORT);
-    if (rebuild) CU(launch_build_leaves(b, precision, st));
+    if (rebuild) CU(launch_build_leaves(b, precision, true, st));  // (gathers too)
     else CU(launch_update_leaves(b, precision, st));
     mk.at(SPH_STAGE_DENSITY, st);
     mk.done(SPH_STAGE_TREE);
@@ -674,7 +679,7 @@ static int enqueue_block_leaves(const BatchView &b, int prec, bool rebuild, cuda
         CU(launch_domain_and_keys(b, st));
         CU(launch_radix_sort(b, st));
         CU(launch_block_gather(b, prec, st));  // (also which particles end their step now)
-        CU(launch_build_leaves(b, prec, st));
+        CU(launch_build_leaves(b, prec, false, st));
         CU(launch_block_tasks(b, prec, st));  // (and the restaging of the particles that keep their solve)
     } else {
         CU(launch_block_leaf_tick(b, prec, st));  // drift, gather, leaf boxes, tasks and restaging
@@ -702,7 +707,7 @@ static int enqueue_block_last(const BatchView &bl, int prec, int L, cudaStream_t
     CU(launch_domain_and_keys(bl, st));
     CU(launch_radix_sort(bl, st));
     CU(launch_block_gather(bl, prec, st));
-    CU(launch_build_leaves(bl, prec, st));
+    CU(launch_build_leaves(bl, prec, false, st));
     return enqueue_block_passes(bl, prec, L, false, 0, 0, st);
 }
 
@@ -902,8 +907,7 @@ int sph_block_step(sph_ctx *c, double *dtmax_out, int64_t *evals_out)
         // the context's leaves do not hold its particles (a batch moved them): build them first
         CU(launch_domain_and_keys(c->bv, st));
         CU(launch_radix_sort(c->bv, st));
-        CU(launch_gather(c->bv, st));
-        CU(launch_build_leaves(c->bv, c->prm.precision, st));
+        CU(launch_build_leaves(c->bv, c->prm.precision, true, st));
     }
     if (st == nullptr) {
         int rc = block_step_eager(c, b, bl);  // the legacy default stream cannot be captured
@@ -1135,8 +1139,7 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     CU(launch_reset_step(b, 1, st));
     CU(launch_domain_and_keys(b, st));
     CU(launch_radix_sort(b, st));
-    CU(launch_gather(b, st));
-    CU(launch_build_leaves(b, c->prm.precision, st));
+    CU(launch_build_leaves(b, c->prm.precision, true, st));
     CU(launch_set_sorted_h(b, h_in, st));
     CU(launch_refit(b, c->prm.precision, st));
     CU(launch_neighbour_export(b, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));

@@ -115,12 +115,23 @@ __global__ void k_block_plan(BatchView b, int L)
     b.scratch64[7] = __double_as_longlong(tau);
 }
 
-__device__ __forceinline__ void next_event(const BatchView &b, long long t)
+// the next event tick: the smallest t of the block's threads (ticks fit an
+// int; kNoTick: none) joins the minimum, one atomic per block (one per warp
+// queued 8192 of them on one address at 64^3 particles)
+constexpr int kNoTick = 0x7fffffff;
+__device__ __forceinline__ void next_event(const BatchView &b, int t)
 {
-    const long long m = warp_min(t);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMin((unsigned long long *)&b.scratch64[2], (unsigned long long)m);
-        __threadfence();  // (before the block reports itself done)
+    __shared__ int red[kBlockThreads / 32];
+    const int m = __reduce_min_sync(0xffffffffu, t);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int v = red[0];
+        for (int w = 1; w < kBlockThreads / 32; ++w) v = min(v, red[w]);
+        if (v != kNoTick) {
+            atomicMin((unsigned long long *)&b.scratch64[2], (unsigned long long)v);
+            __threadfence();  // (before the block reports itself done)
+        }
     }
 }
 
@@ -130,7 +141,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_open(BatchView b, int L
 {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const double dtmax = bits_d(b.scratch64[6]), tau = bits_d(b.scratch64[7]);
-    long long t1 = 0x7fffffffffffffffLL;
+    int t1 = kNoTick;
     if (g < b.ntot && dtmax > 0) {
         const ProbStatic &ps = b.prob[0];
         const long long i = g - ps.base;
@@ -140,7 +151,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_open(BatchView b, int L
         b.blev[g] = l;
         b.bt0[g] = 0;
         b.bt1[g] = (int)((1LL << L) >> l);
-        t1 = b.bt1[g];
+        t1 = (int)((1LL << L) >> l);
         const double hd = half_ticks(t1, tau);
         const long long n = b.ntot;
         b.bvh[g] = block_kick(ps.vx[i], ps.ax[i], hd);
@@ -256,7 +267,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_kick(BatchView b, int L
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long k = b.scratch64[5];
     const double dtmax = bits_d(b.scratch64[6]), tau = bits_d(b.scratch64[7]);
-    long long tnext = 0x7fffffffffffffffLL;
+    int tnext = kNoTick;
     if (g < b.ntot) {
         const ProbStatic &ps = b.prob[0];
         const PhysParams &ph = ps.ph;
@@ -265,6 +276,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_kick(BatchView b, int L
         const double *A[3] = {ps.ax, ps.ay, ps.az};
         double *V[3] = {ps.vx, ps.vy, ps.vz};
         int t0 = b.bt0[g], t1 = b.bt1[g], lev = b.blev[g];
+        bool changed = t1 == k;
         if (t1 == k) {
             // every input first (the stores below could alias them for the
             // compiler: one memory round trip each), the kicked v, u and
@@ -317,12 +329,15 @@ __global__ void __launch_bounds__(kBlockThreads) k_block_kick(BatchView b, int L
                     if (ph.av_switch) b.bvh[4 * n + g] = block_kick(b.bvh[4 * n + g], ps.dalpha[i], corr);
                     t1 = (int)ke;
                     lev = rq;
+                    changed = true;
                 }
             }
         }
-        b.bt0[g] = t0;
-        b.bt1[g] = t1;
-        b.blev[g] = lev;
+        if (changed) {
+            b.bt0[g] = t0;
+            b.bt1[g] = t1;
+            b.blev[g] = lev;
+        }
         if (t1 > k) tnext = t1;
     }
     next_event(b, tnext);

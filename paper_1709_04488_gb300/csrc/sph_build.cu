@@ -19,27 +19,42 @@ namespace sph {
 namespace {
 
 constexpr int kLeafThreads = 256;
-constexpr int kLeafItems = 1;  // consecutive particles per thread
-constexpr int kLeafTile = kLeafThreads * kLeafItems;
+// consecutive particles per thread of the leaf scan: fewer, longer tiles look
+// back over fewer records where there are many (leaf and tree stage with 1, 2
+// and 4: 103823 particles 33.2, 36.5, 40.8 us; 262144: 45.1, 43.0, 45.0; 8e6:
+// 1092, 1018, 984)
+int leaf_items(long long n) { return n <= (1ll << 17) ? 1 : n <= (1ll << 21) ? 2 : 4; }
 // leaf cell: the coarsest cell with at most cell_limit(leaf size) particles
 __host__ __device__ constexpr int cell_limit(int leaf) { return 4 * leaf; }
 constexpr int kHalo = 128;  // >= cell_limit of every leaf size (1..32)
 constexpr unsigned kTileAgg = 1u << 30, kTilePre = 2u << 30, kTileMask = (1u << 30) - 1u;
 constexpr long long kTileSpinLimit = 1ll << 24;
 
+// sorted particle s: position, mass and h into sorted order (p: its problem)
+struct Gathered {
+    double x, y, z, m, h;
+};
+__device__ __forceinline__ Gathered gather_load(const BatchView &b, int p, long long s)
+{
+    const ProbStatic &ps = b.prob[p];
+    const long long i = (long long)b.perm[s] - ps.base;
+    return {ps.x[i], ps.y[i], ps.z[i], ps.uniform_m ? ps.m_uniform : ps.m[i], ps.h[i]};  // (equal masses: no random read)
+}
+__device__ __forceinline__ void gather_store(const BatchView &b, long long s, const Gathered &g)
+{
+    b.sx[s] = g.x;
+    b.sy[s] = g.y;
+    b.sz[s] = g.z;
+    b.sm[s] = g.m;
+    b.sh[s] = g.h;
+}
+
 __global__ void k_gather(BatchView b)
 {
     chain_entry();
     long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= b.ntot) return;
-    int p = (int)(b.keys[0][s] >> kMortonTotal);
-    const ProbStatic &ps = b.prob[p];
-    long long i = (long long)b.perm[s] - ps.base;
-    b.sx[s] = ps.x[i];
-    b.sy[s] = ps.y[i];
-    b.sz[s] = ps.z[i];
-    b.sm[s] = ps.uniform_m ? ps.m_uniform : ps.m[i];  // (equal masses: no random read)
-    b.sh[s] = ps.h[i];
+    gather_store(b, s, gather_load(b, (int)(b.keys[0][s] >> kMortonTotal), s));
 }
 
 __device__ __forceinline__ int common_levels(unsigned long long a, unsigned long long b)
@@ -50,7 +65,7 @@ __device__ __forceinline__ int common_levels(unsigned long long a, unsigned long
 }
 
 // Leaf start flag of sorted particle s (see the file comment for the rule);
-// K holds the keys of [k0, k0 + kLeafTile + 2 kHalo), s inside the middle part.
+// K holds the keys of [k0, k0 + tile + 2 kHalo), s inside the middle part.
 // The common key prefix with s shrinks monotonically away from s, so the
 // cell of s at level l is found by two binary searches; only levels whose
 // cell excludes s - ncell and s + ncell can hold at most ncell particles.
@@ -165,10 +180,14 @@ __device__ void problem_meta(const BatchView &b)
 // Leaf start flags, their inclusive scan (the leaf index of every particle)
 // with a decoupled look-back between tiles, the leaf starts and owners; the
 // last block to finish lays out the leaves and tree levels of every problem
-// and clears the tile state for the next build.
+// and clears the tile state for the next build.  GATHER: also the gather into
+// sorted order, whose random reads are in flight while the flags are found
+// (a launch of its own took 3.3 us at 4096 particles).
+template <int kLeafItems, bool GATHER>
 __global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b, long long sort_words)
 {
     chain_entry();
+    constexpr int kLeafTile = kLeafThreads * kLeafItems;
     __shared__ unsigned long long sk[kLeafTile + 2 * kHalo];
     __shared__ int wsum[kLeafThreads / 32];
     __shared__ unsigned s_tile, s_prefix;
@@ -185,6 +204,13 @@ __global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b, long lo
         sk[k] = (g >= 0 && g < n) ? b.keys[0][g] : 0ull;
     }
     __syncthreads();
+    Gathered ga[kLeafItems];
+    if (GATHER)
+#pragma unroll
+        for (int r = 0; r < kLeafItems; ++r) {
+            const long long s = base + r * kLeafThreads + threadIdx.x;
+            if (s < n) ga[r] = gather_load(b, (int)(sk[s - k0] >> kMortonTotal), s);
+        }
     unsigned f[kLeafItems];
     int tsum = 0;
     const long long s0 = base + (long long)threadIdx.x * kLeafItems;
@@ -192,6 +218,12 @@ __global__ void __launch_bounds__(kLeafThreads) k_leaf_scan(BatchView b, long lo
         f[r] = s0 + r < n ? leaf_flag(b, sk, k0, s0 + r) : 0u;
         tsum += (int)f[r];
     }
+    if (GATHER)
+#pragma unroll
+        for (int r = 0; r < kLeafItems; ++r) {
+            const long long s = base + r * kLeafThreads + threadIdx.x;
+            if (s < n) gather_store(b, s, ga[r]);
+        }
     int agg;
     const int ex = block_excl_scan(tsum, wsum, &agg);
     // decoupled look-back, 32 predecessors per round (warp 0)
@@ -372,11 +404,13 @@ cudaError_t launch_gather(const BatchView &b, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_build_leaves(const BatchView &b, int precision, cudaStream_t st)
+cudaError_t launch_build_leaves(const BatchView &b, int precision, bool gather, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
-    const long long tiles = (b.ntot + kLeafTile - 1) / kLeafTile;
-    launch_chain(SPH_DEP(b), k_leaf_scan, (unsigned)tiles, kLeafThreads, 0, st, b, sort_words(b.key_bits - b.key_lo, b.ntot));
+    const int items = leaf_items(b.ntot);
+    const auto scan = gather ? (items == 1 ? k_leaf_scan<1, true> : items == 2 ? k_leaf_scan<2, true> : k_leaf_scan<4, true>)
+                             : (items == 1 ? k_leaf_scan<1, false> : items == 2 ? k_leaf_scan<2, false> : k_leaf_scan<4, false>);
+    launch_chain(SPH_DEP(b), scan, leaf_tiles(b.ntot), kLeafThreads, 0, st, b, sort_words(b.key_bits - b.key_lo, b.ntot));
     int pb = persistent_blocks(256);
     if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_leaf_props<dbl4, false>, pb, 256, 0, st, b);
     else launch_chain(SPH_DEP(b), k_leaf_props<float4, false>, pb, 256, 0, st, b);
@@ -405,6 +439,10 @@ cudaError_t launch_refit(const BatchView &b, int precision, cudaStream_t st)
     return cudaGetLastError();
 }
 
-long long leaf_tiles(long long n) { return (n + kLeafTile - 1) / kLeafTile; }
+long long leaf_tiles(long long n)
+{
+    const long long t = (long long)kLeafThreads * leaf_items(n);
+    return (n + t - 1) / t;
+}
 
 }  // namespace sph

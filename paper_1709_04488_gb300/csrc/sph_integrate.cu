@@ -69,7 +69,7 @@ __global__ void k_kick_drift(BatchView b, double dt_host)
         double x = x0[k] + vh * dt;
         if (ph.periodic) {
             double lo = ph.box_lo[k], L = ph.box_len[k];
-            if (x >= lo + L) x -= L;
+            if (x >= ph.box_hi[k]) x -= L;
             else if (x < lo) x += L;
         }
         X[k][i] = x;
@@ -100,6 +100,35 @@ __device__ __forceinline__ void add_diag(ProbDiag *d, const double *v)
     double *dst[9] = {&d->mass, &d->mom[0], &d->mom[1], &d->mom[2], &d->energy,
                       &d->fsum[0], &d->fsum[1], &d->fsum[2], &d->dEdt};
     for (int k = 0; k < 9; ++k) atomicAdd(dst[k], v[k]);
+}
+
+// The warp's sums of nine values into red[k][w]: each exchange halves the
+// values a lane carries, 16 FP64 additions in place of 45 (the FP64 pipe is
+// the kernel's bound, and most of a small problem's work is this reduction).
+__device__ __forceinline__ void warp_sum9(const double (&v)[9], double (*red)[kRedThreads / 32], int w)
+{
+    const int lane = threadIdx.x & 31;
+    double a[8], c[4], e[2];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {  // lanes below 16: values 0..7; above: value 8 in a[0]
+        const double hi = k == 0 ? v[8] : 0.0;
+        const double got = __shfl_xor_sync(0xffffffffu, lane & 16 ? v[k] : hi, 16);
+        a[k] = (lane & 16 ? hi : v[k]) + got;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double got = __shfl_xor_sync(0xffffffffu, lane & 8 ? a[k] : a[k + 4], 8);
+        c[k] = (lane & 8 ? a[k + 4] : a[k]) + got;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double got = __shfl_xor_sync(0xffffffffu, lane & 4 ? c[k] : c[k + 2], 4);
+        e[k] = (lane & 4 ? c[k + 2] : c[k]) + got;
+    }
+    double x = (lane & 2 ? e[1] : e[0]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? e[0] : e[1], 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    const int k = (lane & 16 ? 8 : 0) + (lane & 8 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 2 ? 1 : 0);
+    if (!(lane & 1) && k < 9) red[k][w] = x;
 }
 
 // Closing half kick (Eq. LFKDK2, optional) and the FP64 reductions per
@@ -206,10 +235,7 @@ __global__ void k_kick_close(BatchView b, int do_kick, int forces_ran, int items
         v[8] += m * (vel[0] * a[0] + vel[1] * a[1] + vel[2] * a[2] + (adi ? du : 0.0));
     }
     if (pfirst == plast) {
-        for (int k = 0; k < 9; ++k) {
-            double x = warp_sum(v[k]);
-            if ((threadIdx.x & 31) == 0) red[k][threadIdx.x >> 5] = x;
-        }
+        warp_sum9(v, red, threadIdx.x >> 5);
         __syncthreads();
         if (threadIdx.x < 9) {
             double t = 0;

@@ -73,6 +73,8 @@ struct PhysParams {
     float box_len_f[3];  // box_len as float (node tests run in FP32)
     float kr_f;          // support radius in units of h: 2 (M4) or 3 (M6)
     float coord_max;     // periodic: bound of the particles' and boxes' |coordinates|
+    double key_inv;      // periodic: Morton cells per unit length, 2^kMortonBits / largest box side
+    double box_hi[3];    // periodic: box_lo + box_len
     double kr;
     double box_inv[3];   // 1 / box_len (periodic), for minimum-image wraps
     float box_inv_f[3];
@@ -376,7 +378,8 @@ cudaError_t launch_domain_and_keys(const BatchView &b, cudaStream_t st);
 cudaError_t launch_radix_sort(const BatchView &b, cudaStream_t st);
 cudaError_t launch_gather(const BatchView &b, cudaStream_t st);
 cudaError_t launch_set_sorted_h(const BatchView &b, const double *h_in, cudaStream_t st);
-cudaError_t launch_build_leaves(const BatchView &b, int precision, cudaStream_t st);
+// after a sort; gather: with the gather of launch_gather
+cudaError_t launch_build_leaves(const BatchView &b, int precision, bool gather, cudaStream_t st);
 cudaError_t launch_update_leaves(const BatchView &b, int precision, cudaStream_t st);  // tree reuse
 cudaError_t launch_refit(const BatchView &b, int precision, cudaStream_t st);
 cudaError_t launch_density(const BatchView &b, int precision, int use_pred, cudaStream_t st);

@@ -242,7 +242,7 @@ __device__ __forceinline__ bool drift_one(const BatchView &b, long long g, long 
         double x = __dadd_rn(x0[a], __dmul_rn(vh[a], dk));
         if (ph.periodic) {
             const double lo = ph.box_lo[a], Lb = ph.box_len[a];
-            if (x >= lo + Lb) x -= Lb;
+            if (x >= ph.box_hi[a]) x -= Lb;
             else if (x < lo) x += Lb;
         }
         X[a][i] = x;

@@ -184,8 +184,7 @@ extern "C" int sph_density_forces_noalloc(const sph_params *p, int64_t n, const 
     NA_TRY(launch_reset_step(b, 1, st));
     NA_TRY(launch_domain_and_keys(b, st));
     NA_TRY(launch_radix_sort(b, st));
-    NA_TRY(launch_gather(b, st));
-    NA_TRY(launch_build_leaves(b, prec, st));
+    NA_TRY(launch_build_leaves(b, prec, true, st));
     NA_TRY(launch_density(b, prec, 0, st));
     NA_TRY(launch_refit(b, prec, st));
     NA_TRY(launch_forces(b, prec, st));

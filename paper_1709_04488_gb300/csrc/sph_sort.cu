@@ -180,22 +180,16 @@ __device__ __forceinline__ unsigned morton_key_code(const BatchView &b, int p, l
     const ProbStatic &ps = b.prob[p];
     const ProbDyn &d = b.dyn[p];
     long long i = g - ps.base;
-    double X[3] = {ps.x[i], ps.y[i], ps.z[i]};
-    double lo[3], inv;
-    if (ps.ph.periodic) {
-        double ext = fmax(ps.ph.box_len[0], fmax(ps.ph.box_len[1], ps.ph.box_len[2]));
-        for (int a = 0; a < 3; ++a) lo[a] = ps.ph.box_lo[a];
-        inv = 1.0 / ext;
-    } else {
-        for (int a = 0; a < 3; ++a) lo[a] = d.dom_lo[a];
-        inv = d.dom_inv;
-    }
+    const double X[3] = {ps.x[i], ps.y[i], ps.z[i]};
+    const double *lo = ps.ph.periodic ? ps.ph.box_lo : d.dom_lo;
+    // cells per unit length: the inverse extent times 2^kMortonBits (exact)
+    const double inv = ps.ph.periodic ? ps.ph.key_inv : d.dom_inv * (double)(1 << kMortonBits);
     unsigned code = 0;
     for (int a = 0; a < 3; ++a) {
-        double t = (X[a] - lo[a]) * inv * (double)(1 << kMortonBits);
-        int c = t > 0.0 ? (int)t : 0;  // NaN maps to 0
-        c = c > (1 << kMortonBits) - 1 ? (1 << kMortonBits) - 1 : c;
-        code |= spread10((unsigned)c) << a;
+        // (clamped as an integer: the conversion saturates, NaN gives the
+        // smallest integer, hence 0)
+        const int c = __double2int_rz((X[a] - lo[a]) * inv);
+        code |= spread10((unsigned)min(max(c, 0), (1 << kMortonBits) - 1)) << a;
     }
     return code;
 }
