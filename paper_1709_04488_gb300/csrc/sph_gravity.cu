@@ -320,6 +320,11 @@ __global__ void __launch_bounds__(256) k_gravity_reduce(BatchView b)
 // rounded outwards.
 // ---------------------------------------------------------------------------
 constexpr int kTreeThreads = 128;
+// (resident blocks; more would spill: 65536 particles 934 us with 4, 1007 with
+// 5.  The leaves are taken by tickets: with a fixed share per warp the walk
+// lasted as long as the warp with the two heaviest, 971 us, and 21.0 ms at 1e6
+// instead of 17.2)
+constexpr int kTreeBlocksPerSM = 4;
 constexpr int kTreeStage = 128;  // partner particles staged per warp at once
 
 __device__ __forceinline__ float4 ldcg4(const float4 *p) { return __ldcg(p); }
@@ -566,7 +571,7 @@ __device__ __forceinline__ void multipole_acc(T rx, T ry, T rz, T M, const T (&Q
 // per particle each lane takes every lpp-th staged entry and the lanes'
 // sums are added in a fixed order at the end.
 template <typename T>
-__global__ void __launch_bounds__(kTreeThreads) k_gravity_tree(BatchView b)
+__global__ void __launch_bounds__(kTreeThreads, sizeof(T) == 4 ? kTreeBlocksPerSM : 1) k_gravity_tree(BatchView b)
 {
     chain_entry();
     using V4 = typename Vec4<T>::type;
@@ -575,7 +580,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_gravity_tree(BatchView b)
     constexpr int kW = kTreeThreads / 32;
     __shared__ P s_p[kW][kTreeStage];  // partner (x, m) or node (com, M)
     __shared__ H s_h[kW][kTreeStage];  // partner (h, 1/h)
-    __shared__ T s_q[kW][32][6];       // node Q
+    __shared__ V4 s_q[kW][32][2];      // node Q
     __shared__ int s_off[kW][32], s_st[kW][32];  // opened leaves: first staged entry, first particle
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
     // the walk's query: a leaf (its box the opening criterion's), or in a
@@ -586,8 +591,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_gravity_tree(BatchView b)
     // the smaller boxes, and the walks multiply.)
     const bool blk = b.block_on && b.block_tasks;
     const int nitem = blk ? b.counters[kBlockTasks] : b.counters[0];
-    const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    for (int item = w0; item < nitem; item += nw) {
+    for (int item = first_item(); item < nitem; item = next_item(&b.counters[kGravTicket])) {
         int leaf = item, k0 = 0;
         if (blk) {
             const int t = b.btask[item];
@@ -669,20 +673,16 @@ __global__ void __launch_bounds__(kTreeThreads) k_gravity_tree(BatchView b)
                     e.z = A.z;
                     e.w = A.w;
                     s_p[wi][slot] = e;
-                    s_q[wi][slot][0] = B.x;
-                    s_q[wi][slot][1] = B.y;
-                    s_q[wi][slot][2] = B.z;
-                    s_q[wi][slot][3] = B.w;
-                    s_q[wi][slot][4] = C.x;
-                    s_q[wi][slot][5] = C.y;
+                    s_q[wi][slot][0] = B;
+                    s_q[wi][slot][1] = C;
                 }
                 __syncwarp();
                 const int nu = __popc(um);
                 if (pi < cnt) nnode += (nu - sub + lpp - 1) / lpp;
                 for (int e = sub; e < nu; e += lpp) {
                     const P q = s_p[wi][e];
-                    const T Q[6] = {s_q[wi][e][0], s_q[wi][e][1], s_q[wi][e][2],
-                                    s_q[wi][e][3], s_q[wi][e][4], s_q[wi][e][5]};
+                    const V4 qa = s_q[wi][e][0], qb = s_q[wi][e][1];
+                    const T Q[6] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y};
                     multipole_acc(xi - q.x, yi - q.y, zi - q.z, q.w, Q, mx, my, mz);
                 }
                 __syncwarp();
@@ -854,10 +854,10 @@ void launch_gravity(const BatchView &b, int precision, cudaStream_t st)
         if (!sms) sms = dev_info().sm_count;
         if (precision == SPH_PREC_FP64) {
             launch_chain(SPH_DEP(b), k_grav_moments<double>, sms * 8, 256, 0, st, b);
-            launch_chain(SPH_DEP(b), k_gravity_tree<double>, sms * 8, kTreeThreads, 0, st, b);
+            launch_chain(SPH_DEP(b), k_gravity_tree<double>, sms * 2, kTreeThreads, 0, st, b);
         } else {
             launch_chain(SPH_DEP(b), k_grav_moments<float>, sms * 8, 256, 0, st, b);
-            launch_chain(SPH_DEP(b), k_gravity_tree<float>, sms * 8, kTreeThreads, 0, st, b);
+            launch_chain(SPH_DEP(b), k_gravity_tree<float>, sms * kTreeBlocksPerSM, kTreeThreads, 0, st, b);
         }
     }
     if (b.ntot > 0) launch_chain(SPH_DEP(b), k_grav_dt, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b);

@@ -34,6 +34,7 @@ constexpr int kSlowCounter = 8, kPoolCounter = 9, kDensWrapList = 10, kForceWrap
 // per task costs more than the lanes save); 4 in FP64 (the lanes the FP64
 // kernels are built for)
 constexpr int kBlockTasks = 12, kBlockLanesF32 = 32, kBlockLanesF32Walk = 8, kBlockLanesF64 = 4;
+constexpr int kGravTicket = 13;  // gravity tree walk: tickets, cleared with the forces' counters
 constexpr int kDensityCounter = 16, kForceCounter = 32, kDensityWrapCounter = 40, kForceWrapCounter = 56,
               kForceCdCounter = 64;
 constexpr int kDensityClasses = 16, kForceClasses = 8;
@@ -451,8 +452,8 @@ __device__ __forceinline__ void reset_diag(const BatchView &b, int p, int mode)
 // mode 2 those of a forces-only call.
 __device__ __forceinline__ void reset_counter(const BatchView &b, int mode, int k)
 {
-    const bool all = (k >= kSlowCounter && k <= kForceWrapList) || k >= kTimeoutCounter;
-    const bool forces = k == kForceWrapList || k == kTimeoutCounter ||
+    const bool all = (k >= kSlowCounter && k <= kForceWrapList) || k == kGravTicket || k >= kTimeoutCounter;
+    const bool forces = k == kForceWrapList || k == kGravTicket || k == kTimeoutCounter ||
                         (k >= kForceCounter && k < kForceCounter + kForceClasses) ||
                         (k >= kForceWrapCounter && k < kForceWrapCounter + kForceClasses) ||
                         (k >= kForceCdCounter && k < kForceCdCounter + kForceClasses);
