@@ -320,11 +320,14 @@ __global__ void __launch_bounds__(256) k_gravity_reduce(BatchView b)
 // rounded outwards.
 // ---------------------------------------------------------------------------
 constexpr int kTreeThreads = 128;
-// (resident blocks; more would spill: 65536 particles 934 us with 4, 1007 with
-// 5.  The leaves are taken by tickets: with a fixed share per warp the walk
-// lasted as long as the warp with the two heaviest, 971 us, and 21.0 ms at 1e6
-// instead of 17.2)
-constexpr int kTreeBlocksPerSM = 4;
+// Resident blocks.  The leaves are taken by tickets (with a fixed share per
+// warp the walk lasted as long as the warp with the two heaviest); the node
+// visit and the direct sums have one call site each (with four and two the
+// kernel took 125 registers, four blocks) and are not unrolled, so that five
+// blocks fit.  Gravity stage at 65536 and 1e6 particles: fixed shares 971 us
+// and 21.0 ms, tickets 934 us and 17.2 ms, this 889 us and 15.7 ms (four
+// blocks 1011 us and 19.3 ms, unrolled twice 958 us and 15.9 ms).
+constexpr int kTreeBlocksPerSM = 5;
 constexpr int kTreeStage = 128;  // partner particles staged per warp at once
 
 __device__ __forceinline__ float4 ldcg4(const float4 *p) { return __ldcg(p); }
@@ -679,6 +682,7 @@ __global__ void __launch_bounds__(kTreeThreads, sizeof(T) == 4 ? kTreeBlocksPerS
                 __syncwarp();
                 const int nu = __popc(um);
                 if (pi < cnt) nnode += (nu - sub + lpp - 1) / lpp;
+#pragma unroll 1
                 for (int e = sub; e < nu; e += lpp) {
                     const P q = s_p[wi][e];
                     const V4 qa = s_q[wi][e][0], qb = s_q[wi][e][1];
@@ -717,46 +721,66 @@ __global__ void __launch_bounds__(kTreeThreads, sizeof(T) == 4 ? kTreeBlocksPerS
                 }
                 __syncwarp();
                 if (pi < cnt) npair += (nst - sub + lpp - 1) / lpp;
+#pragma unroll 1
                 for (int e = sub; e < nst; e += lpp) grav_pair(xi, yi, zi, T(1), hi, hinv, s_p[wi][e], s_h[wi][e], ax, ay, az);
                 __syncwarp();
             }
         };
-        const int top = d.top_level;
-        unsigned mask[kMaxLevels + 1];
-        int base[kMaxLevels + 1];
-        {
-            const unsigned om = visit((const V4 *)b.gnode[top] + 5LL * d.node_off[top], d.node_cnt[top], ~0u);
-            if (top == 0) direct(om, d.node_off[0]);
-            mask[top] = om;
-            base[top] = 0;
-        }
-        int lvl = top;
-        while (top > 0) {
-            const unsigned m = mask[lvl];
-            if (m == 0u) {
-                if (++lvl > top) break;
-                continue;
+        // depth first, one set of sibling nodes (or a level-1 node's groups of
+        // four leaves, or its leaves) at a time; the visit and the direct sums
+        // have one call site each, and the nodes still to open of each level
+        // are kept in the lanes, as in the pair kernels' walk
+        const int top = d.top_level, off0 = d.node_off[0];
+        unsigned m = 1u, sm = 0u;
+        int base = 0, sb = 0, lvl = top + 1, node = 0;
+        unsigned lf = 0u;  // leaves of the level-1 node `node` under its opened groups, to be visited next
+        for (;;) {
+            const V4 *set;
+            int count, kind;  // 0 nodes, 1 groups of leaves, 2 leaves
+            unsigned filter = ~0u;
+            if (lf) {
+                kind = 2;
+                set = (const V4 *)b.gnode[0] + 5LL * (off0 + node * kBranch);
+                count = min(kBranch, d.node_cnt[0] - node * kBranch);
+                filter = lf;
+                lf = 0u;
+            } else {
+                while (m == 0u && lvl <= top) {
+                    ++lvl;
+                    m = __shfl_sync(0xffffffffu, sm, lvl);
+                    base = __shfl_sync(0xffffffffu, sb, lvl);
+                }
+                if (m == 0u) break;
+                node = base + __ffs(m) - 1;
+                m &= m - 1u;
+                if (lvl == 1 && top > 0) {
+                    // a level-1 node's leaves: its groups of four first (used
+                    // whole where the criterion allows), then the leaves of the
+                    // groups it opens
+                    kind = 1;
+                    set = (const V4 *)b.ggrp + 40LL * (d.node_off[1] + node);
+                    count = (min(kBranch, d.node_cnt[0] - node * kBranch) + 3) >> 2;
+                } else {
+                    kind = lvl == 1 ? 2 : 0;  // (top level 0: its leaves)
+                    set = (const V4 *)b.gnode[lvl - 1] + 5LL * (d.node_off[lvl - 1] + node * kBranch);
+                    count = min(kBranch, d.node_cnt[lvl - 1] - node * kBranch);
+                }
             }
-            const int c = __ffs(m) - 1;
-            mask[lvl] = m & (m - 1u);
-            const int node = base[lvl] + c;
-            const int cnt_ch = min(kBranch, d.node_cnt[lvl - 1] - node * kBranch);
-            if (lvl == 1) {
-                // a level-1 node's leaves: its groups of four first (used
-                // whole where the criterion allows), then the leaves of the
-                // groups it opens
-                const unsigned og = visit((const V4 *)b.ggrp + 40LL * (d.node_off[1] + node), (cnt_ch + 3) >> 2, ~0u);
-                unsigned lf = 0u;
-                for (unsigned m = og; m; m &= m - 1u) lf |= 0xfu << (4 * (__ffs(m) - 1));
-                const unsigned om =
-                    lf ? visit((const V4 *)b.gnode[0] + 5LL * (d.node_off[0] + node * kBranch), cnt_ch, lf) : 0u;
-                direct(om, d.node_off[0] + node * kBranch);
-                continue;
+            const unsigned om = visit(set, count, filter);
+            if (kind == 2) {
+                direct(om, off0 + node * kBranch);
+            } else if (kind == 1) {
+                // bit k of om (a group) to bits 4k .. 4k + 3
+                lf = __ballot_sync(0xffffffffu, (om >> (lane >> 2)) & 1u);
+            } else if (om) {
+                if (lane == lvl) {
+                    sm = m;
+                    sb = base;
+                }
+                --lvl;
+                m = om;
+                base = node * kBranch;
             }
-            const unsigned om = visit((const V4 *)b.gnode[lvl - 1] + 5LL * (d.node_off[lvl - 1] + node * kBranch), cnt_ch, ~0u);
-            --lvl;
-            base[lvl] = node * kBranch;
-            mask[lvl] = om;
         }
         // the lanes of each particle add their sums in a fixed order
         double gx = (double)ax.s + (double)ax.c + (double)mx, gy = (double)ay.s + (double)ay.c + (double)my,
