@@ -88,42 +88,6 @@ __device__ __forceinline__ void grav_pair(T xi, T yi, T zi, T mi, T hi, T hinv_i
     az.add(-mul_rn(w, rz));
 }
 
-// Two FP32 values in one 64-bit register and the packed operations on them
-// (each half rounded as the scalar operation rounds it).
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 pack2(float a, float b)
-{
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(F2 x, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
-}
-__device__ __forceinline__ F2 operator+(F2 a, F2 b)
-{
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 operator*(F2 a, F2 b)
-{
-    F2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
-{
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-// a - b, rounded once: fma(b, -1, a)
-__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
-
 // TwoSumAcc of two particles at once
 struct TwoSumAcc2 {
     F2 s, c;

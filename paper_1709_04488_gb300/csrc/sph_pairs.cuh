@@ -62,6 +62,42 @@ __device__ __forceinline__ double tinf<double>() { return INFINITY; }
 __device__ __forceinline__ bool lt_pos(float a, float b) { return a < b; }
 __device__ __forceinline__ bool lt_pos(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 
+// Two FP32 values in one 64-bit register and the packed operations on them
+// (each half rounded as the scalar operation rounds it).
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float a, float b)
+{
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(F2 x, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 operator+(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+// a - b, rounded once: fma(b, -1, a)
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
+
 // Smoothing kernels of Sec. 2, W(r, h) = sigma f(q) / h^3 with q = r / h and
 // support q < R: fdf(q) gives f and f', df(q) f' alone.
 template <int K>
@@ -737,6 +773,33 @@ __device__ __forceinline__ int next_item(int *ticket)
     return (int)(gridDim.x * (blockDim.x >> 5)) + __shfl_sync(FULL, t, 0);
 }
 
+// The FP32 kernels' candidate buffer: NA arrays (the negated coordinates and
+// what else a test needs) of CH candidates, slot k in the section of the lanes
+// with k % LPP == sub, at place k / LPP.  A lane reads its section four
+// candidates at a time and tests them two at a time in packed operations:
+// about 8 instructions a candidate in place of 11, where every one of them
+// issues for the whole warp's union of neighbourhoods (density pass: cloud 1e6
+// 1.62 -> 1.42 ms, Sedov 64^3 237 -> 209 us, Sod 36864 63.9 -> 59.7 us).  Sections are padded by
+// four, for the sentinels behind the last candidate and to set their banks
+// apart.
+template <int CH, int LPP, int NA>
+struct CandBuf {
+    static constexpr int NARR = NA, SEC = (CH / LPP + 3) / 4 * 4 + 4;
+    static constexpr size_t bytes = sizeof(float) * NA * SEC * LPP;
+    float v[NA][SEC * LPP];
+    static __device__ __forceinline__ int place(int slot) { return slot % LPP * SEC + slot / LPP; }
+    // candidates of lane section `sub` among n
+    static __device__ __forceinline__ int mine(int n, int sub) { return (n - sub + LPP - 1) / LPP; }
+    // far points behind the last candidates, so that the tests take whole fours
+    __device__ __forceinline__ void pad(int n)
+    {
+        // (the square of their distance overflows to infinity; four, as a lane
+        // may go to the end of the longest section, one candidate beyond its own)
+        for (int t = threadIdx.x & 31; t < 4 * LPP; t += 32) v[0][t % LPP * SEC + mine(n, t % LPP) + t / LPP] = -3e38f;
+    }
+};
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
 template <typename T, int LPP, bool UM, int K>
 struct DCfg {
     using V = typename Vec4<T>::type;
@@ -759,7 +822,11 @@ struct DCfg {
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
     // (a row beyond the capacity takes the entries that no longer fit)
     static constexpr size_t lists = (size_t)(LCAP + 1) * 32 * LW * sizeof(T);
-    static constexpr size_t per_warp = CH * sizeof(float4) + lists + scratch + wait;
+    // (more lanes: too few candidates each for the fours to pay; M6: 96 registers, spills)
+    static constexpr bool PACK = !D64 && K == SPH_KERNEL_M4 && LPP <= 2;
+    using Cand = CandBuf<CH, LPP, UM ? 3 : 4>;      // (PACK: -x, -y, -z, m)
+    static constexpr size_t cands = PACK ? (Cand::bytes + 31) & ~(size_t)31 : CH * sizeof(float4);
+    static constexpr size_t per_warp = cands + lists + scratch + wait;
     static constexpr size_t smem = WPB * per_warp;
 };
 
@@ -952,12 +1019,14 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     using V = typename C::V;
     const int lane = threadIdx.x & 31;
     constexpr bool D64 = C::D64;
-    float4 *cand = reinterpret_cast<float4 *>(mine);
-    T *lr = reinterpret_cast<T *>(mine + C::CH * sizeof(float4));  // r_ij^2 per entry (FP64: r_ij)
+    constexpr bool PACK = C::PACK;
+    float4 *cand = reinterpret_cast<float4 *>(mine);                     // (not PACK)
+    typename C::Cand &cb = *reinterpret_cast<typename C::Cand *>(mine);  // (PACK)
+    T *lr = reinterpret_cast<T *>(mine + C::cands);  // r_ij^2 per entry (FP64: r_ij)
     T *lm = lr + (C::LCAP + 1) * 32;  // used only when masses differ
-    StageScratch<float> &sc = *reinterpret_cast<StageScratch<float> *>(mine + C::CH * sizeof(float4) + C::lists);
+    StageScratch<float> &sc = *reinterpret_cast<StageScratch<float> *>(mine + C::cands + C::lists);
     // FP64: the staged candidates' sorted indices, and the pairs that wait
-    int *code = reinterpret_cast<int *>(mine + C::CH * sizeof(float4) + C::lists + C::scratch), *lst = code + C::CH;
+    int *code = reinterpret_cast<int *>(mine + C::cands + C::lists + C::scratch), *lst = code + C::CH;
     const int pp = lane / LPP, sub = lane % LPP;
     const V *pm = (const V *)b.pm;
     const int p = b.leaf_pid[leaf];
@@ -1083,17 +1152,51 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             } else if (LPP == 1 || !bal) {
                 // (an entry beyond the capacity goes to the spare row: no
                 // branch on the append path)
-#pragma unroll 4
-                for (int k = sub; k < nbuf; k += LPP) {
-                    const float4 c = cand[k];
-                    float dx = pf.x - c.x, dyy = pf.y - c.y, dz = pf.z - c.z;
-                    if (wrap2) wrap3s<float>(sc, dx, dyy, dz);
-                    const float r2 = dx * dx + dyy * dyy + dz * dz;
+                const int nk = C::Cand::mine(nbuf, sub), at0 = sub * C::Cand::SEC;
+                auto append = [&](float r2, float mj) {
                     const int o = min(at, C::LCAP * 32 + lane);
                     if (r2 < R2t) {
                         lr[o] = r2;  // (its root where the lists are read: off the append path)
-                        if (!UM) lm[o] = c.w;
+                        if (!UM) lm[o] = mj;
                         at += 32;
+                    }
+                };
+                auto mass = [&](int k) { return UM ? 0.f : cb.v[C::Cand::NARR - 1][at0 + k]; };
+                // (r^2 in the same order of operations on every path of a launch)
+                auto dist2 = [](float dx, float dyy, float dz) {
+                    return WRAP ? fma_rn(dz, dz, fma_rn(dyy, dyy, mul_rn(dx, dx)))
+                                : fma_rn(dz, dz, fma_rn(dx, dx, mul_rn(dyy, dyy)));
+                };
+                if constexpr (!PACK) {
+#pragma unroll 4
+                    for (int k = sub; k < nbuf; k += LPP) {
+                        const float4 c = cand[k];
+                        float dx = pf.x - c.x, dyy = pf.y - c.y, dz = pf.z - c.z;
+                        if (wrap2) wrap3s<float>(sc, dx, dyy, dz);
+                        append(dist2(dx, dyy, dz), c.w);
+                    }
+                } else if (wrap2) {
+                    for (int k = 0; k < nk; ++k) {
+                        float dx = pf.x + cb.v[0][at0 + k], dyy = pf.y + cb.v[1][at0 + k], dz = pf.z + cb.v[2][at0 + k];
+                        wrap3s<float>(sc, dx, dyy, dz);
+                        append(dist2(dx, dyy, dz), mass(k));
+                    }
+                } else {
+                    cb.pad(nbuf);
+                    __syncwarp();
+                    const F2 px = pack2(pf.x, pf.x), py = pack2(pf.y, pf.y), pz = pack2(pf.z, pf.z);
+                    for (int k = 0; k < nk; k += 4) {
+                        const float4 x = ld4(cb.v[0] + at0 + k), y = ld4(cb.v[1] + at0 + k), z = ld4(cb.v[2] + at0 + k);
+#pragma unroll
+                        for (int h2 = 0; h2 < 2; ++h2) {
+                            const F2 dx = px + (h2 ? pack2(x.z, x.w) : pack2(x.x, x.y));
+                            const F2 dyy = py + (h2 ? pack2(y.z, y.w) : pack2(y.x, y.y));
+                            const F2 dz = pz + (h2 ? pack2(z.z, z.w) : pack2(z.x, z.y));
+                            float ra, rb;
+                            unpack2(fma2(dz, dz, WRAP ? fma2(dyy, dyy, dx * dx) : fma2(dx, dx, dyy * dyy)), ra, rb);
+                            append(ra, mass(k + 2 * h2));
+                            append(rb, mass(k + 2 * h2 + 1));
+                        }
                     }
                 }
             } else {
@@ -1103,13 +1206,19 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                     bool hit = false;
                     T r = T(0), mj = T(0);  // (r: r_ij^2)
                     if (k < nbuf) {
-                        const float4 c = cand[k];
-                        float dx = pf.x - c.x, dyy = pf.y - c.y, dz = pf.z - c.z;
+                        float4 q;
+                        if constexpr (PACK) {
+                            const int c = C::Cand::place(k);
+                            q = make_float4(-cb.v[0][c], -cb.v[1][c], -cb.v[2][c], UM ? 0.f : cb.v[C::Cand::NARR - 1][c]);
+                        } else {
+                            q = cand[k];
+                        }
+                        float dx = pf.x - q.x, dyy = pf.y - q.y, dz = pf.z - q.z;
                         if (wrap2) wrap3s<float>(sc, dx, dyy, dz);
                         const float r2 = dx * dx + dyy * dyy + dz * dz;
                         hit = r2 < R2t;
                         r = r2;
-                        mj = c.w;
+                        mj = q.w;
                     }
                     const unsigned gm = (__ballot_sync(FULL, hit) >> (pp * LPP)) & (LPP == 32 ? FULL : (1u << (LPP & 31)) - 1u);
                     if (hit) {
@@ -1178,8 +1287,16 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                     return box_dist2<float>(q, flo, fhi) < Rq2;
                 },
                 [&](int slot, const float4 &q, int, int) {
-                    cand[slot] = q;
-                    if (D64) code[slot] = __float_as_int(q.w);
+                    if constexpr (!PACK) {
+                        cand[slot] = q;
+                        if (D64) code[slot] = __float_as_int(q.w);
+                    } else {
+                        const int c = C::Cand::place(slot);
+                        cb.v[0][c] = -q.x;
+                        cb.v[1][c] = -q.y;
+                        cb.v[2][c] = -q.z;
+                        if (!UM) cb.v[C::Cand::NARR - 1][c] = q.w;
+                    }
                 },
                 flush);
         }
@@ -1605,10 +1722,17 @@ struct FCfg {
     static constexpr int WPB = D64 ? 2 : 4;
     static constexpr int MINB = D64 ? 4 : K == SPH_KERNEL_M6 ? SPH_MINB_M6 : LPP == 1 ? SPH_FORCE_MINB1 : SPH_FORCE_MINB;  // blocks per SM the registers allow
     using Code = std::conditional_t<D64, int, unsigned short>;  // (FP64: the sorted index itself)
-    static_assert(TAB <= 2048 && LC >= 2 * SB / LPP, "force list layout");
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
-    static constexpr size_t codes = ((size_t)(CH + LC * 32) * sizeof(Code) + 31) & ~(size_t)31;
-    static constexpr size_t per_warp = (CH + TAB) * sizeof(float4) + scratch + codes;
+    // (two lanes per particle: Sod 36864 71.7 -> 67.6 us; at one, where five
+    // blocks leave 96 registers, the packed form was 10 % slower)
+    static constexpr bool PACK = !D64 && K == SPH_KERNEL_M4 && LPP == 2;
+    using Cand = CandBuf<CH, LPP, 4>;  // (PACK: -x, -y, -z, 1/h)
+    static constexpr int NCODE = PACK ? Cand::SEC * LPP : CH;  // (codes are placed as the candidates)
+    static constexpr size_t cands = PACK ? (Cand::bytes + 31) & ~(size_t)31 : CH * sizeof(float4);
+    static constexpr size_t codes = ((size_t)(NCODE + LC * 32) * sizeof(Code) + 31) & ~(size_t)31;
+    static_assert(TAB <= 2048 && LC >= 2 * SB / LPP, "force list layout");
+    static_assert(!PACK || SB / LPP % 4 == 0, "the tests take whole fours between room checks");
+    static constexpr size_t per_warp = cands + TAB * sizeof(float4) + scratch + codes;
     static constexpr size_t smem = WPB * per_warp;
 };
 
@@ -1670,12 +1794,14 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     using V = typename C::V;
     const int lane = threadIdx.x & 31;
     constexpr bool D64 = C::D64;
+    constexpr bool PACK = C::PACK;
     float4 *cand = reinterpret_cast<float4 *>(mine);  // staged (offset + leaf shift, 1/h; FP64: R_K h)
-    float4 *table = cand + C::CH;                     // per candidate leaf: (leaf shift, first sorted index)
+    typename C::Cand &cb = *reinterpret_cast<typename C::Cand *>(mine);   // (PACK)
+    float4 *table = reinterpret_cast<float4 *>(mine + C::cands);  // per candidate leaf: (leaf shift, first sorted index)
     StageScratch<float> &sc = *reinterpret_cast<StageScratch<float> *>(table + C::TAB);
     using Code = typename C::Code;
-    Code *code = reinterpret_cast<Code *>(mine + (C::CH + C::TAB) * sizeof(float4) + C::scratch);
-    Code *lst = code + C::CH;
+    Code *code = reinterpret_cast<Code *>(mine + C::cands + C::TAB * sizeof(float4) + C::scratch);
+    Code *lst = code + C::NCODE;
     const int pp = lane / LPP, sub = lane % LPP;
     const V *gph = (const V *)b.ph, *gvc = (const V *)b.vc, *gth = (const V *)b.th;
     const int p = b.leaf_pid[leaf];
@@ -1861,6 +1987,41 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     auto test = [&]() {
         __syncwarp();  // staged candidates visible to every lane
         const int self = tA >= 0 ? ((tA << 5) | pos) : -1;
+        if constexpr (PACK) {
+            if (!wrap2) {
+                cb.pad(nbuf);
+                __syncwarp();
+                const F2 px = pack2(xf.x, xf.x), py = pack2(xf.y, xf.y), pz = pack2(xf.z, xf.z);
+                const int nk = C::Cand::mine(nbuf, 0), at0 = sub * C::Cand::SEC;
+                for (int kb = 0; kb < nk; kb += C::SB / LPP) {
+                    if (__any_sync(FULL, cnt > C::LC - C::SB / LPP)) eval_lists();
+                    const int ke = min(kb + C::SB / LPP, nk);
+                    for (int k = kb; k < ke; k += 4) {
+                        const float4 x = ld4(cb.v[0] + at0 + k), y = ld4(cb.v[1] + at0 + k), z = ld4(cb.v[2] + at0 + k),
+                                     w = ld4(cb.v[3] + at0 + k);
+                        const uint2 c4 = *reinterpret_cast<const uint2 *>(code + at0 + k);
+#pragma unroll
+                        for (int h2 = 0; h2 < 2; ++h2) {
+                            const F2 rx = px + (h2 ? pack2(x.z, x.w) : pack2(x.x, x.y));
+                            const F2 ry = py + (h2 ? pack2(y.z, y.w) : pack2(y.x, y.y));
+                            const F2 rz = pz + (h2 ? pack2(z.z, z.w) : pack2(z.x, z.y));
+                            const float wa = h2 ? w.z : w.x, wb = h2 ? w.w : w.y;
+                            const F2 hm = pack2(xf.w < wa ? xf.w : wa, xf.w < wb ? xf.w : wb);
+                            float ta, tb;
+                            unpack2((fma2(rz, rz, fma2(rx, rx, ry * ry)) * hm) * hm, ta, tb);
+                            const unsigned cc = h2 ? c4.y : c4.x;
+                            const int ca = (int)(cc & 0xffffu), cd = (int)(cc >> 16);
+                            if (active && ca != self && ta < (float)(KF::R * KF::R)) lst[cnt++ * 32 + lane] = (Code)ca;
+                            if (active && cd != self && tb < (float)(KF::R * KF::R)) lst[cnt++ * 32 + lane] = (Code)cd;
+                        }
+                    }
+                }
+                tested += (nbuf - sub + LPP - 1) / LPP;
+                __syncwarp();
+                nbuf = 0;
+                return;
+            }
+        }
         for (int k0 = 0; k0 < nbuf; k0 += C::SB) {
             const int ke = k0 + C::SB < nbuf ? k0 + C::SB : nbuf;
             if constexpr (D64) {
@@ -1894,12 +2055,20 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
             if (__any_sync(FULL, cnt > C::LC - C::SB / LPP)) eval_lists();
 #pragma unroll 4
             for (int k = k0 + sub; k < ke; k += LPP) {
-                const float4 c = cand[k];
+                float4 c;
+                int cd;
+                if constexpr (PACK) {
+                    const int at = C::Cand::place(k);
+                    c = make_float4(-cb.v[0][at], -cb.v[1][at], -cb.v[2][at], cb.v[3][at]);
+                    cd = code[at];
+                } else {
+                    c = cand[k];
+                    cd = code[k];
+                }
                 float rx = xf.x - c.x, ry = xf.y - c.y, rz = xf.z - c.z;
                 if (wrap2) wrap3s<float>(sc, rx, ry, rz);
                 const float r2 = rx * rx + ry * ry + rz * rz;
                 const float hm = xf.w < c.w ? xf.w : c.w;
-                const int cd = code[k];
                 if (active && cd != self && r2 * hm * hm < (float)(KF::R * KF::R))
                     lst[cnt++ * 32 + lane] = (Code)cd;
             }
@@ -1962,8 +2131,18 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
                     return d2 < RA2 || d2 * q.w * q.w < (float)(KF::R * KF::R * 1.0001);
                 },
                 [&](int slot, const float4 &q, int o, int idx) {
-                    cand[slot] = q;
-                    code[slot] = (Code)(D64 ? jq : (((ntab + o) << 5) | idx));
+                    const Code cd = (Code)(D64 ? jq : (((ntab + o) << 5) | idx));
+                    if constexpr (PACK) {
+                        const int at = C::Cand::place(slot);
+                        cb.v[0][at] = -q.x;
+                        cb.v[1][at] = -q.y;
+                        cb.v[2][at] = -q.z;
+                        cb.v[3][at] = q.w;
+                        code[at] = cd;
+                    } else {
+                        cand[slot] = q;
+                        code[slot] = cd;
+                    }
                 },
                 test);
             ntab += __popc(mask);
