@@ -88,17 +88,6 @@ __device__ __forceinline__ void grav_pair(T xi, T yi, T zi, T mi, T hi, T hinv_i
     az.add(-mul_rn(w, rz));
 }
 
-// TwoSumAcc of two particles at once
-struct TwoSumAcc2 {
-    F2 s, c;
-    __device__ __forceinline__ void add(F2 x)
-    {
-        const F2 t = s + x, xp = t - s, sp = t - xp;
-        c = c + ((s - sp) + (x - xp));
-        s = t;
-    }
-};
-
 // The sums of the two particles of a thread over staged partners.  pair()
 // is grav_pair for both, operation for operation (FP32: in packed
 // arithmetic, which halves the instructions of a kernel whose bound is their

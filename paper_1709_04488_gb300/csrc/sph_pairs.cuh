@@ -1753,6 +1753,54 @@ struct TwoSumAcc {
     }
 };
 
+// two TwoSumAcc at once (packed FP32)
+struct TwoSumAcc2 {
+    F2 s, c;
+    __device__ __forceinline__ void add(F2 x)
+    {
+        const F2 t = s + x, xp = t - s, sp = t - xp;
+        c = c + ((s - sp) + (x - xp));
+        s = t;
+    }
+};
+
+template <typename T>
+struct ForceSum {
+    TwoSumAcc<T> x{T(0), T(0)}, y{T(0), T(0)}, z{T(0), T(0)};
+    __device__ __forceinline__ void add(T w, T rx, T ry, T rz)
+    {
+        x.add(mul_rn(w, rx));
+        y.add(mul_rn(w, ry));
+        z.add(mul_rn(w, rz));
+    }
+    __device__ __forceinline__ void get(double &fx, double &fy, double &fz) const
+    {
+        fx = (double)x.s + (double)x.c;
+        fy = (double)y.s + (double)y.c;
+        fz = (double)z.s + (double)z.c;
+    }
+};
+template <>
+struct ForceSum<float> {
+    TwoSumAcc2 xy;
+    TwoSumAcc<float> z{0.f, 0.f};
+    __device__ __forceinline__ ForceSum() : xy{pack2(0.f, 0.f), pack2(0.f, 0.f)} {}
+    __device__ __forceinline__ void add(float w, float rx, float ry, float rz)
+    {
+        xy.add(pack2(w, w) * pack2(rx, ry));
+        z.add(mul_rn(w, rz));
+    }
+    __device__ __forceinline__ void get(double &fx, double &fy, double &fz) const
+    {
+        float s[2], c[2];
+        unpack2(xy.s, s[0], s[1]);
+        unpack2(xy.c, c[0], c[1]);
+        fx = (double)s[0] + (double)c[0];
+        fy = (double)s[1] + (double)c[1];
+        fz = (double)z.s + (double)z.c;
+    }
+};
+
 // conductivity signal speed (Sec. 2.1.1): Wadsley |v_ij . r_hat| (gm1 = 0)
 // or Price sqrt(|P_i - P_j| / rho_bar), P = gm1 rho u from the staged
 // (A, rho, m, u) vectors
@@ -1864,7 +1912,9 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     if (blk && !__any_sync(FULL, due)) return true;  // no particle of this leaf ends its step now
     const T lgap = (T)ph.block_gap;
     T mlev = T(0);
-    TwoSumAcc<T> ax{T(0), T(0)}, ay{T(0), T(0)}, az{T(0), T(0)};
+    // the sums of m_i a_i; x and y together in packed FP32 (additions only, so
+    // the same bits)
+    ForceSum<T> acc;
     T du = T(0), vs = T(-1);
     int pairs = 0, tested = 0;
     const float R = __fmul_ru(KR_f, boxA.plo.w) * 1.0001f;
@@ -1964,9 +2014,7 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
             const T visc = mul_rn(mul_rn(mul_rn(al, vsig), mu), rhob_inv);
             const T S = fma_rn(visc, gbar, -pterm);
             const T wgt = mul_rn(mul_rn(mul_rn(ti.z, a2.z), S), rinv);
-            ax.add(mul_rn(wgt, rx));
-            ay.add(mul_rn(wgt, ry));
-            az.add(mul_rn(wgt, rz));
+            acc.add(wgt, rx, ry, rz);
             if (adi)
                 du += a2.z * (ti.x * vdr * gi +
                               rhob_inv * gbar * (T(-0.5) * al * vsig * mu * mu + aac * ac_speed(vdr, ti, a2, gm1_price, rhob_inv) * (ti.w - a2.w)));
@@ -2199,7 +2247,8 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     eval_lists();
     if (!WRAP && to_wrap) return false;
     // combine the lanes of each particle; FP64 for the compensated sums
-    double Fx = (double)ax.s + (double)ax.c, Fy = (double)ay.s + (double)ay.c, Fz = (double)az.s + (double)az.c;
+    double Fx, Fy, Fz;
+    acc.get(Fx, Fy, Fz);
     Fx = group_sum<LPP>(Fx);
     Fy = group_sum<LPP>(Fy);
     Fz = group_sum<LPP>(Fz);
