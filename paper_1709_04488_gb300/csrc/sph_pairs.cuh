@@ -966,9 +966,10 @@ __device__ __forceinline__ void presolve_f32(const T *lr, const T *lm, int cnt, 
 {
     using KF = Kern<K>;
     const int lane = threadIdx.x & 31;
-    const float m = (float)mi, e3 = (float)eta3, sigma = (float)KF::sigma, mu = (float)mu_all;
+    // the zero is that of S0 - g: one rounding for the constants
+    const float g = (float)(mi * eta3 / T(KF::sigma)), mu = (float)mu_all;
     const float h0 = (float)h, hlim = fminf(1.25f * h0, (float)hs * 0.9999f);
-    float x = h0;
+    float x = h0, xi_last = 1.f, d_last = 0.f;
     bool go = on, moved = false;
     for (int it = 0; it < 6 && __any_sync(FULL, go); ++it) {
         float S0 = 0.f, S1 = 0.f;
@@ -985,10 +986,9 @@ __device__ __forceinline__ void presolve_f32(const T *lr, const T *lm, int cnt, 
         S0 = group_sum<LPP>(S0);
         S1 = group_sum<LPP>(S1);
         if (go) {
-            const float x3 = xi * xi * xi;
-            const float F = sigma * S0 * x3 - m * e3 * x3;
-            const float dF = -sigma * x3 * xi * (3.f * S0 + S1) + 3.f * m * e3 * x3 * xi;
-            const float xn = dF > 0.f ? x - F / dF : -1.f;
+            const float F = S0 - g;
+            const float dF = xi * (3.f * (g - S0) - S1);
+            const float d = F / dF, xn = dF > 0.f ? x - d : -1.f;
             const float step = fabsf(xn - x);
             if (!(xn >= 0.8f * h0) || !(xn <= hlim)) {
                 go = moved = false;
@@ -997,11 +997,16 @@ __device__ __forceinline__ void presolve_f32(const T *lr, const T *lm, int cnt, 
             } else {
                 go = step >= 1e-6f * x;
                 x = xn;
+                xi_last = xi;
+                d_last = d;
                 moved = true;
             }
         }
     }
-    if (moved) h = (T)x;
+    // the last step from the 1/h that the sums used, unrounded: what is left
+    // is the sums' rounding (rounding 1/h, h and three constants to FP32 left
+    // 1e-14 in h after one FP64 pass, twice that of a longer FP64 iteration)
+    if (moved) h = T(1) / (T)xi_last - (T)d_last;
 }
 
 // One query leaf of the density pass.  WRAP: pair vectors are wrapped to
