@@ -431,7 +431,7 @@ int sph_server_destroy(sph_server *s);
  *     which every GPU that loads the library holds until the process exits.
  *   - n is at most 32768, whatever the options (precision, kernel,
  *     self-gravity by direct sum or tree walk; the FP64 tree walk's layout,
- *     the largest, takes about 22 MiB); larger n returns SPH_EINVAL with a
+ *     the largest, takes 23.7 MiB); larger n returns SPH_EINVAL with a
  *     message.  (A layout that did not fit would return SPH_ENOSPACE, before
  *     touching the device, naming the largest n that fits.)
  *   - The caller passes the particle arrays (inputs and outputs as in
