@@ -280,6 +280,13 @@ PhysParams phys_of(const sph_params *p)
     if (p->periodic) {
         const double ext = std::fmax(p->box_len[0], std::fmax(p->box_len[1], p->box_len[2]));
         ph.key_inv = 1.0 / ext * (double)(1 << kMortonBits);
+        ph.unit = frame_unit(ext);
+        ph.frame_max = (float)(2.0 * ext * ph.unit);
+        if (p->precision == SPH_PREC_FP64)  // (the walk's frame)
+            for (int a = 0; a < 3; ++a) {
+                ph.box_len_f[a] = (float)(ph.box_len[a] * ph.unit);
+                ph.box_inv_f[a] = 1.0f / ph.box_len_f[a];
+            }
         for (int a = 0; a < 3; ++a) ph.box_hi[a] = p->box_lo[a] + p->box_len[a];
     }
     if (p->periodic)
@@ -572,7 +579,7 @@ static int enqueue_density(const BatchView &b, int precision, int use_pred, cuda
     CU(launch_density(b, precision, use_pred, st));
     mk.at(SPH_STAGE_REFIT, st);
     mk.done(SPH_STAGE_DENSITY);
-    CU(launch_refit(b, precision, st));
+    CU(launch_refit(b, st));
     mk.at(SPH_STAGE_FORCES, st);
     mk.done(SPH_STAGE_REFIT);
     return SPH_OK;
@@ -691,7 +698,7 @@ static int enqueue_block_passes(const BatchView &b, int prec, int L, bool use_co
                                 cudaGraphConditionalHandle fin, cudaStream_t st)
 {
     CU(launch_density(b, prec, 1, st));  // solves the particles whose step ends
-    CU(launch_refit(b, prec, st));
+    CU(launch_refit(b, st));
     CU(launch_forces(b, prec, st));
     launch_gravity(b, prec, st);  // the long range of the active particles
     CU(cudaGetLastError());
@@ -1140,9 +1147,9 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     CU(launch_domain_and_keys(b, st));
     CU(launch_radix_sort(b, st));
     CU(launch_build_leaves(b, c->prm.precision, true, st));
-    CU(launch_set_sorted_h(b, h_in, st));
-    CU(launch_refit(b, c->prm.precision, st));
-    CU(launch_neighbour_export(b, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
+    CU(launch_set_sorted_h(b, c->prm.precision, h_in, st));
+    CU(launch_refit(b, st));
+    CU(launch_neighbour_export(b, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
     CU(cudaStreamSynchronize(st));
     long long tot = 0;
     CU(cudaMemcpy(&tot, b.scratch64, sizeof tot, cudaMemcpyDeviceToHost));

@@ -316,7 +316,6 @@ __global__ void k_leaf_props(BatchView b)
 // in FP32 from the staged offsets and the float h (rounded up) the density
 // solve left, widened for the offsets' rounding, plus the reference point
 // rounded down (up) that the leaf pass kept.
-template <typename T4>
 __global__ void k_leaf_refit(BatchView b)
 {
     chain_entry();
@@ -334,8 +333,8 @@ __global__ void k_leaf_refit(BatchView b)
         const float kr = ph.kr_f;
         float slo[3], shi[3], hm = 0.f, ex[3] = {0.f, 0.f, 0.f};
         if (on) {
-            const T4 v = ((const T4 *)b.pm)[st + lane];
-            const float o[3] = {offset_f(v.x), offset_f(v.y), offset_f(v.z)};
+            const float4 v = b.pmf[st + lane];
+            const float o[3] = {v.x, v.y, v.z};
             const float h = b.hf[st + lane], h2 = __fmul_ru(kr, h);
             hm = h;
             for (int a = 0; a < 3; ++a) ex[a] = fabsf(o[a]);
@@ -430,12 +429,10 @@ cudaError_t launch_update_leaves(const BatchView &b, int precision, cudaStream_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_refit(const BatchView &b, int precision, cudaStream_t st)
+cudaError_t launch_refit(const BatchView &b, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
-    int pb = persistent_blocks(256);
-    if (precision == SPH_PREC_FP64) launch_chain(SPH_DEP(b), k_leaf_refit<dbl4>, pb, 256, 0, st, b);
-    else launch_chain(SPH_DEP(b), k_leaf_refit<float4>, pb, 256, 0, st, b);
+    launch_chain(SPH_DEP(b), k_leaf_refit, persistent_blocks(256), 256, 0, st, b);
     return cudaGetLastError();
 }
 

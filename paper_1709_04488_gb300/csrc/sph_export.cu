@@ -12,6 +12,7 @@ namespace {
 
 constexpr int kExportCap = 1024;  // neighbours one particle may have in the export
 
+template <bool F64>
 __global__ void k_set_sorted_h(BatchView b, const double *h_in)
 {
     chain_entry();
@@ -21,7 +22,7 @@ __global__ void k_set_sorted_h(BatchView b, const double *h_in)
     long long i = (long long)b.perm[s] - b.prob[p].base;
     const double h = h_in ? h_in[i] : b.prob[p].h[i];
     b.sh[s] = h;
-    b.hf[s] = __double2float_ru(h);
+    b.hf[s] = __double2float_ru(F64 ? h * frame_of(b.prob[p].ph, b.dyn[p]).unit : h);
 }
 
 // the membership test's own arithmetic (i, j: sorted indices)
@@ -45,12 +46,13 @@ __device__ __forceinline__ bool export_member(const BatchView &b, const PhysPara
 // per pass for 103823 particles; this form: 94-114 us.)  The pairs found wait in
 // a short list per lane, so that the lanes write them together.
 // FILL false: counts into cnt[i]; true: ids, in any order, at offsets[i].
+// F64: an FP64 problem, whose FP32 copies are in the walk's frame.
 struct ExportCfg {
     static constexpr int CH = 64, LC = 32, SB = 16, WPB = 4;
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
     static constexpr size_t per_warp = CH * (sizeof(float4) + sizeof(int)) + (size_t)LC * 32 * sizeof(int) + scratch;
 };
-template <bool FILL>
+template <bool FILL, bool F64>
 __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, int kind, unsigned *cnt,
                                                                 const long long *offsets, int *idx, long long cap)
 {
@@ -70,7 +72,9 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
     const int lpp = ps.lpp, pp = lane / lpp, sub = lane % lpp;
     // bound of a staged coordinate's error: each of the two offsets and the
     // shift rounded once, the sums once more
-    const float err = 1e-6f * (ph.periodic ? ph.coord_max : d.coord_max) + 1e-30f;
+    const double unit = F64 ? frame_of(ph, d).unit : 1.0;
+    const float cmax = F64 ? frame_of(ph, d).max : ph.periodic ? ph.coord_max : d.coord_max;
+    const float err = 1e-6f * cmax + 1e-30f;
     const int nleaf = b.counters[0];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (int leaf = w; leaf < nleaf; leaf += nw) {
@@ -89,7 +93,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
         if (kind == 1) problem_top_max(b, d, Rall, extmax), Rall = __fmul_ru(ph.kr_f, Rall) * 1.0001f;
         if (ph.periodic) load_box(sc, ph, flo, fhi);
         const bool wrap2 = ph.periodic && half_width(flo, fhi) + Rall >= half_box(ph);
-        set_query(sc.qb, boxA.plo, boxA.phi, R, ph, d);
+        set_query(sc.qb, boxA.plo, boxA.phi, R, ph, cmax);
         int nbuf = 0, n = 0;
         const long long i = (long long)b.perm[s] - ps.base;
         const long long at = FILL ? offsets[i] : 0;
@@ -142,8 +146,8 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
             const bool in = (leaf_lanes(d.node_cnt[0], nd) >> lane) & 1u;
             const unsigned mask = __ballot_sync(FULL, node(b.nodes[0][first + (in ? lane : 0)]) && in);
             if (mask)
-                stage_group<float, C::CH>(
-                b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
+                stage_group<float, C::CH, F64>(
+                b, leaf, mask, first, ph, unit, nbuf, sc, [](bool, int, int, int, const float4 &) {},
                 [&](int jj) {
                     float4 q = b.pmf[jj];
                     q.w = __int_as_float(jj);
@@ -297,15 +301,16 @@ __global__ void __launch_bounds__(kScanThreads) k_offsets(const unsigned *cnt, l
 
 }  // namespace
 
-cudaError_t launch_set_sorted_h(const BatchView &b, const double *h_in, cudaStream_t st)
+cudaError_t launch_set_sorted_h(const BatchView &b, int precision, const double *h_in, cudaStream_t st)
 {
     if (b.ntot == 0) return cudaSuccess;
-    launch_chain(SPH_DEP(b), k_set_sorted_h, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b, h_in);
+    const auto kern = precision == SPH_PREC_FP64 ? k_set_sorted_h<true> : k_set_sorted_h<false>;
+    launch_chain(SPH_DEP(b), kern, (unsigned)((b.ntot + 255) / 256), 256, 0, st, b, h_in);
     return cudaGetLastError();
 }
 
-cudaError_t launch_neighbour_export(const BatchView &b, int kind, long long *offsets, int *idx, long long cap,
-                                    long long *total_dev, cudaStream_t st)
+cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind, long long *offsets, int *idx,
+                                    long long cap, long long *total_dev, cudaStream_t st)
 {
     if (b.ntot == 0) {
         cudaMemsetAsync(offsets, 0, sizeof(long long), st);
@@ -318,10 +323,13 @@ cudaError_t launch_neighbour_export(const BatchView &b, int kind, long long *off
     const long long n = b.ntot, share = (n + kScanBlocks - 1) / kScanBlocks;
     const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
                          ((share + kScanThreads - 1) / kScanThreads * kScanThreads));
-    launch_chain(SPH_DEP(b), k_export<false>, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
+    const bool f64 = precision == SPH_PREC_FP64;
+    const auto count = f64 ? k_export<false, true> : k_export<false, false>;
+    const auto fill = f64 ? k_export<true, true> : k_export<true, false>;
+    launch_chain(SPH_DEP(b), count, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
     launch_chain(SPH_DEP(b), k_count_sums, nb, kScanThreads, 0, st, cnt, n, part);
     launch_chain(SPH_DEP(b), k_offsets, nb, kScanThreads, 0, st, cnt, n, part, offsets, total_dev);
-    launch_chain(SPH_DEP(b), k_export<true>, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
+    launch_chain(SPH_DEP(b), fill, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
     launch_chain(SPH_DEP(b), k_export_sort, grid, 128, 0, st, b, offsets, idx, cap);
     launch_chain(SPH_DEP(b), k_export_cut, 1, 1024, 0, st, b, kind, offsets, idx, cap);
     return cudaGetLastError();

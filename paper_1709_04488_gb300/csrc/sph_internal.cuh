@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/sph.h"
 
@@ -74,6 +75,8 @@ struct PhysParams {
     float box_len_f[3];  // box_len as float (node tests run in FP32)
     float kr_f;          // support radius in units of h: 2 (M4) or 3 (M6)
     float coord_max;     // periodic: bound of the particles' and boxes' |coordinates|
+    float frame_max;     // periodic, FP64: the same in the walk's frame
+    double unit;         // periodic: the FP32 unit of an FP64 problem (see Frame)
     double key_inv;      // periodic: Morton cells per unit length, 2^kMortonBits / largest box side
     double box_hi[3];    // periodic: box_lo + box_len
     double kr;
@@ -143,7 +146,39 @@ struct ProbDyn {
     int node_cnt[kMaxLevels + 1];  // nodes per level (level 0 = leaves)
     int lists_stale;     // some leaf's final h exceeds what its recorded candidate groups cover
     float coord_max;     // isolated: bound of |coordinates| (twice those of the last sort's domain)
+    float frame_max;     // isolated, FP64: the same in the walk's frame
+    double unit;         // isolated: the FP32 unit of an FP64 problem (see Frame)
 };
+
+// The frame of the FP32 copies of an FP64 problem (boxes, leaf offsets, h,
+// reaches: what its walks stage and test): lengths from the corner of the key
+// domain, times the power of two that brings the domain's extent into [1, 2).
+// FP32 squares of the raw lengths overflow from 1.8e19 and underflow below
+// 1e-22, lengths that FP64 problems have (1 pc is 3.1e18 cm).  A power of two
+// rounds nothing, so the decisions of a problem do not depend on its unit of
+// length; and the rounding of the boxes is that of the extent, wherever the
+// domain lies.  (Mixed precision has the FP32 range throughout: its copies
+// are the raw lengths.)
+struct Frame {
+    double unit;
+    float max;  // bound of the |coordinates|, twice the extent (kept leaves: particles may drift)
+};
+__host__ __device__ inline double frame_unit(double ext)
+{
+    unsigned long long bits;
+    memcpy(&bits, &ext, sizeof bits);
+    const long long e = (long long)((bits >> 52) & 0x7ffull);
+    if (e == 0 || e == 0x7ff) return 1.0;  // (no extent, or none that is finite)
+    const long long u = 2046 - e;
+    const unsigned long long ub = (unsigned long long)(u < 1 ? 1 : u) << 52;
+    double r;
+    memcpy(&r, &ub, sizeof r);
+    return r;
+}
+__host__ __device__ inline Frame frame_of(const PhysParams &ph, const ProbDyn &d)
+{
+    return ph.periodic ? Frame{ph.unit, ph.frame_max} : Frame{d.unit, d.frame_max};
+}
 
 // 32-byte vector of four doubles (FP64 staging)
 struct __align__(32) dbl4 {
@@ -407,11 +442,11 @@ DevInfo dev_info();
 cudaError_t launch_domain_and_keys(const BatchView &b, cudaStream_t st);
 cudaError_t launch_radix_sort(const BatchView &b, cudaStream_t st);
 cudaError_t launch_gather(const BatchView &b, cudaStream_t st);
-cudaError_t launch_set_sorted_h(const BatchView &b, const double *h_in, cudaStream_t st);
+cudaError_t launch_set_sorted_h(const BatchView &b, int precision, const double *h_in, cudaStream_t st);
 // after a sort; gather: with the gather of launch_gather
 cudaError_t launch_build_leaves(const BatchView &b, int precision, bool gather, cudaStream_t st);
 cudaError_t launch_update_leaves(const BatchView &b, int precision, cudaStream_t st);  // tree reuse
-cudaError_t launch_refit(const BatchView &b, int precision, cudaStream_t st);
+cudaError_t launch_refit(const BatchView &b, cudaStream_t st);
 cudaError_t launch_density(const BatchView &b, int precision, int use_pred, cudaStream_t st);
 cudaError_t launch_forces(const BatchView &b, int precision, cudaStream_t st);
 void launch_gravity(const BatchView &b, int precision, cudaStream_t st);  // direct-sum self-gravity
@@ -448,7 +483,7 @@ cudaError_t launch_block_kick(const BatchView &b, int L, bool use_cond, cudaGrap
 cudaError_t launch_block_finish(const BatchView &b, cudaStream_t st);
 cudaError_t launch_kick_close(const BatchView &b, int do_kick, int forces_ran, cudaStream_t st);
 cudaError_t launch_reset_step(const BatchView &b, int mode, cudaStream_t st);  // mode 1 full, 2 forces only
-cudaError_t launch_neighbour_export(const BatchView &b, int kind, long long *offsets, int *idx,
+cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind, long long *offsets, int *idx,
                                     long long cap, long long *total_dev, cudaStream_t st);
 
 // Reset of one problem's per-call diagnostics: mode 1 a whole step's, mode 2

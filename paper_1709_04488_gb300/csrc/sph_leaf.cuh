@@ -92,9 +92,6 @@ __device__ __forceinline__ float axis_of(const float *v, int lane)
     return lane == 0 ? v[0] : lane == 1 ? v[1] : v[2];
 }
 
-__device__ __forceinline__ float offset_f(float v) { return v; }
-__device__ __forceinline__ float offset_f(double v) { return (float)v; }
-
 // Per-axis extents of a leaf's offsets from its reference point (e: this
 // lane's |offset| per axis), packed for the minimum-image test of the pair
 // kernels: 10 bits per axis in units of L_a / 2046, rounded up (1023: half
@@ -127,6 +124,8 @@ __device__ __forceinline__ void leaf_props_one(const BatchView &b, int leaf)
         const int st = b.leaf_start[leaf], cnt = b.leaf_start[leaf + 1] - st;
         const ProbStatic &ps = b.prob[b.leaf_pid[leaf]];
         const bool on = lane < cnt;
+        constexpr bool F64 = sizeof(T4) == sizeof(dbl4);  // the FP32 copies in the walk's frame
+        const double unit = F64 ? frame_of(ps.ph, b.dyn[b.leaf_pid[leaf]]).unit : 1.0;
         // reference point: the centre of the leaf's box (its first particle
         // shifted by the float midpoint of the offsets from it), so that the
         // offsets stay within half the leaf's width
@@ -151,13 +150,14 @@ __device__ __forceinline__ void leaf_props_one(const BatchView &b, int leaf)
             v.z = (decltype(v.z))d[2];
             v.w = ps.uniform_m ? (decltype(v.w))ps.m_uniform : (decltype(v.w))b.sm[st + lane];
             ((T4 *)b.pm)[st + lane] = v;
-            if (sizeof(v.x) == 8) b.pmf[st + lane] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
-            const float o[3] = {offset_f(v.x), offset_f(v.y), offset_f(v.z)};
+            const float o[3] = {F64 ? (float)(d[0] * unit) : (float)v.x, F64 ? (float)(d[1] * unit) : (float)v.y,
+                                F64 ? (float)(d[2] * unit) : (float)v.z};
+            if (F64) b.pmf[st + lane] = make_float4(o[0], o[1], o[2], (float)v.w);
             for (int a = 0; a < 3; ++a) ex[a] = fabsf(o[a]);
             // predicted smoothing spheres: 1.1 x the guessed h (the h the
             // density solve starts from); the force pass reuses the density
             // walk's candidates when no final h exceeds its prediction
-            hp = __fmul_ru(kHPredict, __double2float_ru(b.sh[st + lane]));
+            hp = __fmul_ru(kHPredict, __double2float_ru(F64 ? b.sh[st + lane] * unit : b.sh[st + lane]));
             const float h2 = __fmul_ru(ps.ph.kr_f, hp);  // support radius R_K h
             for (int a = 0; a < 3; ++a) {
                 lo[a] = widen_dn(o[a], fabsf(o[a]));
@@ -182,9 +182,10 @@ __device__ __forceinline__ void leaf_props_one(const BatchView &b, int leaf)
         const float ext = leaf_ext_bits(ex, ps.ph);
         float bl = 0.f, bh = 0.f, sl = 0.f, sh = 0.f;
         if (lane < 3) {
-            const double ca = lane == 0 ? c[0] : lane == 1 ? c[1] : c[2];
-            const float cd = __double2float_rd(ca), cu = __double2float_ru(ca);
+            double ca = lane == 0 ? c[0] : lane == 1 ? c[1] : c[2];
             b.leaf_c[3 * (long long)leaf + lane] = ca;
+            if (F64) ca = (ca - (ps.ph.periodic ? ps.ph.box_lo[lane] : b.dyn[b.leaf_pid[leaf]].dom_lo[lane])) * unit;
+            const float cd = __double2float_rd(ca), cu = __double2float_ru(ca);
             b.leaf_cf[6 * (long long)leaf + lane] = cd;
             b.leaf_cf[6 * (long long)leaf + 3 + lane] = cu;
             bl = __fadd_rd(cd, axis_of(lo, lane));

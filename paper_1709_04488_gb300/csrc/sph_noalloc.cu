@@ -186,7 +186,7 @@ extern "C" int sph_density_forces_noalloc(const sph_params *p, int64_t n, const 
     NA_TRY(launch_radix_sort(b, st));
     NA_TRY(launch_build_leaves(b, prec, true, st));
     NA_TRY(launch_density(b, prec, 0, st));
-    NA_TRY(launch_refit(b, prec, st));
+    NA_TRY(launch_refit(b, st));
     NA_TRY(launch_forces(b, prec, st));
     launch_gravity(b, prec, st);
     NA_TRY(cudaGetLastError());

@@ -250,8 +250,11 @@ __device__ __forceinline__ T Kern<SPH_KERNEL_M6>::df(T q)
 __device__ __forceinline__ float fast_div(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double fast_div(double a, double b) { return a / b; }
 
-__device__ __forceinline__ float to_float_ru(float v) { return v; }
-__device__ __forceinline__ float to_float_ru(double v) { return __double2float_ru(v); }
+// a length in the unit of the FP32 copies (FP64 problems: the walk's frame)
+__device__ __forceinline__ float frame_len(float v, double) { return v; }
+__device__ __forceinline__ float frame_len(double v, double unit) { return (float)(v * unit); }
+__device__ __forceinline__ float frame_len_ru(float v, double) { return v; }
+__device__ __forceinline__ float frame_len_ru(double v, double unit) { return __double2float_ru(v * unit); }
 
 // sorted particle index carried in the w slot of a staged vector: bit
 // pattern in FP32 staging (only ever copied), exact value in FP64 staging
@@ -278,8 +281,9 @@ struct QueryBox {
     // R for sure and above which it is not; s doubled; R^2 of the definition
     float in2, out2, s2, R2;
 };
+// cmax: bound of the problem's and its boxes' |coordinates|
 __device__ __forceinline__ void set_query(QueryBox &qb, const float4 &lo, const float4 &hi, float R, const PhysParams &ph,
-                                          const ProbDyn &d)
+                                          float cmax)
 {
     const int lane = threadIdx.x & 31;
     __syncwarp();
@@ -287,7 +291,7 @@ __device__ __forceinline__ void set_query(QueryBox &qb, const float4 &lo, const 
         const float l = lane == 0 ? lo.x : lane == 1 ? lo.y : lo.z, h = lane == 0 ? hi.x : lane == 1 ? hi.y : hi.z;
         qb.ax[lane] = make_float4(l + h, h - l, ph.periodic ? 2.f * ph.box_len_f[lane] : INFINITY, 0.f);
     } else if (lane == 3) {
-        const float s = 1e-5f * ((ph.periodic ? ph.coord_max : d.coord_max) + R) + 1e-29f;
+        const float s = 1e-5f * (cmax + R) + 1e-29f;
         const float in = 2.f * (R - 2.f * s), out = 2.f * (R + 2.f * s);
         qb.in2 = in > 0.f ? in * in : -1.f;
         qb.out2 = out * out;
@@ -609,11 +613,12 @@ __device__ __forceinline__ double min_image_bits(double d, double L, int periodi
     return d;
 }
 // shift of candidate leaf B's reference point from the query leaf A's: FP64
-// difference, minimum image, cast
-template <typename T>
-__device__ __forceinline__ T leaf_shift(double cb, double ca, double L, int periodic)
+// difference, minimum image, cast (SCALED: in units of 1 / unit)
+template <typename T, bool SCALED>
+__device__ __forceinline__ T leaf_shift(double cb, double ca, double L, int periodic, double unit)
 {
-    return (T)min_image_bits(cb - ca, L, periodic);
+    const double d = min_image_bits(cb - ca, L, periodic);
+    return SCALED ? (T)(d * unit) : (T)d;
 }
 
 // Stage the particles of the leaves first + k (bit k of mask) that keep()
@@ -629,9 +634,9 @@ __device__ __forceinline__ T leaf_shift(double cb, double ca, double L, int peri
 // that fall into the chunk, one bit each, gathered by one warp reduction
 // (a binary search over the first elements took five dependent shared-memory
 // reads per chunk).
-template <typename T, int CH, class Group, class Load, class Keep, class Store, class Flush>
+template <typename T, int CH, bool SCALED = false, class Group, class Load, class Keep, class Store, class Flush>
 __device__ __forceinline__ void stage_group(const BatchView &b, int A, unsigned mask, int first, const PhysParams &ph,
-                                            int &nbuf, StageScratch<T> &sc, Group &&group, Load &&load,
+                                            double unit, int &nbuf, StageScratch<T> &sc, Group &&group, Load &&load,
                                             Keep &&keep, Store &&store, Flush &&flush)
 {
     using V = typename Vec4<T>::type;
@@ -646,9 +651,9 @@ __device__ __forceinline__ void stage_group(const BatchView &b, int A, unsigned 
         stB = b.leaf_start[B];
         nB = b.leaf_start[B + 1] - stB;
         const double *cb = b.leaf_c + 3LL * B, *ca = b.leaf_c + 3LL * A;
-        D.x = leaf_shift<T>(cb[0], ca[0], ph.box_len[0], ph.periodic);
-        D.y = leaf_shift<T>(cb[1], ca[1], ph.box_len[1], ph.periodic);
-        D.z = leaf_shift<T>(cb[2], ca[2], ph.box_len[2], ph.periodic);
+        D.x = leaf_shift<T, SCALED>(cb[0], ca[0], ph.box_len[0], ph.periodic, unit);
+        D.y = leaf_shift<T, SCALED>(cb[1], ca[1], ph.box_len[1], ph.periodic, unit);
+        D.z = leaf_shift<T, SCALED>(cb[2], ca[2], ph.box_len[2], ph.periodic, unit);
     }
     group(has, first + lane, stB, ord, D);
     const int incl = warp_incl_scan<T>(nB);
@@ -874,7 +879,7 @@ __device__ __forceinline__ void task_box(const BatchView &b, int leaf, const V &
 template <typename T>
 __device__ __forceinline__ void density_epilogue(const BatchView &b, const ProbStatic &ps, long long s,
                                                  typename Vec4<T>::type pi, T h, T S0, T S1, int use_pred,
-                                                 T sigma, T Z = T(0))
+                                                 T sigma, double unit, T Z = T(0))
 {
     using V = typename Vec4<T>::type;
     const PhysParams &ph = ps.ph;
@@ -910,7 +915,7 @@ __device__ __forceinline__ void density_epilogue(const BatchView &b, const ProbS
     }
     T A = P / (omega * rho * rho);
     b.sh[s] = (double)h;
-    b.hf[s] = to_float_ru(h);
+    b.hf[s] = frame_len_ru(h, unit);
     b.srho[s] = (double)rho;
     b.somega[s] = (double)omega;
     b.sP[s] = (double)P;
@@ -1047,13 +1052,16 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     const V pi = pm[s];
     const float4 pf = b.pmf[s];  // (FP32: pi)
     const T mi = pi.w;
-    // FP64: bound of a staged coordinate's error (its offset and shift rounded
-    // once each, their sum once more), and the particle's position
-    const float err = D64 ? 1e-6f * (ps.ph.periodic ? ps.ph.coord_max : b.dyn[p].coord_max) + 1e-30f : 0.f;
+    // FP64: the walk's frame, the bound of a staged coordinate's error (its
+    // offset and shift rounded once each, their sum once more), and the
+    // particle's position
+    const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
+    const float cmax = D64 ? frame_of(ph, dy).max : ph.periodic ? ph.coord_max : dy.coord_max;
+    const float err = D64 ? 1e-6f * cmax : 0.f;
     const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles (the others
     // of the leaf keep their last solve, restaged by k_block_restage)
-    if (k0 >= 0) task_box(b, leaf, pi, active, boxA.plo.w, boxA);
+    if (k0 >= 0) task_box(b, leaf, pf, active, boxA.plo.w, boxA);
     float4 flo, fhi;
     frame_box<float4, float>(pf, active, flo, fhi);
     const float halfL = ph.periodic ? half_box(ph) : INFINITY;
@@ -1064,7 +1072,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     const T hbox = (T)(Lmin / (2.0 * KF::R));  // support beyond half the box: SPH_EBOX
     T h = active ? (T)b.sh[s] : T(1);
     // the leaf pass predicted this particle's sphere from the same start
-    const float hpred = active ? __fmul_ru(kHPredict, __double2float_ru(b.sh[s])) : 0.f;
+    const float hpred = active ? __fmul_ru(kHPredict, __double2float_ru(D64 ? b.sh[s] * unit : b.sh[s])) : 0.f;
     if (active && !(h > T(0))) {
         double ext = ph.periodic ? fmax(ph.box_len[0], fmax(ph.box_len[1], ph.box_len[2])) : 1.0 / dy.dom_inv;
         h = (T)(ph.eta * cbrt(ext * ext * ext / (double)(ps.n > 0 ? ps.n : 1)));
@@ -1092,7 +1100,8 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     float Rq_last = 0.f;
     for (int attempt = 0;; ++attempt) {
         const T hs = h * (T)kListMargin;
-        float Rq = warp_max((active && !fail) ? __fmul_ru(KR_f, (float)hs) : 0.f) * 1.0001f;
+        const float hsf = frame_len(hs, unit);
+        float Rq = warp_max((active && !fail) ? __fmul_ru(KR_f, hsf) : 0.f) * 1.0001f;
         const T R2 = (T(KF::R) * hs) * (T(KF::R) * hs);
         Rq_last = Rq;
         if (!D64 && ph.periodic) set_thr(sc, boxA.slo.w, Rq);
@@ -1100,7 +1109,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         ng = 0;
         cnt = 0;
         int gcnt = 0, at = lane;  // at: where this lane's next entry goes
-        const float Rs = KR_f * (float)hs;
+        const float Rs = KR_f * hsf;
         const float R2t = active && !fail ? D64 ? Rs * (Rs * 1.00002f + 8.f * err) + err * err : (float)R2 : -1.f;
         bool ovf = false;
         int nbuf = 0;
@@ -1244,7 +1253,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             nbuf = 0;
         };
         const float Rq2 = (Rq + 4.f * err) * (Rq + 4.f * err);
-        set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, dy);
+        set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, cmax);
         // visit leaves within Rq (gather) or whose predicted smoothing
         // spheres reach this leaf (what the force pass will need); stage
         // only the former
@@ -1279,8 +1288,8 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             if (!WRAP && am) to_wrap = true;
             if (!WRAP && to_wrap) break;
             const unsigned amo = WRAP ? by_order(am, gm) : 0u;
-            stage_group<float, C::CH>(
-                b, leaf, gm, first, ph, nbuf, sc, [](bool, int, int, int, const float4 &) {},
+            stage_group<float, C::CH, D64>(
+                b, leaf, gm, first, ph, unit, nbuf, sc, [](bool, int, int, int, const float4 &) {},
                 [&](int j) {
                     float4 q = b.pmf[j];
                     if (D64) q.w = __int_as_float(j);
@@ -1438,14 +1447,14 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         Z = group_sum<LPP>(Z);
     }
     if (fin && sub == 0) {
-        density_epilogue<T>(b, ps, s, pi, h, S0, S1, use_pred, sigma, Z);
+        density_epilogue<T>(b, ps, s, pi, h, S0, S1, use_pred, sigma, unit, Z);
         if (noconv && !(b.block_on && ((const T *)b.slev)[s] < T(0))) {  // (a kept solve is not this one)
             atomicOr(&ps.diag->status, ST_NOCONV);
             atomicAdd(&ps.diag->unconverged, 1);
         }
         // the recorded candidate groups cover this particle's pairs only
         // if its final h stays within the walk radius and its prediction
-        const float hf = to_float_ru(h);
+        const float hf = frame_len_ru(h, unit);
         if (hf > hpred || hf > Rq_last / KR_cap) atomicOr(&b.dyn[p].lists_stale, 1);
     }
     if (active && fail && sub == 0) {
@@ -1553,6 +1562,9 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
         const ProbDyn &dy = b.dyn[p];
         const PhysParams &ph = ps.ph;
         const NodeBox boxA = b.nodes[0][leaf];
+        constexpr bool D64 = sizeof(T) == 8;  // (the walk in its frame, the staged positions as they are)
+        const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
+        const float cmax = D64 ? frame_of(ph, dy).max : ph.periodic ? ph.coord_max : dy.coord_max;
         const V pi = pm[s];
         const T eta3 = (T)(ph.eta * ph.eta * ph.eta);
         const T tol = (T)ph.h_tol;
@@ -1568,11 +1580,12 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
         long long pairs = 0;
         T S0, S1;
         int nn;
-        // every particle within Rq of particle s, staged in groups of
-        // leaves; fn(r2, m_j) sees one candidate per lane
-        auto visit_all = [&](float Rq, auto &&fn) {
-            const T Rq2 = (T)Rq * (T)Rq;
-            set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, dy);
+        // every particle within the support R_K hh of particle s, staged in
+        // groups of leaves; fn(r2, m_j) sees one candidate per lane
+        auto visit_all = [&](T hh, auto &&fn) {
+            const float Rq = __fmul_ru(ph.kr_f, frame_len(hh, unit)) * 1.0001f;
+            const T Rt = D64 ? KR * hh * T(1.0001) : (T)Rq, Rq2 = Rt * Rt;
+            set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, cmax);
             int nbuf = 0;
             auto flush = [&]() {
                 __syncwarp();
@@ -1594,7 +1607,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
                 const unsigned mask = __ballot_sync(FULL, box_within(sc.qb, b.nodes[0][first + (in ? lane : 0)], ph) && in);
                 if (mask)
                     stage_group<T, kFbCH>(
-                        b, leaf, mask, first, ph, nbuf, sc, [](bool, int, int, int, const V &) {},
+                        b, leaf, mask, first, ph, unit, nbuf, sc, [](bool, int, int, int, const V &) {},
                         [&](int j) { return pm[j]; },
                         [&](V &q, int) {
                             if (per) wrap_near<T>(sc, q, pi.x, pi.y, pi.z);  // then pi - q is the minimum image
@@ -1612,7 +1625,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
             const T R2 = (KR * hs) * (KR * hs);
             cnt = 0;
             bool ovf = false;
-            visit_all(__fmul_ru(ph.kr_f, (float)hs) * 1.0001f, [&](T r2, T mj) {
+            visit_all(hs, [&](T r2, T mj) {
                 if (r2 < R2) {
                     if (cnt < kFbPerLane) {
                         fr[cnt * 32 + lane] = sqrt(r2);
@@ -1645,7 +1658,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
                 }
             } else {
                 const T R2 = (KR * hh) * (KR * hh);
-                visit_all(__fmul_ru(ph.kr_f, (float)hh) * 1.0001f, [&](T r2, T mj) {
+                visit_all(hh, [&](T r2, T mj) {
                     if (r2 < R2) {
                         T f, df, qq = sqrt(r2) * hinv;
                         kern_fdf(kk, qq, f, df);
@@ -1686,9 +1699,9 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
         sums(h);
         pairs += nn;
         if (lane == 0) {
-            const float hf = to_float_ru(h);
+            const float hf = frame_len_ru(h, unit);
             if (hf > b.hf[s] || hf > b.leaf_hcap[leaf]) atomicOr(&b.dyn[p].lists_stale, 1);
-            density_epilogue<T>(b, ps, s, pi, h, S0, S1, use_pred, sigma, Z);
+            density_epilogue<T>(b, ps, s, pi, h, S0, S1, use_pred, sigma, unit, Z);
             if (noconv) {
                 atomicOr(&ps.diag->status, ST_NOCONV);
                 atomicAdd(&ps.diag->unconverged, 1);
@@ -1876,11 +1889,13 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     } else {
         xf = xi;
     }
-    const float err = D64 ? 1e-6f * (ps.ph.periodic ? ps.ph.coord_max : b.dyn[p].coord_max) + 1e-30f : 0.f;
+    const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
+    const float cmax = D64 ? frame_of(ph, dy).max : ph.periodic ? ph.coord_max : dy.coord_max;
+    const float err = D64 ? 1e-6f * cmax : 0.f;
     const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles, whose
     // largest h sets the gather reach
-    if (k0 >= 0) task_box(b, leaf, xi, active, warp_max(active ? b.hf[s] : 0.f), boxA);
+    if (k0 >= 0) task_box(b, leaf, xf, active, warp_max(active ? b.hf[s] : 0.f), boxA);
     const T alpha = (T)ph.alpha_av, beta = (T)ph.beta_av, aac = (T)ph.alpha_ac;
     // Price conductivity: v'_sig = sqrt(|P_i - P_j| / rho_bar) with P = (gamma - 1) rho u
     // (adiabatic); 0 selects Wadsley's |v_ij . r_hat|
@@ -2130,7 +2145,7 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         __syncwarp();
         nbuf = 0;
     };
-    set_query(sc.qb, boxA.plo, boxA.phi, R, ph, dy);
+    set_query(sc.qb, boxA.plo, boxA.phi, R, ph, cmax);
     auto node_test = [&](const NodeBox &nb) {
         const bool near = box_within(sc.qb, nb, ph);
         return box_overlap(sc.qb, nb, ph) || near;
@@ -2150,8 +2165,8 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
             if (!WRAP && am) to_wrap = true;
             if (!WRAP && to_wrap) return;
             const unsigned amo = WRAP ? by_order(am, mask) : 0u;
-            stage_group<float, C::CH>(
-                b, leaf, mask, first, ph, nbuf, sc,
+            stage_group<float, C::CH, D64>(
+                b, leaf, mask, first, ph, unit, nbuf, sc,
                 [&](bool has, int B, int stB, int ord, const float4 &D) {
                     if (D64) return;
                     if (has) {
@@ -2427,7 +2442,8 @@ __device__ __forceinline__ void block_tasks_one(const BatchView &b, int leaf, in
     if (lane == 0 && nt > 0) base = atomicAdd(&b.counters[kBlockTasks], nt);
     base = __shfl_sync(FULL, base, 0);
     if (lane < nt) b.btask[base + lane] = (leaf << 5) | (lane * size);
-    if (lane < n && !due) density_epilogue<T>(b, b.prob[0], s, ((const V *)b.pm)[s], T(1), T(0), T(0), use_pred, T(0));
+    const double unit = sizeof(T) == 8 ? frame_of(b.prob[0].ph, b.dyn[0]).unit : 1.0;
+    if (lane < n && !due) density_epilogue<T>(b, b.prob[0], s, ((const V *)b.pm)[s], T(1), T(0), T(0), use_pred, T(0), unit);
 }
 
 // the tasks of a tick that built its leaves

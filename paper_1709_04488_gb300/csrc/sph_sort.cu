@@ -163,6 +163,8 @@ __global__ void k_domain(BatchView b)
         double cm = 0.0;
         for (int a = 0; a < 3; ++a) cm = fmax(cm, fabs(d.dom_lo[a]) + ext);
         d.coord_max = (float)(2.0 * cm);  // (kept leaves: particles may drift beyond the domain)
+        d.unit = frame_unit(ext);
+        d.frame_max = (float)(2.0 * ext * d.unit);
         ext = ext * (1.0 + 1e-9) + 1e-300;
     }
     d.dom_inv = ext > 0.0 ? 1.0 / ext : 1.0;

@@ -1,0 +1,98 @@
+"""A problem in another unit of length: every length times 2^k, masses,
+velocities and internal energies as they are.  A power of two rounds nothing,
+so each output of an FP64 problem is the unscaled one times its power of two,
+bit for bit, and the neighbour lists are the same lists.  (Squares of the
+lengths leave the range of FP32 at k = 70 and k = -80: 1.2e21 and 8e-25.)"""
+import numpy as np
+import pytest
+
+from paper_1709_04488_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+
+POWER = dict(x=1, y=1, z=1, vx=0, vy=0, vz=0, u=0, m=0, h=1, rho=-3, omega=0, P=-3, c=0, ax=-1, ay=-1, az=-1, du=-1, vsig=0)
+
+
+@pytest.fixture(scope="module")
+def S():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1709_04488_gb300 import build as b
+    b.build()
+    from paper_1709_04488_gb300 import sph
+    return sph
+
+
+def _problem(kind):
+    kw = {}
+    if kind == "thin":
+        a, p = ics.sod(left=(96, 12, 12), right=(48, 6, 6), length=0.75, width=0.09375, jitter=0.05)
+    elif kind == "isolated":
+        a, p = ics.cloud(2000, seed=6)
+        a["m"] = a["m"] * np.random.default_rng(1).uniform(0.9, 1.1, 2000)
+    else:
+        a, p = ics.lattice(12, seed=5)
+    if kind == "m6":
+        kw = dict(kernel=1, eta=1.0)
+        a["h"] = a["h"] / 1.2
+    if kind == "slow":  # first guesses that overflow the lists: the slow density path
+        a["h"] = a["h"] * 1.6
+    if kind == "block":
+        kw = dict(block_levels=2)
+    rng = np.random.default_rng(3)
+    for c in ("vx", "vy", "vz"):
+        a[c] = rng.normal(0.0, 0.3, len(a["x"]))
+    return a, p, kw
+
+
+def _scaled(a, p, s):
+    a, q = dict(a), dict(p)
+    for c in "xyzh":
+        a[c] = a[c] * s
+    if p["periodic"]:
+        q["box_lo"] = tuple(v * s for v in p["box_lo"])
+        q["box_len"] = tuple(v * s for v in p["box_len"])
+    return a, q
+
+
+@pytest.mark.parametrize("k", [70, -80])
+@pytest.mark.parametrize("kind", ["lattice", "thin", "isolated", "m6", "slow", "block"])
+def test_fp64_outputs_scale_exactly(S, kind, k):
+    a, p, kw = _problem(kind)
+    out = []
+    for s in (1.0, 2.0 ** k):
+        b, q = _scaled(a, p, s)
+        prob = S.Problem(b, S.make_params(S.PREC_FP64, **q, tree_rebuild_every=2, **kw))
+        prob.density_h()
+        prob.forces()
+        got = [prob.numpy(*POWER)]
+        if kind == "block":
+            prob.block_step()
+        else:
+            for _ in range(3):  # (leaves kept and built)
+                prob.step()
+        got.append(prob.numpy(*POWER))
+        d = prob.diagnostics()
+        out.append((got, d.ngb_min, d.ngb_max, d.force_pairs))
+        prob.close()
+    for g0, g1 in zip(out[0][0], out[1][0]):
+        for f, w in POWER.items():
+            assert np.array_equal(g1[f], np.ldexp(g0[f], w * k)), f
+    assert out[0][1:] == out[1][1:]
+
+
+@pytest.mark.parametrize("k", [70, -80])
+@pytest.mark.parametrize("kind", ["lattice", "thin", "isolated", "m6"])
+@pytest.mark.parametrize("prec", ["fp64"])
+def test_lists_do_not_depend_on_the_unit(S, kind, k, prec):
+    a, p, kw = _problem(kind)
+    lists = []
+    for s in (1.0, 2.0 ** k):
+        b, q = _scaled(a, p, s)
+        prob = S.Problem(b, S.make_params(S.PREC_FP64 if prec == "fp64" else S.PREC_MIXED, **q, **kw))
+        lists.append([t.cpu().numpy() for n in (0, 1) for t in prob.neighbours(n)])
+        prob.close()
+    assert len(lists[0][1]) > 20 * len(a["x"])
+    for x, y in zip(*lists):
+        assert np.array_equal(x, y)
