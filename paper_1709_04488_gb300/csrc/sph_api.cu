@@ -1149,7 +1149,8 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     CU(launch_build_leaves(b, c->prm.precision, true, st));
     CU(launch_set_sorted_h(b, c->prm.precision, h_in, st));
     CU(launch_refit(b, st));
-    CU(launch_neighbour_export(b, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap, b.scratch64, st));
+    CU(launch_neighbour_export(b, c->host_ps.ph, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap,
+                               b.scratch64, st));
     CU(cudaStreamSynchronize(st));
     long long tot = 0;
     CU(cudaMemcpy(&tot, b.scratch64, sizeof tot, cudaMemcpyDeviceToHost));

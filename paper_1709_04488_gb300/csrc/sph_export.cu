@@ -46,13 +46,20 @@ __device__ __forceinline__ bool export_member(const BatchView &b, const PhysPara
 // per pass for 103823 particles; this form: 94-114 us.)  The pairs found wait in
 // a short list per lane, so that the lanes write them together.
 // FILL false: counts into cnt[i]; true: ids, in any order, at offsets[i].
-// F64: an FP64 problem, whose FP32 copies are in the walk's frame.
+// F64: an FP64 problem, whose FP32 copies are in the walk's frame.  SCALED: a
+// mixed one whose raw lengths have squares that leave the range of FP32; they
+// are brought to the size of its coordinates as they are read.
+// (Raw lengths up to 2^60 have finite squares, and from 2^-20 on the tests'
+// tolerances are far above the smallest ones.  Scaled throughout, the count
+// and fill of 103823 particles took 3 % longer, as one kernel with both
+// forms 22 %.)
+__host__ __device__ inline bool export_in_range(float coord_max) { return coord_max >= 0x1p-20f && coord_max <= 0x1p60f; }
 struct ExportCfg {
     static constexpr int CH = 64, LC = 32, SB = 16, WPB = 4;
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
     static constexpr size_t per_warp = CH * (sizeof(float4) + sizeof(int)) + (size_t)LC * 32 * sizeof(int) + scratch;
 };
-template <bool FILL, bool F64>
+template <bool FILL, bool F64, bool SCALED>
 __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, int kind, unsigned *cnt,
                                                                 const long long *offsets, int *idx, long long cap)
 {
@@ -60,6 +67,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
     using C = ExportCfg;
     __shared__ __align__(32) unsigned char smem[C::WPB * C::per_warp];
     __shared__ int wrote[C::WPB][32];
+    if (!F64 && export_in_range(coord_bound<false>(b.prob[0].ph, b.dyn[0])) == SCALED) return;  // the other launch's
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     unsigned char *mine = smem + wib * C::per_warp;
     float4 *cand = reinterpret_cast<float4 *>(mine);  // staged (x, y, z, R_K h rounded up)
@@ -72,9 +80,17 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
     const int lpp = ps.lpp, pp = lane / lpp, sub = lane % lpp;
     // bound of a staged coordinate's error: each of the two offsets and the
     // shift rounded once, the sums once more
-    const double unit = F64 ? frame_of(ph, d).unit : 1.0;
-    const float cmax = F64 ? frame_of(ph, d).max : ph.periodic ? ph.coord_max : d.coord_max;
-    const float err = 1e-6f * cmax + 1e-30f;
+    const float u = SCALED ? (float)fmin(frame_unit((double)coord_bound<F64>(ph, d)), 0x1p126) : 1.f;
+    const double unit = F64 ? frame_of(ph, d).unit : (double)u;
+    const float cmax = coord_bound<F64>(ph, d) * u;
+    const float err = 1e-6f * cmax;
+    constexpr float kFloor = 1e-36f;  // (squares below it may have underflowed: decided in FP64)
+    auto reach = [&](float h) { return __fmul_ru(ph.kr_f, SCALED ? __fmul_ru(h, u) : h); };
+    auto staged = [&](long long k) {
+        float4 q = b.pmf[k];
+        if (SCALED) q.x *= u, q.y *= u, q.z *= u;
+        return q;
+    };
     const int nleaf = b.counters[0];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (int leaf = w; leaf < nleaf; leaf += nw) {
@@ -82,17 +98,17 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
         const int st = b.leaf_start[leaf], nA = b.leaf_start[leaf + 1] - st;
         const bool active = pp < nA;
         const int s = st + (active ? pp : 0);
-        float4 pi = b.pmf[s];
-        pi.w = __fmul_ru(ph.kr_f, b.hf[s]);
+        float4 pi = staged(s);
+        pi.w = reach(b.hf[s]);
         float4 flo, fhi;
         frame_box<float4, float>(pi, active, flo, fhi);
-        const float R = __fmul_ru(ph.kr_f, boxA.plo.w) * 1.0001f + 4.f * err;
-        const float R2 = R * R;
+        const float R = reach(boxA.plo.w) * 1.0001f + 4.f * err;
+        const float R2 = R * R + kFloor;
         // the largest reach of a pair of this leaf, for the image handling
         float Rall = R, extmax;
-        if (kind == 1) problem_top_max(b, d, Rall, extmax), Rall = __fmul_ru(ph.kr_f, Rall) * 1.0001f;
-        if (ph.periodic) load_box(sc, ph, flo, fhi);
-        const bool wrap2 = ph.periodic && half_width(flo, fhi) + Rall >= half_box(ph);
+        if (kind == 1) problem_top_max(b, d, Rall, extmax), Rall = reach(Rall) * 1.0001f;
+        if (ph.periodic) load_box(sc, ph, flo, fhi, u);
+        const bool wrap2 = ph.periodic && half_width(flo, fhi) + Rall >= half_box(ph) * u;
         set_query(sc.qb, boxA.plo, boxA.phi, R, ph, cmax);
         int nbuf = 0, n = 0;
         const long long i = (long long)b.perm[s] - ps.base;
@@ -123,7 +139,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
                     if (wrap2) wrap3s<float>(sc, rx, ry, rz);
                     const float r2 = rx * rx + ry * ry + rz * rz;
                     const float Rk = kind == 1 ? fmaxf(pi.w, c.w) : pi.w;
-                    const float gap = r2 - Rk * Rk, tol = Rk * (8.f * err + 1e-5f * Rk) + err * err;
+                    const float gap = r2 - Rk * Rk, tol = Rk * (8.f * err + 1e-5f * Rk) + err * err + kFloor;
                     const int j = code[k];
                     if (active && gap < tol && !(kind == 1 && j == s))
                         lst[n++ * 32 + lane] = 2 * j + (gap > -tol);
@@ -133,7 +149,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
             nbuf = 0;
         };
         auto node = [&](const NodeBox &nb) {
-            return up_within(sc.qb, nb) || (kind == 1 && up_overlap(sc.qb, nb));
+            return up_within(sc.qb, nb, u) || (kind == 1 && up_overlap(sc.qb, nb, u));
         };
         int j = 0;
         float Rj = 0.f;
@@ -146,19 +162,19 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
             const bool in = (leaf_lanes(d.node_cnt[0], nd) >> lane) & 1u;
             const unsigned mask = __ballot_sync(FULL, node(b.nodes[0][first + (in ? lane : 0)]) && in);
             if (mask)
-                stage_group<float, C::CH, F64>(
+                stage_group<float, C::CH, F64 || SCALED>(
                 b, leaf, mask, first, ph, unit, nbuf, sc, [](bool, int, int, int, const float4 &) {},
                 [&](int jj) {
-                    float4 q = b.pmf[jj];
+                    float4 q = staged(jj);
                     q.w = __int_as_float(jj);
                     return q;
                 },
                 [&](float4 &q, int) {
                     j = __float_as_int(q.w);
-                    Rj = __fmul_ru(ph.kr_f, b.hf[j]);
+                    Rj = reach(b.hf[j]);
                     if (ph.periodic) wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
                     const float d2 = box_dist2<float>(q, flo, fhi), Rjj = Rj + 4.f * err;
-                    return d2 < R2 || (kind == 1 && d2 < Rjj * Rjj * 1.0001f);
+                    return d2 < R2 || (kind == 1 && d2 < Rjj * Rjj * 1.0001f + kFloor);
                 },
                 [&](int slot, const float4 &q, int, int) {
                     cand[slot] = make_float4(q.x, q.y, q.z, Rj);
@@ -175,7 +191,6 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
         __syncwarp();
     }
 }
-
 // Sorts each particle's ids (one warp per particle; ids are distinct, so an
 // id's place is the number of smaller ones).  A particle whose list crosses
 // cap is left to k_export_cut.
@@ -309,8 +324,8 @@ cudaError_t launch_set_sorted_h(const BatchView &b, int precision, const double 
     return cudaGetLastError();
 }
 
-cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind, long long *offsets, int *idx,
-                                    long long cap, long long *total_dev, cudaStream_t st)
+cudaError_t launch_neighbour_export(const BatchView &b, const PhysParams &ph, int precision, int kind, long long *offsets,
+                                    int *idx, long long cap, long long *total_dev, cudaStream_t st)
 {
     if (b.ntot == 0) {
         cudaMemsetAsync(offsets, 0, sizeof(long long), st);
@@ -324,12 +339,21 @@ cudaError_t launch_neighbour_export(const BatchView &b, int precision, int kind,
     const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
                          ((share + kScanThreads - 1) / kScanThreads * kScanThreads));
     const bool f64 = precision == SPH_PREC_FP64;
-    const auto count = f64 ? k_export<false, true> : k_export<false, false>;
-    const auto fill = f64 ? k_export<true, true> : k_export<true, false>;
-    launch_chain(SPH_DEP(b), count, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
+    // (an isolated problem's coordinates are known on the device: both forms
+    // are launched, and one leaves at once)
+    const bool raw = !f64 && (!ph.periodic || export_in_range(ph.coord_max));
+    const bool scaled = !f64 && !(ph.periodic && export_in_range(ph.coord_max));
+    auto launch = [&](auto kern) {
+        launch_chain(SPH_DEP(b), kern, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, (const long long *)offsets, idx, cap);
+    };
+    if (f64) launch(k_export<false, true, false>);
+    if (raw) launch(k_export<false, false, false>);
+    if (scaled) launch(k_export<false, false, true>);
     launch_chain(SPH_DEP(b), k_count_sums, nb, kScanThreads, 0, st, cnt, n, part);
     launch_chain(SPH_DEP(b), k_offsets, nb, kScanThreads, 0, st, cnt, n, part, offsets, total_dev);
-    launch_chain(SPH_DEP(b), fill, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, offsets, idx, cap);
+    if (f64) launch(k_export<true, true, false>);
+    if (raw) launch(k_export<true, false, false>);
+    if (scaled) launch(k_export<true, false, true>);
     launch_chain(SPH_DEP(b), k_export_sort, grid, 128, 0, st, b, offsets, idx, cap);
     launch_chain(SPH_DEP(b), k_export_cut, 1, 1024, 0, st, b, kind, offsets, idx, cap);
     return cudaGetLastError();

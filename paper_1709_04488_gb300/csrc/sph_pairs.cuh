@@ -301,6 +301,13 @@ __device__ __forceinline__ void set_query(QueryBox &qb, const float4 &lo, const 
     __syncwarp();
 }
 
+// bound of the problem's |coordinates| (F64: in the walk's frame)
+template <bool F64>
+__device__ __forceinline__ float coord_bound(const PhysParams &ph, const ProbDyn &d)
+{
+    return F64 ? frame_of(ph, d).max : ph.periodic ? ph.coord_max : d.coord_max;
+}
+
 // twice the gap between the query box and [blo, bhi] along one axis (minimum
 // image if periodic), negative where they overlap
 __device__ __forceinline__ float node_gap(const float4 &qa, float blo, float bhi)
@@ -308,11 +315,11 @@ __device__ __forceinline__ float node_gap(const float4 &qa, float blo, float bhi
     const float d = qa.x - (blo + bhi);
     return fminf(fabsf(d), fabsf(qa.z - fabsf(d))) - (qa.y + (bhi - blo));
 }
-__device__ __forceinline__ float node_dist2(const QueryBox &qb, const float4 &blo, const float4 &bhi)
+__device__ __forceinline__ float node_dist2(const QueryBox &qb, const float4 &blo, const float4 &bhi, float u = 1.f)
 {
-    const float gx = fmaxf(node_gap(qb.ax[0], blo.x, bhi.x), 0.f);
-    const float gy = fmaxf(node_gap(qb.ax[1], blo.y, bhi.y), 0.f);
-    const float gz = fmaxf(node_gap(qb.ax[2], blo.z, bhi.z), 0.f);
+    const float gx = fmaxf(node_gap(qb.ax[0], blo.x, bhi.x), 0.f) * u;
+    const float gy = fmaxf(node_gap(qb.ax[1], blo.y, bhi.y), 0.f) * u;
+    const float gz = fmaxf(node_gap(qb.ax[2], blo.z, bhi.z), 0.f) * u;
     return gx * gx + gy * gy + gz * gz;
 }
 __device__ __forceinline__ float node_sep(const QueryBox &qb, const float4 &blo, const float4 &bhi)
@@ -368,12 +375,16 @@ __device__ __forceinline__ bool leaf_overlap(const QueryBox &qb, const float4 &b
 
 // Tests of one node per lane, called by the whole warp: the position box
 // within R (up_within: nodes above the leaves), the smoothing-sphere box
-// overlapping the query.
-__device__ __forceinline__ bool up_within(const QueryBox &qb, const NodeBox &nb)
+// overlapping the query.  u: a power of two, where the query's R and cmax
+// were given in units of 1 / u (gaps multiplied by it before they are squared).
+__device__ __forceinline__ bool up_within(const QueryBox &qb, const NodeBox &nb, float u = 1.f)
 {
-    return node_dist2(qb, nb.plo, nb.phi) <= qb.out2;
+    return node_dist2(qb, nb.plo, nb.phi, u) <= qb.out2;
 }
-__device__ __forceinline__ bool up_overlap(const QueryBox &qb, const NodeBox &nb) { return node_sep(qb, nb.slo, nb.shi) <= qb.s2; }
+__device__ __forceinline__ bool up_overlap(const QueryBox &qb, const NodeBox &nb, float u = 1.f)
+{
+    return node_sep(qb, nb.slo, nb.shi) * u <= qb.s2;
+}
 __device__ __forceinline__ bool box_within(const QueryBox &qb, const NodeBox &nb, const PhysParams &ph)
 {
     const float g2 = node_dist2(qb, nb.plo, nb.phi);
@@ -506,15 +517,15 @@ __device__ __forceinline__ float box_Li<float>(const PhysParams &ph, int a) { re
 template <>
 __device__ __forceinline__ double box_Li<double>(const PhysParams &ph, int a) { return ph.box_inv[a]; }
 
-// lanes 0..2 copy the box lengths and the query box's centre into the
-// warp's scratch
+// lanes 0..2 copy the box lengths (times the power of two u, as lo and hi
+// are) and the query box's centre into the warp's scratch
 template <typename T, typename V>
-__device__ __forceinline__ void load_box(StageScratch<T> &sc, const PhysParams &ph, const V &lo, const V &hi)
+__device__ __forceinline__ void load_box(StageScratch<T> &sc, const PhysParams &ph, const V &lo, const V &hi, T u = T(1))
 {
     const int lane = threadIdx.x & 31;
     if (lane < 3) {
-        sc.L[lane] = box_L<T>(ph, lane);
-        sc.Li[lane] = box_Li<T>(ph, lane);
+        sc.L[lane] = box_L<T>(ph, lane) * u;
+        sc.Li[lane] = box_Li<T>(ph, lane) * (T(1) / u);
         sc.C[lane] = T(0.5) * (lane == 0 ? lo.x + hi.x : lane == 1 ? lo.y + hi.y : lo.z + hi.z);
         sc.ihl[lane] = 2.f * ph.box_inv_f[lane];
     }
@@ -1056,8 +1067,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     // offset and shift rounded once each, their sum once more), and the
     // particle's position
     const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
-    const float cmax = D64 ? frame_of(ph, dy).max : ph.periodic ? ph.coord_max : dy.coord_max;
-    const float err = D64 ? 1e-6f * cmax : 0.f;
+    const float err = D64 ? 1e-6f * coord_bound<D64>(ph, dy) : 0.f;
     const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles (the others
     // of the leaf keep their last solve, restaged by k_block_restage)
@@ -1253,7 +1263,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             nbuf = 0;
         };
         const float Rq2 = (Rq + 4.f * err) * (Rq + 4.f * err);
-        set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, cmax);
+        set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, coord_bound<D64>(ph, dy));
         // visit leaves within Rq (gather) or whose predicted smoothing
         // spheres reach this leaf (what the force pass will need); stage
         // only the former
@@ -1564,7 +1574,6 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
         const NodeBox boxA = b.nodes[0][leaf];
         constexpr bool D64 = sizeof(T) == 8;  // (the walk in its frame, the staged positions as they are)
         const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
-        const float cmax = D64 ? frame_of(ph, dy).max : ph.periodic ? ph.coord_max : dy.coord_max;
         const V pi = pm[s];
         const T eta3 = (T)(ph.eta * ph.eta * ph.eta);
         const T tol = (T)ph.h_tol;
@@ -1585,7 +1594,7 @@ __global__ void __launch_bounds__(FbCfg<T>::WPB * 32) k_density_fallback(BatchVi
         auto visit_all = [&](T hh, auto &&fn) {
             const float Rq = __fmul_ru(ph.kr_f, frame_len(hh, unit)) * 1.0001f;
             const T Rt = D64 ? KR * hh * T(1.0001) : (T)Rq, Rq2 = Rt * Rt;
-            set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, cmax);
+            set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, coord_bound<D64>(ph, dy));
             int nbuf = 0;
             auto flush = [&]() {
                 __syncwarp();
@@ -1890,8 +1899,7 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         xf = xi;
     }
     const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
-    const float cmax = D64 ? frame_of(ph, dy).max : ph.periodic ? ph.coord_max : dy.coord_max;
-    const float err = D64 ? 1e-6f * cmax : 0.f;
+    const float err = D64 ? 1e-6f * coord_bound<D64>(ph, dy) : 0.f;
     const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles, whose
     // largest h sets the gather reach
@@ -2145,7 +2153,7 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         __syncwarp();
         nbuf = 0;
     };
-    set_query(sc.qb, boxA.plo, boxA.phi, R, ph, cmax);
+    set_query(sc.qb, boxA.plo, boxA.phi, R, ph, coord_bound<D64>(ph, dy));
     auto node_test = [&](const NodeBox &nb) {
         const bool near = box_within(sc.qb, nb, ph);
         return box_overlap(sc.qb, nb, ph) || near;

@@ -84,7 +84,7 @@ def test_fp64_outputs_scale_exactly(S, kind, k):
 
 @pytest.mark.parametrize("k", [70, -80])
 @pytest.mark.parametrize("kind", ["lattice", "thin", "isolated", "m6"])
-@pytest.mark.parametrize("prec", ["fp64"])
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
 def test_lists_do_not_depend_on_the_unit(S, kind, k, prec):
     a, p, kw = _problem(kind)
     lists = []
