@@ -39,8 +39,8 @@ __device__ __forceinline__ bool export_member(const BatchView &b, const PhysPara
 
 // One warp per leaf, as in the pair kernels: the leaf's candidates are staged
 // in FP32 in its frame, and each lane tests them for its particle.  A pair
-// within the rounding of the staged coordinates of the boundary (a few in
-// 1e4) is decided in FP64 (export_member); the others are decided by FP32.
+// within the rounding of the staged coordinates of the boundary (stage_err;
+// a few in 1e4) is decided in FP64 (export_member); the others by FP32.
 // (One walk per particle with every candidate tested in FP64, the first form
 // of this kernel, was bound by the FP64 pipe, 1/64 of the FP32 rate: 3.04 ms
 // per pass for 103823 particles; this form: 94-114 us.)  The pairs found wait in
@@ -49,8 +49,8 @@ __device__ __forceinline__ bool export_member(const BatchView &b, const PhysPara
 // F64: an FP64 problem, whose FP32 copies are in the walk's frame.  SCALED: a
 // mixed one whose raw lengths have squares that leave the range of FP32; they
 // are brought to the size of its coordinates as they are read.
-// (Raw lengths up to 2^60 have finite squares, and from 2^-20 on the tests'
-// tolerances are far above the smallest ones.  Scaled throughout, the count
+// (Raw lengths up to 2^60 have finite squares, and from 2^-20 on the squares
+// of their spacings are far above kTinySq.  Scaled throughout, the count
 // and fill of 103823 particles took 3 % longer, as one kernel with both
 // forms 22 %.)
 __host__ __device__ inline bool export_in_range(float coord_max) { return coord_max >= 0x1p-20f && coord_max <= 0x1p60f; }
@@ -78,13 +78,9 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
     const ProbDyn &d = b.dyn[0];
     const PhysParams &ph = ps.ph;
     const int lpp = ps.lpp, pp = lane / lpp, sub = lane % lpp;
-    // bound of a staged coordinate's error: each of the two offsets and the
-    // shift rounded once, the sums once more
     const float u = SCALED ? (float)fmin(frame_unit((double)coord_bound<F64>(ph, d)), 0x1p126) : 1.f;
     const double unit = F64 ? frame_of(ph, d).unit : (double)u;
     const float cmax = coord_bound<F64>(ph, d) * u;
-    const float err = 1e-6f * cmax;
-    constexpr float kFloor = 1e-36f;  // (squares below it may have underflowed: decided in FP64)
     auto reach = [&](float h) { return __fmul_ru(ph.kr_f, SCALED ? __fmul_ru(h, u) : h); };
     auto staged = [&](long long k) {
         float4 q = b.pmf[k];
@@ -102,8 +98,9 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
         pi.w = reach(b.hf[s]);
         float4 flo, fhi;
         frame_box<float4, float>(pi, active, flo, fhi);
-        const float R = reach(boxA.plo.w) * 1.0001f + 4.f * err;
-        const float R2 = R * R + kFloor;
+        const float pmax = box_abs(flo, fhi);
+        float emax = 0.f;  // this lane's largest stage_err since the buffer was last emptied
+        const float R = reach(boxA.plo.w) * 1.0001f;
         // the largest reach of a pair of this leaf, for the image handling
         float Rall = R, extmax;
         if (kind == 1) problem_top_max(b, d, Rall, extmax), Rall = reach(Rall) * 1.0001f;
@@ -130,6 +127,8 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
         };
         auto test = [&]() {
             __syncwarp();  // staged candidates visible to every lane
+            const float err = warp_max(emax);
+            emax = 0.f;
             for (int k0 = 0; k0 < nbuf; k0 += C::SB) {
                 if (__any_sync(FULL, n > C::LC - C::SB)) drain();
                 const int ke = min(k0 + C::SB, nbuf);
@@ -139,7 +138,7 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
                     if (wrap2) wrap3s<float>(sc, rx, ry, rz);
                     const float r2 = rx * rx + ry * ry + rz * rz;
                     const float Rk = kind == 1 ? fmaxf(pi.w, c.w) : pi.w;
-                    const float gap = r2 - Rk * Rk, tol = Rk * (8.f * err + 1e-5f * Rk) + err * err + kFloor;
+                    const float gap = r2 - Rk * Rk, tol = Rk * (8.f * err + 1e-5f * Rk) + err * err + kTinySq;
                     const int j = code[k];
                     if (active && gap < tol && !(kind == 1 && j == s))
                         lst[n++ * 32 + lane] = 2 * j + (gap > -tol);
@@ -169,12 +168,17 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
                     q.w = __int_as_float(jj);
                     return q;
                 },
-                [&](float4 &q, int) {
+                [&](float4 &q, int o) {
                     j = __float_as_int(q.w);
                     Rj = reach(b.hf[j]);
+                    const float aq = abs3(q);
                     if (ph.periodic) wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
-                    const float d2 = box_dist2<float>(q, flo, fhi), Rjj = Rj + 4.f * err;
-                    return d2 < R2 || (kind == 1 && d2 < Rjj * Rjj * 1.0001f + kFloor);
+                    // (scaled: the raw copies may be below the smallest normal number)
+                    const float e = stage_err(abs3(sc.leaf[o]), aq, abs3(q), pmax) + (SCALED ? 1e-44f * u : 0.f);
+                    const float Rt = (kind == 1 ? fmaxf(R, Rj) : R) * 1.0001f + 2.f * e;
+                    if (!(box_dist2<float>(q, flo, fhi) < Rt * Rt + kTinySq)) return false;
+                    emax = fmaxf(emax, e);
+                    return true;
                 },
                 [&](int slot, const float4 &q, int, int) {
                     cand[slot] = make_float4(q.x, q.y, q.z, Rj);

@@ -715,6 +715,25 @@ __device__ __forceinline__ void stage_group(const BatchView &b, int A, unsigned 
     }
 }
 
+// The staged coordinates of FP64 problems and of the neighbour lists are
+// rounded copies; a pair is decided by them only outside a band around the
+// radius.  Roundings of a staged particle q (of a leaf with shift D; moved to
+// the image q') against a query particle p, in units of 2^-24, per axis: the
+// offset q - D, the shift, their sum, the image (box length, product, sum),
+// p, the difference and its own image come to at most 2 |D| + 3 |q| + 7 |q'|
+// + 6 |p|, so three axes move the distance by less than 0.8 stage_err, and
+// a reach grown by 2 stage_err misses no pair.  It scales with separations,
+// leaf widths and reaches, not with the domain (1e-6 of the domain, as large as
+// h where that is 1e-6 of it, let every staged particle of a clump pass to
+// FP64).
+template <typename V>
+__device__ __forceinline__ float abs3(const V &v) { return fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))); }
+__device__ __forceinline__ float box_abs(const float4 &lo, const float4 &hi) { return fmaxf(abs3(lo), abs3(hi)); }
+// D, q, q' as above, pmax: largest |coordinate| of the query particles
+__device__ __forceinline__ float stage_err(float D, float q, float q1, float pmax) { return 1e-6f * (D + q + q1 + pmax); }
+// squares below this may have underflowed (lengths below 1e-18 of the domain)
+constexpr float kTinySq = 1e-36f;
+
 // Box of the query leaf's particles in its own frame (offsets from the
 // reference point), over the lanes with on set.
 template <typename V, typename T>
@@ -1063,17 +1082,17 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
     const V pi = pm[s];
     const float4 pf = b.pmf[s];  // (FP32: pi)
     const T mi = pi.w;
-    // FP64: the walk's frame, the bound of a staged coordinate's error (its
-    // offset and shift rounded once each, their sum once more), and the
-    // particle's position
+    // FP64: the walk's frame and the particle's position
     const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
-    const float err = D64 ? 1e-6f * coord_bound<D64>(ph, dy) : 0.f;
     const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles (the others
     // of the leaf keep their last solve, restaged by k_block_restage)
     if (k0 >= 0) task_box(b, leaf, pf, active, boxA.plo.w, boxA);
     float4 flo, fhi;
     frame_box<float4, float>(pf, active, flo, fhi);
+    // (FP64) this lane's largest stage_err since the buffer was last emptied
+    const float pmax = D64 ? box_abs(flo, fhi) : 0.f;
+    float emax = 0.f;
     const float halfL = ph.periodic ? half_box(ph) : INFINITY;
     const T eta3 = (T)(ph.eta * ph.eta * ph.eta);
     const T tol = (T)ph.h_tol;
@@ -1120,7 +1139,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         cnt = 0;
         int gcnt = 0, at = lane;  // at: where this lane's next entry goes
         const float Rs = KR_f * hsf;
-        const float R2t = active && !fail ? D64 ? Rs * (Rs * 1.00002f + 8.f * err) + err * err : (float)R2 : -1.f;
+        const float R2t = active && !fail ? (float)R2 : -1.f;  // (FP64: see flush)
         bool ovf = false;
         int nbuf = 0;
         // FP64: the waiting pairs' distances, from the FP64 positions
@@ -1152,6 +1171,9 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                 // tested in FP32 with the coordinates' error to spare; the hits
                 // are dealt to the particle's lanes by rank
                 const unsigned below = (1u << sub) - 1u;
+                const float Rt = Rs * 1.00001f + 2.f * warp_max(emax);
+                const float R2t = active && !fail ? Rt * Rt + kTinySq : -1.f;
+                emax = 0.f;
                 for (int kb = 0; kb < nbuf; kb += C::SB) {
                     if (__any_sync(FULL, gcnt > C::LC * LPP - C::SB)) drain();
                     const int ke = min(kb + C::SB, nbuf);
@@ -1262,7 +1284,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
             __syncwarp();
             nbuf = 0;
         };
-        const float Rq2 = (Rq + 4.f * err) * (Rq + 4.f * err);
+        const float Rq2 = Rq * Rq;
         set_query(sc.qb, boxA.plo, boxA.phi, Rq, ph, coord_bound<D64>(ph, dy));
         // visit leaves within Rq (gather) or whose predicted smoothing
         // spheres reach this leaf (what the force pass will need); stage
@@ -1306,9 +1328,17 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                     return q;
                 },
                 [&](float4 &q, int o) {
+                    const float aq = D64 ? abs3(q) : 0.f;
                     if (D64 ? ph.periodic != 0 : WRAP && ((amo >> o) & 1u))
                         wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
-                    return box_dist2<float>(q, flo, fhi) < Rq2;
+                    const float d2 = box_dist2<float>(q, flo, fhi);
+                    if constexpr (D64) {
+                        const float e = stage_err(abs3(sc.leaf[o]), aq, abs3(q), pmax), Rt = Rq + 2.f * e;
+                        if (!(d2 < Rt * Rt + kTinySq)) return false;
+                        emax = fmaxf(emax, e);
+                        return true;
+                    }
+                    return d2 < Rq2;
                 },
                 [&](int slot, const float4 &q, int, int) {
                     if constexpr (!PACK) {
@@ -1889,8 +1919,7 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     const bool active = task_member<T>(b, st, nA, k0, pp, pos);
     const int s = st + (active ? pos : 0);
     const V xi = gph[s], vi = gvc[s], ti = gth[s];
-    // the walk's copy of the particle, its membership data (FP64: R_K h and the
-    // bound of a staged coordinate's error) and its position
+    // the walk's copy of the particle, its membership data (FP64: R_K h) and its position
     float4 xf;
     if constexpr (D64) {
         xf = b.pmf[s];
@@ -1899,7 +1928,6 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
         xf = xi;
     }
     const double unit = D64 ? frame_of(ph, dy).unit : 1.0;
-    const float err = D64 ? 1e-6f * coord_bound<D64>(ph, dy) : 0.f;
     const double X[3] = {D64 ? b.sx[s] : 0.0, D64 ? b.sy[s] : 0.0, D64 ? b.sz[s] : 0.0};
     // a block-step task walks from the box of its own particles, whose
     // largest h sets the gather reach
@@ -1946,9 +1974,12 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     T du = T(0), vs = T(-1);
     int pairs = 0, tested = 0;
     const float R = __fmul_ru(KR_f, boxA.plo.w) * 1.0001f;
-    const float RA2 = (R + 4.f * err) * (R + 4.f * err);
+    const float RA2 = R * R;
     float4 flo, fhi;
     frame_box<float4, float>(xf, active, flo, fhi);
+    // (FP64) this lane's largest stage_err since the buffer was last emptied
+    const float pmax = D64 ? box_abs(flo, fhi) : 0.f;
+    float emax = 0.f;
     const float halfL = ph.periodic ? half_box(ph) : INFINITY;
     if (ph.periodic) {
         load_box(sc, ph, flo, fhi);
@@ -2063,6 +2094,8 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
     auto test = [&]() {
         __syncwarp();  // staged candidates visible to every lane
         const int self = tA >= 0 ? ((tA << 5) | pos) : -1;
+        const float e2 = D64 ? 2.f * warp_max(emax) : 0.f;
+        emax = 0.f;
         if constexpr (PACK) {
             if (!wrap2) {
                 cb.pad(nbuf);
@@ -2114,10 +2147,9 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
                         const float4 c = cand[k];
                         float rx = xf.x - c.x, ry = xf.y - c.y, rz = xf.z - c.z;
                         if (wrap2) wrap3s<float>(sc, rx, ry, rz);
-                        const float Rm = fmaxf(xf.w, c.w);
+                        const float Rm = fmaxf(xf.w, c.w) * 1.00001f + e2;
                         j = code[k];
-                        hit = active && j != s &&
-                              rx * rx + ry * ry + rz * rz < Rm * (Rm * 1.00002f + 8.f * err) + err * err;
+                        hit = active && j != s && rx * rx + ry * ry + rz * rz < Rm * Rm + kTinySq;
                     }
                     const unsigned gm = (__ballot_sync(FULL, hit) >> (pp * LPP)) & ((1u << LPP) - 1u);
                     if (hit) {
@@ -2195,14 +2227,17 @@ __device__ __forceinline__ bool force_leaf(const BatchView &b, int leaf, int k0,
                     }
                 },
                 [&](float4 &q, int o) {
+                    const float aq = D64 ? abs3(q) : 0.f;
                     if (D64 ? ph.periodic != 0 : WRAP && ((amo >> o) & 1u))
                         wrap_near<float>(sc, q, sc.C[0], sc.C[1], sc.C[2]);
                     const float d2 = box_dist2<float>(q, flo, fhi);
                     if constexpr (D64) {
                         jq = __float_as_int(q.w);
                         q.w = __fmul_ru(KR_f, b.hf[jq]);
-                        const float Rj = q.w * 1.0001f + 4.f * err;
-                        return d2 < RA2 || d2 < Rj * Rj;
+                        const float e = stage_err(abs3(sc.leaf[o]), aq, abs3(q), pmax), Rj = fmaxf(R, q.w) * 1.0001f + 2.f * e;
+                        if (!(d2 < Rj * Rj + kTinySq)) return false;
+                        emax = fmaxf(emax, e);
+                        return true;
                     }
                     return d2 < RA2 || d2 * q.w * q.w < (float)(KF::R * KF::R * 1.0001);
                 },

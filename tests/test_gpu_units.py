@@ -96,3 +96,71 @@ def test_lists_do_not_depend_on_the_unit(S, kind, k, prec):
     assert len(lists[0][1]) > 20 * len(a["x"])
     for x, y in zip(*lists):
         assert np.array_equal(x, y)
+
+
+def test_far_clumps(S):
+    """Two copies of a clump 2^18 of its sizes apart: the lists of each are
+    the clump's, although the walk's boxes are as coarse as the domain."""
+    a, p = ics.cloud(1500, seed=6)
+    two = {k: np.concatenate([v, v]) for k, v in a.items()}
+    two["x"][1500:] += 2.0 ** 18
+    for prec in (S.PREC_FP64, S.PREC_MIXED):
+        for kind in (0, 1):
+            lists = []
+            for b in (a, two):
+                prob = S.Problem(b, S.make_params(prec, **p))
+                lists.append([t.cpu().numpy() for t in prob.neighbours(kind, h=b["h"])])
+                prob.close()
+            (o1, i1), (o2, i2) = lists
+            # (the moved copy's coordinates are rounded to 2^-35: its own
+            # lists may differ in pairs at the radius, the first copy's not)
+            assert np.array_equal(o2[:1501], o1) and np.array_equal(i2[:o1[-1]], i1)
+            assert abs(int(o2[-1]) - 2 * int(o1[-1])) <= 4
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("periodic", [False, True])
+def test_reach_out_of_the_domain_s_scale(S, prec, periodic):
+    """Smoothing lengths whose squares leave the range of FP32 beside a domain
+    of order one: every particle alone, or (isolated) every pair."""
+    a, p = ics.random_cloud(900, 8, periodic=periodic)
+    n = 900
+    prob = S.Problem(a, S.make_params(S.PREC_FP64 if prec == "fp64" else S.PREC_MIXED, **p))
+    for h in (1e-22, 1e-30, 1e25):
+        if h > 1 and periodic:
+            continue
+        for kind in (0, 1):
+            off, idx = (t.cpu().numpy() for t in prob.neighbours(kind, h=np.full(n, h)))
+            want = np.ones((n, n), bool) if h > 1 else np.eye(n, dtype=bool)
+            if kind:
+                np.fill_diagonal(want, False)
+            assert np.array_equal(off, np.concatenate([[0], np.cumsum(want.sum(1))]))
+            assert np.array_equal(idx, np.nonzero(want)[1])
+    prob.close()
+
+
+def test_far_clumps_take_no_longer(S):
+    """The band of pairs that FP64 decides is the rounding of separations, not
+    of the domain: the FP64 force pass of two clumps 2^18 of their sizes apart
+    takes the time of two clumps 2^8 apart (best of five; 1.07 times; with a
+    band of 1e-6 of the domain, wider than h, 5.7 times)."""
+    import torch
+    a, p = ics.cloud(1500, seed=6)
+    best = []
+    for e in (8, 18):
+        b = {k: np.concatenate([v, v]) for k, v in a.items()}
+        b["x"][1500:] += 2.0 ** e
+        prob = S.Problem(b, S.make_params(S.PREC_FP64, **p))
+        prob.density_h()
+        prob.forces()
+        t = []
+        for _ in range(5):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            t0.record()
+            prob.forces()
+            t1.record()
+            t1.synchronize()
+            t.append(t0.elapsed_time(t1))
+        best.append(min(t))
+        prob.close()
+    assert best[1] < 2.0 * best[0]
