@@ -336,8 +336,10 @@ cudaError_t launch_neighbour_export(const BatchView &b, const PhysParams &ph, in
         cudaMemsetAsync(total_dev, 0, sizeof(long long), st);
         return cudaGetLastError();
     }
-    unsigned *cnt = b.flag;                        // reuse: the leaf flags are no longer needed,
-    long long *part = (long long *)b.keys[1];      // nor the sort's second key buffer
+    // the sort's second buffers (the leaf of each particle, b.flag, serves the
+    // slow density path of the steps that keep these leaves)
+    unsigned *cnt = b.vals[0];
+    long long *part = (long long *)b.keys[1];
     const int sms = dev_info().sm_count, grid = sms * 8;
     const long long n = b.ntot, share = (n + kScanBlocks - 1) / kScanBlocks;
     const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
