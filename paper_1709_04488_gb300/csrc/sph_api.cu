@@ -1144,13 +1144,23 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     const BatchView &b = c->bv;
     cudaStream_t st = c->stream;
     CU(launch_reset_step(b, 1, st));
-    CU(launch_domain_and_keys(b, st));
-    CU(launch_radix_sort(b, st));
-    CU(launch_build_leaves(b, c->prm.precision, true, st));
+    if (c->since_build > 0 && c->since_build < c->prm.tree_rebuild_every) {
+        // kept leaves: their order is that of what the last passes staged
+        CU(launch_gather(b, st));
+        CU(launch_update_leaves(b, c->prm.precision, st));
+    } else {
+        CU(launch_domain_and_keys(b, st));
+        CU(launch_radix_sort(b, st));
+        CU(launch_build_leaves(b, c->prm.precision, true, st));
+    }
     CU(launch_set_sorted_h(b, c->prm.precision, h_in, st));
     CU(launch_refit(b, st));
     CU(launch_neighbour_export(b, c->host_ps.ph, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap,
                                b.scratch64, st));
+    if (h_in) {  // the boxes of a force pass that follows are those of the state's h
+        CU(launch_set_sorted_h(b, c->prm.precision, nullptr, st));
+        CU(launch_refit(b, st));
+    }
     CU(cudaStreamSynchronize(st));
     long long tot = 0;
     CU(cudaMemcpy(&tot, b.scratch64, sizeof tot, cudaMemcpyDeviceToHost));

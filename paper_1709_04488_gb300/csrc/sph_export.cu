@@ -227,11 +227,15 @@ __global__ void __launch_bounds__(128) k_export_sort(BatchView b, const long lon
 
 // The particle whose list crosses cap, if there is one (one block): its ids
 // are gathered again from all particles and those below cap written in order.
+// (As the call's last kernel it also has a force pass that follows walk the
+// tree: the leaf pass cleared the mark that the groups recorded by the last
+// density walk do not cover its h.)
 __global__ void __launch_bounds__(1024) k_export_cut(BatchView b, int kind, const long long *offsets, int *idx, long long cap)
 {
     chain_entry();
     __shared__ int buf[kExportCap];
     __shared__ int s_pos, s_n;
+    if (threadIdx.x == 0) b.dyn[0].lists_stale = 1;
     if (offsets[b.ntot] <= cap) return;
     const ProbStatic &ps = b.prob[0];
     long long lo = 0, hi = b.ntot - 1;  // the last particle that starts below cap

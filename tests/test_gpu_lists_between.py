@@ -44,3 +44,35 @@ def test_slow_path_of_a_step_that_keeps_the_leaves(S, kind, prec):
         prob.close()
     for f in ("h", "rho"):
         assert np.max(np.abs(got[1][f] / got[0][f] - 1.0)) < (1e-10 if prec == "fp64" else 1e-5)
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("kind", ["lattice", "cloud"])
+@pytest.mark.parametrize("h", [None, 0.3, 1.2])
+@pytest.mark.parametrize("after", ["density", "short guess", "kept step"])
+def test_forces_after_lists(S, kind, prec, h, after):
+    """A force pass after the lists sees the boxes of the state's h, the order
+    of what the density pass staged, and no recorded groups that do not cover
+    its h: the same bits as without the lists."""
+    a, p = ics.lattice(12, seed=5) if kind == "lattice" else ics.cloud(1800, seed=6)
+    if after == "short guess":  # (h grows beyond the recorded groups)
+        a["h"] = a["h"] * 0.7
+    pr = S.PREC_FP64 if prec == "fp64" else S.PREC_MIXED
+    got = []
+    for lists in (False, True):
+        prob = S.Problem(a, S.make_params(pr, **p, tree_rebuild_every=4))
+        prob.density_h()
+        if after == "kept step":
+            prob.forces()
+            prob.step(2e-3)
+            prob.step(2e-3)
+        if lists:
+            prob.neighbours(1, h=None if h is None else prob.numpy("h")["h"] * h)
+        prob.forces()
+        f0 = prob.numpy("ax", "ay", "az", "du", "vsig")
+        prob.step(1e-3)
+        got.append((f0, prob.numpy("x", "vx", "u", "h", "rho", "ax")))
+        prob.close()
+    for x, y in zip(*got):
+        for f in x:
+            assert np.array_equal(x[f], y[f]), f
