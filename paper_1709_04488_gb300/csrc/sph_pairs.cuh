@@ -842,10 +842,9 @@ struct DCfg {
     // particle within the list radius (M4 at eta = 1.2: ~63; M6 at eta = 1.0:
     // ~123, served by 2 or more lanes per particle)
     static constexpr bool D64 = sizeof(T) == 8;
-    // (FP64 deals its entries to the lanes by rank, so that they fill evenly:
-    // room for 120 (M6: 192) per particle)
-    static constexpr int LCAP = D64 ? (K == SPH_KERNEL_M6 ? 192 : 120) / LPP
-                                : K == SPH_KERNEL_M6 ? (LPP <= 2 ? 96 : LPP == 4 ? 64 : 32)
+    // (FP64, two or four lanes, deals its entries to the lanes by rank; room for
+    // a first h 1.26 and 1.36 times too large in a uniform M4 problem)
+    static constexpr int LCAP = K == SPH_KERNEL_M6 ? (LPP <= 2 ? 96 : LPP == 4 ? 64 : 32)
                                                      : LPP == 1 ? SPH_DENS_LCAP1 : LPP == 2 ? 64 : LPP == 4 ? 40 : 24;
     static constexpr int CH = SPH_DENS_CH;
     static constexpr int WPB = D64 ? 2 : 4;
@@ -1138,6 +1137,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         ng = 0;
         cnt = 0;
         int gcnt = 0, at = lane;  // at: where this lane's next entry goes
+        int g0 = 0;  // (FP64) waiting entries start at this rank, so that the dealing goes on where it stopped
         const float Rs = KR_f * hsf;
         const float R2t = active && !fail ? (float)R2 : -1.f;  // (FP64: see flush)
         bool ovf = false;
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
         auto drain = [&]() {
             __syncwarp();
             const int n = gcnt > sub ? (gcnt - sub - 1) / LPP + 1 : 0;
-            for (int e = 0; e < n; ++e) {
+            for (int e = sub < g0 ? 1 : 0; e < n; ++e) {
                 const int j = lst[e * 32 + lane];
                 const T dx = (T)min_image_bits(X[0] - b.sx[j], ph.box_len[0], ph.periodic);
                 const T dyy = (T)min_image_bits(X[1] - b.sy[j], ph.box_len[1], ph.periodic);
@@ -1162,7 +1162,7 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                     }
                 }
             }
-            gcnt = 0;
+            g0 = gcnt = gcnt % LPP;
             __syncwarp();
         };
         auto flush = [&]() {

@@ -164,3 +164,20 @@ def test_far_clumps_take_no_longer(S):
         best.append(min(t))
         prob.close()
     assert best[1] < 2.0 * best[0]
+
+
+@pytest.mark.parametrize("kernel,lanes,over", [(0, 2, 1.2), (0, 4, 1.3), (1, 2, 1.1), (1, 4, 1.22)])
+@pytest.mark.parametrize("equal", [True, False])
+def test_a_first_guess_too_large_stays_in_the_lists(S, kernel, lanes, over, equal):
+    """FP64 neighbour lists hold 128 and 160 entries a particle (M6 192 and
+    256) at two and four lanes: 1.26, 1.36 (1.16, 1.27) times the solved h of
+    a uniform problem.  Beyond that each particle takes the slow path."""
+    a, p = ics.lattice(16, seed=3)
+    a["h"] = a["h"] * over / (1.2 if kernel else 1.0)
+    if not equal:
+        a["m"] = a["m"] * np.random.default_rng(1).uniform(0.999, 1.001, len(a["m"]))
+    kw = dict(kernel=1, eta=1.0) if kernel else {}
+    prob = S.Problem(a, S.make_params(S.PREC_FP64, **p, lanes_per_particle=lanes, **kw))
+    prob.density_h()
+    assert prob.diagnostics().fallback == 0
+    prob.close()
