@@ -197,6 +197,7 @@ struct sph_ctx {
     ProbDiag *diag;
     ProbStatic host_ps;
     bool have_forces;
+    bool unclean;                 // see begin_builds
     int since_build;              // steps since the leaves were last built
     cudaGraphExec_t graph;        // one step that rebuilds the leaves
     cudaGraphExec_t graph_reuse;  // one step that keeps them
@@ -206,6 +207,23 @@ struct sph_ctx {
     bool timing;
     bool stage_ran[SPH_NSTAGES];
 };
+
+// The sort and the leaf scan find their state zero because the kernels that
+// use it clear it again (the sort's is cleared by the leaf scan).  A call that
+// fails between the two leaves it as it is, and a sort that starts from there
+// writes out of range: every call that builds leaves is unclean until its
+// launches are made, and after one that stayed so the state is cleared first.
+static int begin_builds(bool &unclean, const BatchView &b, cudaStream_t st)
+{
+    if (unclean) CU(cudaMemsetAsync(b.zero_lo, 0, b.zero_bytes, st));
+    unclean = true;
+    return SPH_OK;
+}
+static int begin_builds(sph_ctx *c)
+{
+    if (c->unclean) c->since_build = c->prm.tree_rebuild_every;  // (nor are the leaves there to be kept)
+    return begin_builds(c->unclean, c->bv, c->stream);
+}
 
 static void clear_ran(sph_ctx *c)
 {
@@ -435,6 +453,7 @@ int sph_setup(sph_ctx **out, const sph_params *p, int64_t n, const sph_state *st
     c->stream = (cudaStream_t)stream;
     c->lpp = lpp_of(p, n);
     c->have_forces = false;
+    c->unclean = false;
     c->since_build = 0;
     c->graph = nullptr;
     c->graph_reuse = nullptr;
@@ -897,6 +916,7 @@ int sph_sync(sph_ctx *c)
     CU(cudaStreamSynchronize(c->stream));
     unsigned st = 0;
     CU(cudaMemcpy(&st, &c->diag->status, sizeof st, cudaMemcpyDeviceToHost));
+    if (st & ST_TIMEOUT) c->unclean = true;
     return status_to_code(st);
 }
 
@@ -910,6 +930,7 @@ int sph_block_step(sph_ctx *c, double *dtmax_out, int64_t *evals_out)
     clear_ran(c);
     const BatchView b = block_view(c), bl = block_view(c, false);
     cudaStream_t st = c->stream;
+    if (int rc = begin_builds(c)) return rc;
     if (block_every(c) > 1 && c->since_build >= block_every(c)) {
         // the context's leaves do not hold its particles (a batch moved them): build them first
         CU(launch_domain_and_keys(c->bv, st));
@@ -926,6 +947,7 @@ int sph_block_step(sph_ctx *c, double *dtmax_out, int64_t *evals_out)
         }
         CU(cudaGraphLaunch(c->block_graph, st));
     }
+    c->unclean = false;
     long long evals = 0, dbits = 0;
     CU(cudaMemcpyAsync(&evals, b.scratch64 + 3, sizeof evals, cudaMemcpyDeviceToHost, st));
     CU(cudaMemcpyAsync(&dbits, b.scratch64 + 6, sizeof dbits, cudaMemcpyDeviceToHost, st));
@@ -961,9 +983,12 @@ int sph_density_h(sph_ctx *c)
 {
     if (!c) return fail(SPH_EINVAL, "ctx is NULL");
     clear_ran(c);
-    CU(launch_reset_step(c->bv, 1, c->stream));
-    int rc = enqueue_density(c->bv, c->prm.precision, 0, c->stream, marks_of(c));
+    int rc = begin_builds(c);
     if (rc) return rc;
+    CU(launch_reset_step(c->bv, 1, c->stream));
+    rc = enqueue_density(c->bv, c->prm.precision, 0, c->stream, marks_of(c));
+    if (rc) return rc;
+    c->unclean = false;
     CU(launch_kick_close(c->bv, 0, 0, c->stream));
     c->have_forces = false;
     c->since_build = 0;
@@ -996,9 +1021,12 @@ int sph_step(sph_ctx *c, double dt, double *dt_used)
         return fail(SPH_EINVAL, "no CFL step yet: call sph_density_h and sph_forces first, or pass dt > 0");
     if (!std::isfinite(dt)) return fail(SPH_EINVAL, "dt must be finite");
     clear_ran(c);
-    const bool rebuild = next_is_rebuild(c);
-    int rc = enqueue_step(c->bv, c->prm.precision, dt, c->stream, marks_of(c), rebuild);
+    int rc = begin_builds(c);
     if (rc) return rc;
+    const bool rebuild = next_is_rebuild(c);
+    rc = enqueue_step(c->bv, c->prm.precision, dt, c->stream, marks_of(c), rebuild);
+    if (rc) return rc;
+    c->unclean = false;
     count_step(c, rebuild);
     c->have_forces = true;
     if (dt_used) {
@@ -1046,6 +1074,7 @@ int sph_run(sph_ctx *c, int nsteps)
     if (nsteps < 0) return fail(SPH_EINVAL, "nsteps must be >= 0");
     if (!c->have_forces) return fail(SPH_EINVAL, "no CFL step yet: call sph_density_h and sph_forces first");
     if (nsteps == 0) return SPH_OK;
+    if (int rc = begin_builds(c)) return rc;
     for (int k = 0; k < nsteps; ++k) {
         const bool rebuild = next_is_rebuild(c);
         cudaGraphExec_t *slot = rebuild ? &c->graph : &c->graph_reuse;
@@ -1065,6 +1094,7 @@ int sph_run(sph_ctx *c, int nsteps)
         }
         count_step(c, rebuild);
     }
+    c->unclean = false;
     return finish_call(c);
 }
 
@@ -1143,6 +1173,7 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     if (cap < 0) return fail(SPH_EINVAL, "cap must be >= 0");
     const BatchView &b = c->bv;
     cudaStream_t st = c->stream;
+    if (int rc = begin_builds(c)) return rc;
     CU(launch_reset_step(b, 1, st));
     if (c->since_build > 0 && c->since_build < c->prm.tree_rebuild_every) {
         // kept leaves: their order is that of what the last passes staged
@@ -1157,6 +1188,7 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
     CU(launch_refit(b, st));
     CU(launch_neighbour_export(b, c->host_ps.ph, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap,
                                b.scratch64, st));
+    c->unclean = false;
     if (h_in) {  // the boxes of a force pass that follows are those of the state's h
         CU(launch_set_sorted_h(b, c->prm.precision, nullptr, st));
         CU(launch_refit(b, st));
@@ -1346,6 +1378,7 @@ struct sph_batch {
     cudaGraphExec_t graph = nullptr;
     int graph_kernels = 0;
     int eager = 0;  // steps enqueued before the capture
+    bool unclean = false;  // see begin_builds
     bool timing = false;
     cudaEvent_t ev[SPH_NSTAGES + 1] = {};
     bool stage_ran[SPH_NSTAGES] = {};
@@ -1424,6 +1457,8 @@ int sph_batch_run(sph_batch *bt, int nsteps)
 {
     if (!bt) return fail(SPH_EINVAL, "batch is NULL");
     if (nsteps < 0) return fail(SPH_EINVAL, "nsteps must be >= 0");
+    if (nsteps == 0) return SPH_OK;
+    if (int rc = begin_builds(bt->unclean, bt->b, bt->st)) return rc;
     for (int s = 0; s < nsteps; ++s) {
         if (!bt->graph && bt->eager == 0) {
             // the first step runs eagerly (it sets the kernels' lazily set
@@ -1439,7 +1474,8 @@ int sph_batch_run(sph_batch *bt, int nsteps)
         }
         CU(cudaGraphLaunch(bt->graph, bt->st));
     }
-    if (nsteps > 0) after_batch_steps(bt->ctxs.data(), (int)bt->ctxs.size(), bt->b, bt->st);
+    bt->unclean = false;
+    after_batch_steps(bt->ctxs.data(), (int)bt->ctxs.size(), bt->b, bt->st);
     return SPH_OK;
 }
 
@@ -1447,7 +1483,9 @@ int sph_batch_sync(sph_batch *bt, int *status)
 {
     if (!bt) return fail(SPH_EINVAL, "batch is NULL");
     CU(cudaStreamSynchronize(bt->st));
-    return batch_statuses(bt->ctxs.data(), (int)bt->ctxs.size(), status);
+    const int worst = batch_statuses(bt->ctxs.data(), (int)bt->ctxs.size(), status);
+    if (worst == SPH_ETIMEOUT || worst == SPH_ECUDA) bt->unclean = true;
+    return worst;
 }
 
 int sph_batch_stage_times(sph_batch *bt, double *ms)
