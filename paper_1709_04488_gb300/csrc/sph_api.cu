@@ -50,7 +50,7 @@ DevInfo dev_info()
 
 // ---- workspace layout -------------------------------------------------------
 // Carve the per-step scratch arrays for `ntot` particles over `nprob` problems.
-void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precision, int grav_chunks, int grav_tree,
+void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precision, long long grav_parts, int grav_tree,
                   int block)
 {
     const long long n = ntot > 0 ? ntot : 1;
@@ -72,7 +72,7 @@ void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precis
     b.cdold = c.take<double>(n);
     b.cdxi = c.take<double>(n);
     b.szg = c.take<char>(v4 / 4 * n);
-    b.gpart = grav_chunks > 1 ? c.take<double>(3LL * grav_chunks * n) : nullptr;
+    b.gpart = grav_parts > 0 ? c.take<double>(grav_parts) : nullptr;
     b.gpos = grav_tree ? (void *)c.take<char>(v4 * n) : nullptr;
     b.gh = grav_tree ? (void *)c.take<char>(v4 / 2 * n) : nullptr;
     int **bi[] = {&b.blev, &b.bnml, &b.breq, &b.bt0, &b.bt1};
@@ -417,7 +417,7 @@ size_t sph_workspace_bytes(int64_t n, const sph_params *p)
     BatchView b;
     memset(&b, 0, sizeof b);
     carve_tables(c, b, 1);
-    carve_arrays(c, b, n, 1, p->precision, p->gravity ? gravity_chunks(n, p->grav_theta) : 0,
+    carve_arrays(c, b, n, 1, p->precision, gravity_parts(n, *p),
                  p->gravity && p->grav_theta > 0, p->block_levels > 0);
     return c.off + 256;
 }
@@ -472,7 +472,7 @@ int sph_setup(sph_ctx **out, const sph_params *p, int64_t n, const sph_state *st
     c->diag = cv.take<ProbDiag>(1);
     memset(&c->bv, 0, sizeof c->bv);
     carve_tables(cv, c->bv, 1);
-    carve_arrays(cv, c->bv, n, 1, p->precision, p->gravity ? gravity_chunks(n, p->grav_theta) : 0,
+    carve_arrays(cv, c->bv, n, 1, p->precision, gravity_parts(n, *p),
                  p->gravity && p->grav_theta > 0, p->block_levels > 0);
     c->bv.ntot = n;
     c->bv.key_bits = key_bits_for(1);
@@ -1233,18 +1233,19 @@ size_t sph_batch_workspace_bytes(sph_ctx *const *ctxs, int nctx)
 {
     if (batch_check(ctxs, nctx) != SPH_OK) return 0;
     long long ntot = 0;
-    int gch = 0, gtree = 0;
+    long long gparts = 0;
+    int gtree = 0;
     for (int k = 0; k < nctx; ++k) {
         const sph_params &q = ctxs[k]->prm;
         ntot += ctxs[k]->n;
-        if (q.gravity && gravity_chunks(ctxs[k]->n, q.grav_theta) > gch) gch = gravity_chunks(ctxs[k]->n, q.grav_theta);
+        gparts += gravity_parts(ctxs[k]->n, q);
         if (q.gravity && q.grav_theta > 0) gtree = 1;
     }
     Carver c{nullptr};
     BatchView b;
     memset(&b, 0, sizeof b);
     carve_tables(c, b, nctx);
-    carve_arrays(c, b, ntot, nctx, ctxs[0]->prm.precision, gch, gtree);
+    carve_arrays(c, b, ntot, nctx, ctxs[0]->prm.precision, gparts, gtree);
     return c.off + 256;
 }
 
@@ -1267,8 +1268,8 @@ static int batch_view(sph_ctx *const *ctxs, int nctx, void *workspace, size_t ws
     std::vector<long long> bases(nctx + 1);
     int mask = 0, dmask = 0, b_any_isolated = 0, b_any_periodic = 0, b_any_general = 0, b_any_gravity = 0;
     int b_any_cd = 0;
-    long long grav_blocks = 0;
-    int gch = 0, gtree = 0;
+    long long grav_blocks = 0, gparts = 0;
+    int gtree = 0;
     for (int k = 0; k < nctx; ++k) {
         tab[k] = ctxs[k]->host_ps;
         tab[k].base = ntot;
@@ -1285,13 +1286,14 @@ static int batch_view(sph_ctx *const *ctxs, int nctx, void *workspace, size_t ws
         tab[k].gchunks = tab[k].ph.gravity ? gravity_chunks(ctxs[k]->n, tab[k].ph.grav_theta) : 0;
         if (tab[k].ph.gravity) grav_blocks += gravity_blocks(ctxs[k]->n, tab[k].ph.grav_theta);
         if (tab[k].ph.gravity && tab[k].ph.grav_theta > 0) gtree = 1;
-        if (tab[k].gchunks > gch) gch = tab[k].gchunks;
+        tab[k].gpart0 = gparts;
+        gparts += gravity_parts(ctxs[k]->n, ctxs[k]->prm);
     }
     bases[nctx] = ntot;
     Carver cv{(char *)workspace};
     memset(&b, 0, sizeof b);
     carve_tables(cv, b, nctx);
-    carve_arrays(cv, b, ntot, nctx, prec, gch, gtree);
+    carve_arrays(cv, b, ntot, nctx, prec, gparts, gtree);
     b.ntot = ntot;
     b.key_bits = key_bits_for(nctx);
     b.key_lo = key_low_bits(ntot);
@@ -1303,7 +1305,7 @@ static int batch_view(sph_ctx *const *ctxs, int nctx, void *workspace, size_t ws
     b.any_gravity = b_any_gravity;
     b.any_cd = b_any_cd;
     b.grav_blocks = grav_blocks;
-    b.grav_split = gch > 1;
+    b.grav_split = gparts > 0;
     b.any_grav_tree = gtree;
     CU(cudaMemcpyAsync(b.prob, tab.data(), sizeof(ProbStatic) * nctx, cudaMemcpyHostToDevice, st));
     CU(cudaMemcpyAsync(b.prob_base, bases.data(), sizeof(long long) * (nctx + 1), cudaMemcpyHostToDevice, st));

@@ -210,11 +210,11 @@ __global__ void __launch_bounds__(kGravThreads, sizeof(T) == 4 ? kGravBlocksPerS
     auto store = [&](long long i, int k) {
         const double F[3] = {two.sum(0, k), two.sum(1, k), two.sum(2, k)};
         if (b.block_on && ((const T *)b.slev)[i] < T(0)) return;  // block step: not this particle's force pass
-        if (C > 1) {  // partial of range ch, layout [ch][axis][ntot]
-            double *g = b.gpart + (long long)ch * 3 * b.ntot + i;
+        if (C > 1) {  // partial of range ch, layout [ch][axis][n]
+            double *g = b.gpart + ps.gpart0 + 3 * n * ch + (i - base);
             g[0] = F[0];
-            g[b.ntot] = F[1];
-            g[2 * b.ntot] = F[2];
+            g[n] = F[1];
+            g[2 * n] = F[2];
             return;
         }
         const long long io = (long long)b.perm[i] - ps.base;
@@ -249,11 +249,12 @@ __global__ void __launch_bounds__(256) k_gravity_reduce(BatchView b)
     const ProbStatic &ps = b.prob[p];
     if (!ps.ph.gravity || ps.gchunks <= 1) return;
     double fx = 0.0, fy = 0.0, fz = 0.0;
-    for (int ch = 0; ch < ps.gchunks; ++ch) {
-        const double *g = b.gpart + (long long)ch * 3 * b.ntot + i;
+    const long long n = ps.n;
+    const double *g = b.gpart + ps.gpart0 + (i - ps.base);
+    for (int ch = 0; ch < ps.gchunks; ++ch, g += 3 * n) {
         fx += g[0];
-        fy += g[b.ntot];
-        fz += g[2 * b.ntot];
+        fy += g[n];
+        fz += g[2 * n];
     }
     const long long io = (long long)b.perm[i] - ps.base;
     const double Gm = ps.ph.G * (ps.uniform_m ? ps.inv_m_uniform : 1.0 / ps.m[io]);
@@ -828,8 +829,11 @@ __global__ void __launch_bounds__(256) k_grav_dt(BatchView b)
 
 }  // namespace
 
-// C partner ranges for N particles: four waves of blocks (8 per SM), of at
-// least 128 partners each.  The kernel's time was its slowest block's: blocks
+// C partner ranges for N particles: up to four waves of blocks (8 per SM), of
+// at least 128 partners each and at most 32.  Up to 32768 particles their
+// partial sums are also held to the allocation-free call's scratch, in every
+// call alike (the sums are then the same bits): 29 ranges and 1.9 waves at
+// 20001 particles, 9 and just under one at 32768; 32 at 32769.  The kernel's time was its slowest block's: blocks
 // near their own particles' diagonal take the softened branch.  One wave,
 // two, three and four, 20001 particles (three evaluations, the whole pass):
 // 3.43, 3.03, 2.94, 2.90 ms; 65536: 21.0, 19.9, 19.0, 18.7 ms (with ranges of

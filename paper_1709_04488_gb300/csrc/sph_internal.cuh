@@ -130,6 +130,7 @@ struct ProbStatic {
     int uniform_m;   // all masses equal (m_uniform): neighbour lists keep distances only
     int gblk0;       // gravity: the problem's first block of the direct-sum launch
     int gchunks;     // gravity: ranges the partners are split into (one block per range and 256 particles)
+    long long gpart0;  // gravity: the problem's first partial sum in BatchView::gpart
     double m_uniform;
     double inv_m_uniform;  // 1 / m_uniform (0 unless uniform_m)
     PhysParams ph;
@@ -223,7 +224,7 @@ struct BatchView {
     long long grav_blocks;       // blocks of the direct-sum launch (all gravity problems)
     int grav_split;              // some gravity problem splits its partners (partial sums to reduce)
     int any_grav_tree;           // some gravity problem walks the tree (grav_theta > 0)
-    double *gpart;               // gravity: partial forces [chunk][ntot][3] of split problems
+    double *gpart;               // gravity: partial forces of split problems, [chunk][3][n] each from its gpart0
     // gravity tree: five Vec4 per node of each level (centre of mass relative
     // to the key-domain corner and mass; Q_xx, Q_xy, Q_xz, Q_yy; Q_yz, Q_zz,
     // l^2, h_max; box min; box max), element type float4 or dbl4
@@ -453,6 +454,12 @@ void launch_gravity(const BatchView &b, int precision, cudaStream_t st);  // dir
 // direct-sum launch of one problem (none when it walks the tree, theta > 0):
 long long gravity_blocks(long long n, double theta);  // blocks (particle blocks x partner ranges)
 int gravity_chunks(long long n, double theta);        // partner ranges
+// partial sums of a problem of n particles (none unless its partners are split)
+inline long long gravity_parts(long long n, const sph_params &p)
+{
+    const int c = p.gravity ? gravity_chunks(n, p.grav_theta) : 0;
+    return c > 1 ? 3ll * c * n : 0;
+}
 cudaError_t launch_kick_drift(const BatchView &b, double dt_host, cudaStream_t st);  // also selects dt, resets diagnostics
 // block time-steps (sph_block.cu).  Every quantity a tick needs lives on the
 // device, so that the ticks can run as a loop of a captured graph; scratch64:
@@ -545,7 +552,7 @@ struct Carver {
     }
 };
 int fail(int code, const char *fmt, ...);  // records the thread's error message, returns code
-void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precision, int grav_chunks = 0,
+void carve_arrays(Carver &c, BatchView &b, long long ntot, int nprob, int precision, long long grav_parts = 0,
                   int grav_tree = 0, int block = 0);
 void carve_tables(Carver &c, BatchView &b, int nprob);
 int key_bits_for(int nprob);

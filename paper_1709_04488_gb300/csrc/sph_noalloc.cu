@@ -60,7 +60,7 @@ size_t noalloc_bytes(const sph_params *p, long long n)
     BatchView b;
     memset(&b, 0, sizeof b);
     carve_tables(c, b, 1);
-    carve_arrays(c, b, n, 1, p->precision, p->gravity ? gravity_chunks(n, p->grav_theta) : 0,
+    carve_arrays(c, b, n, 1, p->precision, gravity_parts(n, *p),
                  p->gravity && p->grav_theta > 0);
     return c.off;
 }
@@ -124,7 +124,7 @@ extern "C" int sph_density_forces_noalloc(const sph_params *p, int64_t n, const 
     BatchView b;
     memset(&b, 0, sizeof b);
     carve_tables(c, b, 1);
-    carve_arrays(c, b, n, 1, p->precision, p->gravity ? gravity_chunks(n, p->grav_theta) : 0,
+    carve_arrays(c, b, n, 1, p->precision, gravity_parts(n, *p),
                  p->gravity && p->grav_theta > 0);
     if (c.off > kNoAllocBytes)  // (checked above; kept as a guard on the layout)
         return fail(SPH_ENOSPACE, "fixed scratch too small for %lld particles", (long long)n);
