@@ -1208,7 +1208,8 @@ __device__ __forceinline__ bool density_leaf(const BatchView &b, int leaf, int k
                     }
                 };
                 auto mass = [&](int k) { return UM ? 0.f : cb.v[C::Cand::NARR - 1][at0 + k]; };
-                // (r^2 in the same order of operations on every path of a launch)
+                // (r^2 in the same order of operations on every path of a launch; the
+                // launches differ in it only to keep the bits they have had)
                 auto dist2 = [](float dx, float dyy, float dz) {
                     return WRAP ? fma_rn(dz, dz, fma_rn(dyy, dyy, mul_rn(dx, dx)))
                                 : fma_rn(dz, dz, fma_rn(dx, dx, mul_rn(dyy, dyy)));

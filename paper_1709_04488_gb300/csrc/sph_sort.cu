@@ -25,6 +25,8 @@ constexpr int kSortThreads = 256;
 #ifndef SPH_SORT_ITEMS_L
 #define SPH_SORT_ITEMS_L 8
 #endif
+constexpr bool pass_items(int k) { return k == 2 || k == 4 || k == 8; }
+static_assert(pass_items(SPH_SORT_ITEMS_S) && pass_items(SPH_SORT_ITEMS_M) && pass_items(SPH_SORT_ITEMS_L), "built: 2, 4, 8");
 int sort_items(long long n)
 {
     return n <= (1ll << 16) ? SPH_SORT_ITEMS_S : n <= 3 * (1ll << 16) ? SPH_SORT_ITEMS_M : SPH_SORT_ITEMS_L;
@@ -398,7 +400,7 @@ cudaError_t launch_radix_sort(const BatchView &b, cudaStream_t st)
     for (int pass = 0; pass < passes; ++pass) {
         const bool last = pass == passes - 1;
         unsigned *vdst = last ? (unsigned *)b.perm : b.vals[src ^ 1];
-        auto kern = items == 1 ? k_onesweep<1> : items == 2 ? k_onesweep<2> : items == 4 ? k_onesweep<4> : k_onesweep<8>;
+        auto kern = items == 2 ? k_onesweep<2> : items == 4 ? k_onesweep<4> : k_onesweep<8>;
         launch_chain(SPH_DEP(b), kern, ntile, kSortThreads, 0, st, b.keys[src], b.vals[src], b.keys[src ^ 1], vdst, n, b.key_lo + 8 * pass,
                                              hist + pass * 256, status + (size_t)pass * ntile * 256, ctr + pass,
                                              pass == 0, (unsigned *)&b.counters[kTimeoutCounter]);
