@@ -1184,18 +1184,25 @@ int sph_neighbours(sph_ctx *c, int kind, const double *h_in, int64_t *offsets, i
         CU(launch_radix_sort(b, st));
         CU(launch_build_leaves(b, c->prm.precision, true, st));
     }
-    CU(launch_set_sorted_h(b, c->prm.precision, h_in, st));
-    CU(launch_refit(b, st));
-    CU(launch_neighbour_export(b, c->host_ps.ph, c->prm.precision, kind, (long long *)offsets, (int *)idx, (long long)cap,
-                               b.scratch64, st));
     c->unclean = false;
-    if (h_in) {  // the boxes of a force pass that follows are those of the state's h
-        CU(launch_set_sorted_h(b, c->prm.precision, nullptr, st));
+    const bool mixed = c->prm.precision == SPH_PREC_MIXED;
+    bool scaled = mixed && c->prm.periodic && !lists_in_range(c->host_ps.ph.coord_max);
+    long long res[2];  // entries, whether the form of the lists' kernel was the right one
+    for (;; scaled = true) {
+        CU(launch_set_sorted_h(b, c->prm.precision, h_in, st));
         CU(launch_refit(b, st));
+        CU(launch_neighbour_export(b, c->prm.precision, scaled, kind, (long long *)offsets, (int *)idx, (long long)cap, st));
+        if (h_in) {  // the boxes of a force pass that follows are those of the state's h
+            CU(launch_set_sorted_h(b, c->prm.precision, nullptr, st));
+            CU(launch_refit(b, st));
+        }
+        CU(cudaStreamSynchronize(st));
+        res[0] = 0;
+        res[1] = 1;
+        CU(cudaMemcpy(res, b.scratch64, sizeof res, cudaMemcpyDeviceToHost));
+        if (!mixed || scaled || c->n == 0 || res[1]) break;
     }
-    CU(cudaStreamSynchronize(st));
-    long long tot = 0;
-    CU(cudaMemcpy(&tot, b.scratch64, sizeof tot, cudaMemcpyDeviceToHost));
+    const long long tot = res[0];
     *total = tot;
     unsigned s = 0;
     CU(cudaMemcpy(&s, &c->diag->status, sizeof s, cudaMemcpyDeviceToHost));

@@ -53,7 +53,6 @@ __device__ __forceinline__ bool export_member(const BatchView &b, const PhysPara
 // of their spacings are far above kTinySq.  Scaled throughout, the count
 // and fill of 103823 particles took 3 % longer, as one kernel with both
 // forms 22 %.)
-__host__ __device__ inline bool export_in_range(float coord_max) { return coord_max >= 0x1p-20f && coord_max <= 0x1p60f; }
 struct ExportCfg {
     static constexpr int CH = 64, LC = 32, SB = 16, WPB = 4;
     static constexpr size_t scratch = (sizeof(StageScratch<float>) + 31) & ~(size_t)31;
@@ -67,7 +66,12 @@ __global__ void __launch_bounds__(ExportCfg::WPB * 32, 7) k_export(BatchView b, 
     using C = ExportCfg;
     __shared__ __align__(32) unsigned char smem[C::WPB * C::per_warp];
     __shared__ int wrote[C::WPB][32];
-    if (!F64 && export_in_range(coord_bound<false>(b.prob[0].ph, b.dyn[0])) == SCALED) return;  // the other launch's
+    if (!F64 && !SCALED && !lists_in_range(coord_bound<false>(b.prob[0].ph, b.dyn[0]))) {
+        if (!FILL)  // (empty lists; the caller comes back for the scaled form)
+            for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < b.ntot; k += (long long)gridDim.x * blockDim.x)
+                cnt[k] = 0u;
+        return;
+    }
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     unsigned char *mine = smem + wib * C::per_warp;
     float4 *cand = reinterpret_cast<float4 *>(mine);  // staged (x, y, z, R_K h rounded up)
@@ -235,7 +239,10 @@ __global__ void __launch_bounds__(1024) k_export_cut(BatchView b, int kind, cons
     chain_entry();
     __shared__ int buf[kExportCap];
     __shared__ int s_pos, s_n;
-    if (threadIdx.x == 0) b.dyn[0].lists_stale = 1;
+    if (threadIdx.x == 0) {
+        b.dyn[0].lists_stale = 1;
+        b.scratch64[1] = lists_in_range(coord_bound<false>(b.prob[0].ph, b.dyn[0]));
+    }
     if (offsets[b.ntot] <= cap) return;
     const ProbStatic &ps = b.prob[0];
     long long lo = 0, hi = b.ntot - 1;  // the last particle that starts below cap
@@ -332,12 +339,15 @@ cudaError_t launch_set_sorted_h(const BatchView &b, int precision, const double 
     return cudaGetLastError();
 }
 
-cudaError_t launch_neighbour_export(const BatchView &b, const PhysParams &ph, int precision, int kind, long long *offsets,
-                                    int *idx, long long cap, long long *total_dev, cudaStream_t st)
+// The number of entries goes to scratch64[0]; scratch64[1]: 0 if the scaled form
+// has to be launched (mixed precision; an isolated problem's coordinates are
+// known on the device only).
+cudaError_t launch_neighbour_export(const BatchView &b, int precision, bool scaled, int kind, long long *offsets, int *idx,
+                                    long long cap, cudaStream_t st)
 {
     if (b.ntot == 0) {
         cudaMemsetAsync(offsets, 0, sizeof(long long), st);
-        cudaMemsetAsync(total_dev, 0, sizeof(long long), st);
+        cudaMemsetAsync(b.scratch64, 0, sizeof(long long), st);
         return cudaGetLastError();
     }
     // the sort's second buffers (the leaf of each particle, b.flag, serves the
@@ -349,21 +359,13 @@ cudaError_t launch_neighbour_export(const BatchView &b, const PhysParams &ph, in
     const int nb = (int)((n + (share + kScanThreads - 1) / kScanThreads * kScanThreads - 1) /
                          ((share + kScanThreads - 1) / kScanThreads * kScanThreads));
     const bool f64 = precision == SPH_PREC_FP64;
-    // (an isolated problem's coordinates are known on the device: both forms
-    // are launched, and one leaves at once)
-    const bool raw = !f64 && (!ph.periodic || export_in_range(ph.coord_max));
-    const bool scaled = !f64 && !(ph.periodic && export_in_range(ph.coord_max));
     auto launch = [&](auto kern) {
         launch_chain(SPH_DEP(b), kern, grid, ExportCfg::WPB * 32, 0, st, b, kind, cnt, (const long long *)offsets, idx, cap);
     };
-    if (f64) launch(k_export<false, true, false>);
-    if (raw) launch(k_export<false, false, false>);
-    if (scaled) launch(k_export<false, false, true>);
+    launch(f64 ? k_export<false, true, false> : scaled ? k_export<false, false, true> : k_export<false, false, false>);
     launch_chain(SPH_DEP(b), k_count_sums, nb, kScanThreads, 0, st, cnt, n, part);
-    launch_chain(SPH_DEP(b), k_offsets, nb, kScanThreads, 0, st, cnt, n, part, offsets, total_dev);
-    if (f64) launch(k_export<true, true, false>);
-    if (raw) launch(k_export<true, false, false>);
-    if (scaled) launch(k_export<true, false, true>);
+    launch_chain(SPH_DEP(b), k_offsets, nb, kScanThreads, 0, st, cnt, n, part, offsets, b.scratch64);
+    launch(f64 ? k_export<true, true, false> : scaled ? k_export<true, false, true> : k_export<true, false, false>);
     launch_chain(SPH_DEP(b), k_export_sort, grid, 128, 0, st, b, offsets, idx, cap);
     launch_chain(SPH_DEP(b), k_export_cut, 1, 1024, 0, st, b, kind, offsets, idx, cap);
     return cudaGetLastError();

@@ -490,8 +490,10 @@ cudaError_t launch_block_kick(const BatchView &b, int L, bool use_cond, cudaGrap
 cudaError_t launch_block_finish(const BatchView &b, cudaStream_t st);
 cudaError_t launch_kick_close(const BatchView &b, int do_kick, int forces_ran, cudaStream_t st);
 cudaError_t launch_reset_step(const BatchView &b, int mode, cudaStream_t st);  // mode 1 full, 2 forces only
-cudaError_t launch_neighbour_export(const BatchView &b, const PhysParams &ph, int precision, int kind, long long *offsets,
-                                    int *idx, long long cap, long long *total_dev, cudaStream_t st);
+// coordinates whose squares the neighbour lists of mixed contexts form unscaled
+__host__ __device__ inline bool lists_in_range(float coord_max) { return coord_max >= 0x1p-20f && coord_max <= 0x1p60f; }
+cudaError_t launch_neighbour_export(const BatchView &b, int precision, bool scaled, int kind, long long *offsets, int *idx,
+                                    long long cap, cudaStream_t st);
 
 // Reset of one problem's per-call diagnostics: mode 1 a whole step's, mode 2
 // those of a forces-only call.

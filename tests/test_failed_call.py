@@ -28,7 +28,6 @@ extern "C" void fake_reset(const char *fail) { g_trace.clear(); g_fail = fail; }
 struct CUstream_st;
 namespace sph {
 struct BatchView;
-struct PhysParams;
 typedef const BatchView &V;
 typedef CUstream_st *S;
 typedef unsigned long long H;
@@ -45,7 +44,7 @@ F(launch_radix_sort, V, S) F(launch_reset_step, V, int, S) F(launch_block_drift,
 F(launch_block_finish, V, S) F(launch_block_gather, V, int, S) F(launch_build_leaves, V, int, bool, S)
 F(launch_set_sorted_h, V, int, const double *, S) F(launch_update_leaves, V, int, S) F(launch_block_leaf_tick, V, int, S)
 F(launch_domain_and_keys, V, S) F(launch_block_tick_begin, V, int, H, S)
-F(launch_neighbour_export, V, const PhysParams &, int, int, long long *, int *, long long, long long *, S)
+F(launch_neighbour_export, V, int, bool, int, long long *, int *, long long, S)
 void launch_gravity(V, int, S) { hit("launch_gravity"); }
 }
 extern "C" {
