@@ -311,8 +311,9 @@ int sph_diagnostics(sph_ctx *ctx, sph_diag *out);
 
 /* Exact FP64 neighbour lists in CSR form, ids ascending (Sec. 4.2 tree walk
  * retrieves them per leaf).  kind 0: {j : |r_ij|^2 < (2 h_i)^2} including i;
- * kind 1: {j != i : |r_ij|^2 < (2 max(h_i,h_j))^2}.  h_in: device array of n
- * smoothing lengths to use (NULL: state->h).  Distances are formed in FP64 as
+ * kind 1: {j != i : |r_ij|^2 < (2 max(h_i,h_j))^2}.  At any scale of lengths
+ * whose squares FP64 holds.  h_in: device array of n smoothing lengths to use
+ * (NULL: state->h).  Distances are formed in FP64 as
  * dx*dx + dy*dy + dz*dz without fused multiply-add, after the periodic minimum
  * image of each coordinate difference.  offsets (n+1 entries) and idx (cap
  * entries) are device arrays; *total receives the number of entries (if it
@@ -431,7 +432,7 @@ int sph_server_destroy(sph_server *s);
  *     which every GPU that loads the library holds until the process exits.
  *   - n is at most 32768, whatever the options (precision, kernel,
  *     self-gravity by direct sum or tree walk; the FP64 tree walk's layout,
- *     the largest, takes 23.7 MiB); larger n returns SPH_EINVAL with a
+ *     the largest, takes 23.6 MiB); larger n returns SPH_EINVAL with a
  *     message.  (A layout that did not fit would return SPH_ENOSPACE, before
  *     touching the device, naming the largest n that fits.)
  *   - The caller passes the particle arrays (inputs and outputs as in
@@ -454,7 +455,9 @@ int sph_density_forces_noalloc(const sph_params *p, int64_t n, const sph_state *
  * The table is process-wide and copied; it applies to contexts set up after
  * the call.  lanes[k] must be 1, 2, 4 or 8 and n_max must increase;
  * otherwise SPH_EINVAL and the table is unchanged.  At most 32 rows.  The
- * FP64 path clamps lanes to 2 or 4.  No counterpart in the paper: the
+ * FP64 path takes 4 lanes up to 8000 particles, beyond that the table's
+ * clamped to 2 or 4 (lanes that the params ask for are clamped alike, at
+ * every size).  No counterpart in the paper: the
  * package's autotuner measures the table on the GPU and installs it. */
 int sph_set_launch_table(const int64_t *n_max, const int32_t *lanes, int rows);
 

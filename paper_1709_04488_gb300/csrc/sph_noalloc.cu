@@ -22,7 +22,7 @@ using namespace sph;
 // workspace layout of every option for 32768 particles: the FP64 layout
 // (15.7 MiB) plus self-gravity's buffers (partial sums of split partner
 // ranges, 23.3 MiB in all at most; the tree walk's copies; the FP64 tree
-// walk's layout is the largest, 23.7 MiB), plus the diagnostics record.  noalloc_max_n() finds the
+// walk's layout is the largest, 23.6 MiB), plus the diagnostics record.  noalloc_max_n() finds the
 // largest n for a layout that would not fit (a guard: none does now).
 constexpr long long kNoAllocMaxN = 32768;
 constexpr size_t kNoAllocBytes = (size_t)24 << 20;

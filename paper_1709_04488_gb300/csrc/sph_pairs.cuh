@@ -11,12 +11,13 @@
 // in-range candidates so that the arithmetic runs without divergence.
 //
 // FP64 problems (SPH_PREC_FP64): this GPU runs FP64 at 1/64 of the FP32 rate,
-// so the walk, the staging and the tests of the candidates run in FP32 with
-// the rounding of the staged coordinates to spare, and only the pairs that
-// pass take FP64: their distance from the FP64 positions, the exact
-// membership, the sums.  The FP64 pipe is 72-75 % busy (k_forces 947 -> 660 us,
-// k_density 626 -> 510 us at 36864 particles of the Sod tube, two lanes per
-// particle; smaller problems 1.7-4 times faster).
+// so the walk, the staging and the tests of the candidates run in FP32, in a
+// frame of the domain's size (Frame), with the rounding of the staged
+// coordinates to spare (stage_err), and only the pairs that pass take FP64:
+// their distance from the FP64 positions, the exact membership, the sums.  The
+// FP64 pipe is 74 % busy in k_forces and 70 % in k_density (36864 particles of
+// the Sod tube, two lanes per particle: 947 -> 660 us and 626 -> 510 us;
+// smaller problems 1.7-4 times faster).
 //
 //  k_density   Eqs. SPHRHO, HRHO, OMEGA: Newton-Raphson on
 //              F(h) = rho(h) - m (eta/h)^3 over the cached list of (r^2, m_j)
