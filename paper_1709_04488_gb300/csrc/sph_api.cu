@@ -454,7 +454,7 @@ int sph_setup(sph_ctx **out, const sph_params *p, int64_t n, const sph_state *st
     c->lpp = lpp_of(p, n);
     c->have_forces = false;
     c->unclean = false;
-    c->since_build = 0;
+    c->since_build = p->tree_rebuild_every;  // (no leaves to be kept yet)
     c->graph = nullptr;
     c->graph_reuse = nullptr;
     c->block_graph = nullptr;

@@ -169,3 +169,16 @@ def test_batch_state_is_cleared_after_a_failed_call(L):
     assert L.sph_batch_run(bt, 1) == sph.OK
     assert zero not in _trace(L)
     L.sph_batch_destroy(bt)
+
+
+def test_a_first_step_without_a_density_solve_builds_the_leaves(L):
+    """With tree reuse a context keeps leaves only once it has some."""
+    ctx, _ = _context(L, 0, tree_rebuild_every=4)
+    L.fake_reset(b"")
+    assert L.sph_step(ctx, C.c_double(1e-3), None) == sph.OK
+    t = _trace(L)
+    assert t.index("launch_radix_sort") < t.index("launch_build_leaves") < t.index("launch_density")
+    L.fake_reset(b"")
+    assert L.sph_step(ctx, C.c_double(1e-3), None) == sph.OK
+    assert "launch_update_leaves" in _trace(L) and "launch_radix_sort" not in _trace(L)
+    L.sph_destroy(ctx)
