@@ -174,9 +174,11 @@ static int choose_lpp(long long n, int precision, int requested, int kernel)
     if (kernel == SPH_KERNEL_M6 && requested == 0) l = l >= 4 ? 8 : 2 * l;
     if (kernel == SPH_KERNEL_M6 && l < 2) l = 2;
     // FP64 pair kernels run 2 or 4 lanes; 4 where leaves of 16 particles would
-    // not fill one wave of warps (12 per SM): lattice 4096, two evaluations and
-    // three steps: 2.74 ms with 2 lanes, 1.66 with 4; from about 1e4 particles
-    // on the two differ by the last wave's fill only
+    // not fill one wave of warps (8 per SM): a step with 2 and 4 lanes, lattice
+    // and cloud, us: 4096 particles 397, 249 and 631, 370; 8000: 496, 378 and
+    // 686, 553; 10648: 649, 606 and 749, 654; beyond, they differ by the last
+    // wave's fill (15625: 683, 834 and 982, 851; 27000: 1227, 1141 and 1300,
+    // 1236)
     if (precision == SPH_PREC_FP64) l = l >= 4 || (requested == 0 && n <= 8000) ? 4 : 2;
     return l;
 }
